@@ -35,6 +35,18 @@ int ensure_buffer(vomt_ctx *ctx, void **p, size_t *cap, size_t bytes, const char
     return VOMT_OK;
 }
 
+int ensure_history(vomt_ctx *ctx, int rows)
+{
+    if (ctx->hist_cap >= rows) return VOMT_OK;
+    if (ctx->dhist) cudaFree(ctx->dhist);
+    ctx->dhist = nullptr;
+    ctx->hist_cap = 0;
+    cudaError_t e = cudaMalloc(&ctx->dhist, sizeof(double) * NMET * (size_t)rows);
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "history");
+    ctx->hist_cap = rows;
+    return VOMT_OK;
+}
+
 cudaError_t copy_planes(float *dst, int dst_pitch, const float *src, int src_pitch, int n, size_t planes,
                         cudaMemcpyKind kind, cudaStream_t st)
 {

@@ -92,7 +92,7 @@ struct DevStatus {
     int checks;     // checks run
     int error;      // 0 or VOMT_ERR_NONFINITE / VOMT_ERR_BARRIER_TIMEOUT
     int raw;        // 1: met[2], met[3] hold ||r||^2 and ||rho0 - rho1||^2 (finish_raw_row)
-    int reserved;
+    int slot;       // marching form: which of its two states holds the iterate of the last check
     double met[NMET];
 };
 
@@ -230,6 +230,11 @@ int ensure_buffer(vomt_ctx *ctx, void **p, size_t *cap, size_t bytes, const char
 int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg,
                  const vomt_params &p, const float *rho0, const float *rho1,
                  float *u, float *w, float *phi, cudaStream_t st);
+// its marching form for vector problems (march2d.cu); *taken: whether it ran the solve
+int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg, const vomt_params &p,
+                const float *rho0, const float *rho1, float *u, float *w, float *phi, cudaStream_t st, bool *taken);
+// rows of the check history on the device
+int ensure_history(vomt_ctx *ctx, int rows);
 // resident engine (vector_resident.cu)
 struct ResidentPlan {
     int Gx, Gy, TXm, TYm, H, threads, P;
@@ -266,10 +271,10 @@ constexpr int kMetricBlocks = 608;
 // Fixed-order sum of per-block FP64 partials (NRED per block), the stopping
 // decision and the history row (one block of kFinThreads threads, one warp per
 // slot; vector_stream.cu).  t < 0: the iteration is the last check's plus -t
-// (replayed graphs).
+// (replayed graphs).  slot: recorded in the status block.
 constexpr int kFinThreads = 32 * NRED;
 __global__ void k_finalize(const double *__restrict__ partials, int nblocks, SolveCfg cfg, int t, DevStatus *st,
-                           double *hist, int hist_cap);
+                           double *hist, int hist_cap, int slot);
 
 bool resident_plan(int n, int k, int max_blocks, int force_H, ResidentPlan *out);
 bool resident_plan_wave(int n, int k, int count, int max_blocks, ResidentPlan *out);

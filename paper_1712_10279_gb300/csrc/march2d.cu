@@ -1,0 +1,253 @@
+// Marching form of the streaming engine: host side (kernels in march2d.cuh).
+#include <math.h>
+#include <string.h>
+
+#include <algorithm>
+
+#include "march2d.h"
+
+namespace vomt {
+namespace {
+
+using namespace march;
+
+constexpr int kWarps = 4;             // warps per block (march2d.cuh)
+
+Kernels pick(int k, int un, int wn, bool reg)
+{
+    switch (k) {
+        case 1:
+        case 2: return pick_k12(k, un, wn, reg);
+        case 3: return pick_k3(k, un, wn, reg);
+        case 4: return pick_k4(k, un, wn, reg);
+        case 5: return pick_k5(k, un, wn, reg);
+        case 6: return pick_k6(k, un, wn, reg);
+        case 7: return pick_k7(k, un, wn, reg);
+        default: return pick_k8(k, un, wn, reg);
+    }
+}
+
+// The pairwise form of a channel graph's operator: every row of G is +1/c_e at one channel
+// and -1/c_e at a later one, Dv its transpose, all weights 1.  False for any other operator
+// (matrix fields).
+bool graph_of(const OpDev &g, const StepDev &s, const SolveCfg &cfg, MarchOp *out)
+{
+    if (g.k < 1 || g.k > KVEC || g.l > LVEC) return false;
+    MarchOp m;
+    memset(&m, 0, sizeof m);
+    for (int e = 0; e < LVEC; ++e) m.edge[e] = -1;
+    for (int c = 0; c < g.k; ++c)
+        if (g.wc[c] != 1.0f) return false;
+    for (int e = 0; e < g.l; ++e) {
+        int lo = -1, hi = -1;
+        for (int c = 0; c < g.k; ++c) {
+            if (g.Dv[c][e] != g.G[e][c]) return false;
+            if (g.G[e][c] == 0.0f) continue;
+            if (lo < 0) lo = c;
+            else if (hi < 0) hi = c;
+            else return false;
+        }
+        if (hi < 0 || g.we[e] != 1.0f || !(g.G[e][lo] > 0.0f) || g.G[e][hi] != -g.G[e][lo]) return false;
+        const int q = lo * (2 * g.k - lo - 1) / 2 + hi - lo - 1;
+        if (m.edge[q] >= 0) return false;
+        m.edge[q] = e;
+        m.inv[q] = g.G[e][lo];
+        m.nuinv[q] = s.nu * g.G[e][lo];
+    }
+    m.n = s.n;
+    m.l = g.l;
+    m.reg = s.reg;
+    m.ih = s.ih;
+    m.mu = s.mu;
+    m.nu = s.nu;
+    m.tau = s.tau;
+    m.alpha = s.alpha;
+    m.eps = s.eps;
+    m.su = s.reg ? s.su : 1.0f;
+    m.sw = s.reg ? s.sw : 1.0f;
+    (void)cfg;
+    *out = m;
+    return true;
+}
+
+// One kind of pass: its stages, chunks and estimated time.
+struct Pass {
+    int stages = 0, rows = 0, strips = 0, warps = 0, blocks = 0;
+    double us = 0.0;
+};
+
+// Chunk rows of a pass with S stages: those of the least arithmetic time.  A warp takes
+// rows + 2 S row-steps of S stages; a stage of a row costs a scheduler `issue` cycles when
+// enough warps share it and `lat` cycles when a warp is alone (the chain through two
+// shuffles and a reciprocal square root).  The estimate adds what every pass costs besides
+// (launch, first rows, last stores) and is no shorter than the pass's bytes take: 6.3 TB/s
+// from HBM, 12 TB/s where the states stay in L2.  Against every chunk length on a GB300 its
+// choice was within 5% of the fastest for k = 1, 2, 3, 5, 6, 8 and n = 32 .. 2048.
+Pass plan_pass(int n, int k, int groups, int S, int blocks_per_sm, int sms)
+{
+    const double issue = 20.0 + 40.0 * k + 4.0 * k * (k - 1), lat = 180.0, ghz = 1.95;
+    const int W = 32 - 2 * S, strips = (n + W - 1) / W;
+    const long cap = (long)blocks_per_sm * sms;
+    Pass best;
+    for (int chunks = 1; chunks <= n; ++chunks) {
+        const int rows = (n + chunks - 1) / chunks;
+        if (chunks > 1 && (n + rows - 1) / rows != chunks) continue;       // the same rows again
+        const long warps = (long)strips * chunks, blocks = (warps + kWarps - 1) / kWarps;
+        if (blocks > (1l << 30)) break;
+        const long full = blocks / cap, rest = blocks % cap;
+        const double per_sched = (double)kWarps / 4.0;                    // warps a block puts on a scheduler
+        double cycles = (double)full * std::max(lat, issue * per_sched * blocks_per_sm);
+        if (rest) cycles += std::max(lat, issue * per_sched * ceil((double)rest / sms));
+        const double us = cycles * S * (rows + 2 * S) / (ghz * 1e3);
+        if (best.stages == 0 || us < best.us) best = Pass{S, rows, strips, (int)warps, (int)blocks, us};
+    }
+    const double mb = 16e-6 * n * n * (2 * groups + (k + 3) / 4);
+    best.us = 3.5 + std::max(best.us, mb / (mb > 110.0 ? 6.3 : 12.0));
+    return best;
+}
+
+}  // namespace
+
+// The solve of stream_solve for vector problems.  *taken = false (and VOMT_OK) where this
+// form does not apply: operators other than a channel graph's, state that does not fit the
+// device's memory, and up to four channels with fewer than four iterations between checks,
+// where the one-iteration kernels need no second layout and are as fast (2048^2, three
+// channels: 79 us against 84 with one stage).
+int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg, const vomt_params &p,
+                const float *rho0, const float *rho1, float *u, float *w, float *phi, cudaStream_t st, bool *taken)
+{
+    *taken = false;
+    MarchOp op;
+    if (p.u_norm > VOMT_U_L1 || p.w_norm > VOMT_W_L2 || !graph_of(g, s, cfg, &op)) return VOMT_OK;
+    const int n = s.n, k = g.k;
+    const int interval = std::min(p.check_every, std::max(p.max_iters, 0));
+    if (k <= 4 && interval < 4) return VOMT_OK;
+    const Kernels K = pick(k, p.u_norm, p.w_norm, s.reg != 0);
+
+    Pass pass[3];
+    int main_pass = 0;
+    for (int q = 0; q < 3; ++q) {
+        if (!K.step[q]) continue;
+        cudaError_t e = cudaFuncSetAttribute((const void *)K.step[q], cudaFuncAttributeMaxDynamicSharedMemorySize, K.smem);
+        int per_sm = 0;
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)K.step[q], 32 * kWarps, K.smem);
+        if (e != cudaSuccess) return set_cuda_error(ctx, e, "marching kernel");
+        if (per_sm < 1) continue;
+        pass[q] = plan_pass(n, k, K.groups, kStages[q], per_sm, ctx->sm_count);
+        if (kStages[q] <= std::max(interval, 1) &&
+            (pass[main_pass].stages == 0 || pass[q].us / kStages[q] < pass[main_pass].us / kStages[main_pass]))
+            main_pass = q;
+    }
+    if (pass[0].stages == 0) return VOMT_OK;
+
+    // b, two states, and the state one iteration before a check where a pass of several
+    // iterations ends on it
+    const int states = main_pass > 0 ? 3 : 2;
+    const size_t state4 = (size_t)n * ((n + 31) / 32) * K.groups * 32, b4 = (size_t)n * ((n + 31) / 32) * K.bgroups * 32;
+    int rc = ensure_buffer(ctx, (void **)&ctx->ws, &ctx->ws_floats, sizeof(float4) * (b4 + states * state4), "workspace");
+    if (rc) {
+        ctx->err.clear();
+        return VOMT_OK;
+    }
+    float4 *b = (float4 *)ctx->ws, *S[3] = {b + b4, b + b4 + state4, b + b4 + 2 * state4};
+
+    // the check: strips of 30 columns, chunks that give every SM work, at most kMetricBlocks blocks
+    CheckArgs ca;
+    memset(&ca, 0, sizeof ca);
+    ca.strips = (n + 29) / 30;
+    ca.rows = std::max(4, (int)(((long)ca.strips * n + kMetricBlocks * kWarps - 1) / (kMetricBlocks * kWarps)));
+    ca.items = ca.strips * ((n + ca.rows - 1) / ca.rows);
+    const int mblocks = std::min((ca.items + kWarps - 1) / kWarps, kMetricBlocks);
+    rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * (size_t)mblocks * NRED, "partials");
+    if (rc) return rc;
+    ca.partials = ctx->partials;
+    ca.b = b;
+    ca.st = ctx->dstatus;
+    rc = ensure_history(ctx, p.max_iters / p.check_every + 2);
+    if (rc) return rc;
+    cudaError_t e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "status reset");
+    *taken = true;
+    ctx->hist_raw = false;           // k_finalize writes finished rows
+    ctx->last_blocks = pass[main_pass].blocks;
+
+    const PlanarArgs planar{rho0, rho1, u, w, phi, p.warm_start};
+    const dim3 lgrid((n + 127) / 128, std::min(n, 2048));
+    K.in<<<lgrid, 128, 0, st>>>(planar, op, S[0], b);
+    ctx->launches += 1;
+
+    int cur = 0;                     // the state that holds the iterate
+    const float4 *before = S[0];     // its predecessor, after `run` with `last`
+    auto one = [&](int q, bool last) {
+        const Pass &ps = pass[q];
+        MarchArgs a;
+        a.in = S[cur];
+        a.out = S[cur ^ 1];
+        a.prev = last && ps.stages > 1 ? S[2] : nullptr;
+        a.b = b;
+        a.st = ctx->dstatus;
+        a.rows = ps.rows;
+        a.strips = ps.strips;
+        a.warps = ps.warps;
+        launch_pdl(K.step[q], dim3(ps.blocks), dim3(32 * kWarps), (size_t)K.smem, st, a, op);
+        ctx->launches += 1;
+        before = a.prev ? a.prev : a.in;
+        cur ^= 1;
+    };
+    // m iterations, fewer-stage passes first
+    auto run = [&](int m) {
+        int q = main_pass, odd = m % kStages[q];
+        for (int r = q - 1; r >= 0; --r)
+            for (; pass[r].stages && odd >= kStages[r]; odd -= kStages[r], m -= kStages[r]) one(r, m == kStages[r]);
+        for (; m > 0; m -= kStages[q]) one(q, m == kStages[q]);
+    };
+    auto check = [&](int t) {
+        CheckArgs c = ca;
+        c.cur = S[cur];
+        c.prv = before;
+        launch_pdl(K.check, dim3(mblocks), dim3(32 * kWarps), 0, st, c, op);
+        launch_pdl(k_finalize, dim3(1), dim3(kFinThreads), 0, st, (const double *)ctx->partials, mblocks, cfg, t,
+                   ctx->dstatus, ctx->dhist, ctx->hist_cap, cur);
+        ctx->launches += 2;
+    };
+    if (p.max_iters == 0) check(0);
+    const bool tol_mode = cfg.tol_gap > 0.0;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    if (tol_mode)
+        for (int q = 0; q < 2; ++q) cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming);
+    const int chunk = p.check_every * ((2048 + p.check_every - 1) / p.check_every);
+    int t = 0, nchunk = 0;
+    bool stopped = false;
+    while (t < p.max_iters && !stopped) {
+        const int end = p.max_iters - t > chunk ? t + chunk : p.max_iters;
+        while (t < end) {
+            const int m = std::min(p.check_every, p.max_iters - t);
+            run(m);
+            t += m;
+            check(t);
+        }
+        if (tol_mode) {
+            const int slot = nchunk & 1;
+            cudaMemcpyAsync(&ctx->hstatus[slot], ctx->dstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st);
+            cudaEventRecord(ev[slot], st);
+            if (nchunk >= 1) {
+                // the previous chunk's flag: the GPU keeps running the chunk just queued
+                cudaEventSynchronize(ev[slot ^ 1]);
+                if (ctx->hstatus[slot ^ 1].stop) stopped = true;
+            }
+            ++nchunk;
+        }
+    }
+    K.out<<<lgrid, 128, 0, st>>>(planar, op, S[0], S[1], ctx->dstatus);
+    ctx->launches += 1;
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&ctx->hstatus[0], ctx->dstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    for (int q = 0; q < 2; ++q)
+        if (ev[q]) cudaEventDestroy(ev[q]);
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "solve");
+    return VOMT_OK;
+}
+
+}  // namespace vomt

@@ -1,0 +1,577 @@
+// Streaming engine, marching form: S iterations of Section 7.2 (vector OMT) in one pass
+// over the grid.
+//
+// A warp owns a strip of 32 columns, one per lane, and marches up a chunk of rows.  Per
+// row-step it takes in one row of the state (phi, u_x, u_y, w) and of b, and every stage
+// s = 1 .. S advances one row by one iteration: with rows y - s and y - s + 1 of the
+// iterate after s - 1 iterations at hand, stage s forms row y - s of the next one.  All
+// of it stays in registers: the row above is what the previous stage has just produced,
+// 2u' - u of the row below is carried from the previous row-step, and the neighbours
+// along x are the neighbouring lanes' (shuffles).  u' is computed once per point and
+// stage, and there is no barrier.
+//
+// The neighbours that a strip and a chunk lack cost redundant work: each stage loses one
+// column on either side and one row at either end, so a warp writes 32 - 2 S columns and
+// reads S more rows on either side of its chunk.  In return one pass over memory serves S
+// iterations: 2048^2 with three channels takes 25 us per iteration at S = 4 (a pass moves
+// 0.47 GB in 100 us, 70% of the measured copy rate, the rest is issue: 0.7 instructions
+// per cycle and scheduler), where one iteration per pass with TMA tiles takes 79 us and
+// is bound by HBM alone; 1024^2 with one channel 3.4 us (was 9.2), 512^2 with eight
+// channels 21 us (118 us: the recomputed shrinks of the one-iteration kernel spill).
+//
+// The state is kept in units of the thresholds: u / mu and w / nu.  The shrinks then have
+// the thresholds 1 and alpha, the gradients enter without mu and nu, and a sum of squares
+// that underflows belongs to a flux that shrinks to zero anyway, so the reciprocal square
+// root needs no denormal handling (at three channels about 30 of 142 instructions per
+// point and stage less than with u and w themselves).
+//
+// Rows and columns outside the grid hold finite values that never reach a stored point:
+// the differences across the grid's edge are multiplied by 0.
+#pragma once
+
+#include <stdint.h>
+
+#include "internal.h"
+#include "march2d.h"
+#include "pdhg_device.cuh"
+
+namespace vomt {
+namespace march {
+
+constexpr int WARPS = 4, NTHR = 32 * WARPS;      // warps per block, each on its own strip and chunk
+
+// Rows in flight per warp (a power of two).  Four cover the latency of HBM (at 2048^2, three
+// channels, S = 3, eight rows were no faster); from six channels on a row is 5 KB and more
+// and two leave room for a second block on the SM.
+__host__ __device__ constexpr int depth(int K) { return K <= 5 ? 4 : 2; }
+// Blocks per SM the registers are limited for.
+__host__ __device__ constexpr int min_blocks(int K, int S)
+{
+    return K == 1 ? 6 : (K == 2 ? 4 : (K == 3 ? (S == 4 ? 3 : (S == 2 ? 4 : 5)) : (S == 1 && K <= 5 ? 3 : 2)));
+}
+
+__host__ __device__ constexpr int pairs(int K) { return K * (K - 1) / 2; }
+__host__ __device__ constexpr int slots(int K) { return pairs(K) > 0 ? pairs(K) : 1; }
+// Number of the pair lo < hi of K channels in the order (0,1), (0,2), ..., (1,2), ...
+__host__ __device__ constexpr int pair_at(int K, int lo, int hi) { return lo * (2 * K - lo - 1) / 2 + hi - lo - 1; }
+
+// State layout: the groups of four values of a point (phi, u_x, u_y, w, padded with zeros),
+// interleaved in blocks of 32 columns, float4 [y][x / 32][group][x % 32]; b likewise.  A
+// lane moves four values per access, rows of any length are aligned, and all groups of a
+// point sit at fixed distances from one address.  w holds one value per pair of channels
+// (pairs without an edge stay zero).
+template <int K>
+struct Quads {
+    static constexpr int NQ = (3 * K + pairs(K) + 3) / 4, NB = (K + 3) / 4;
+};
+__host__ __device__ inline size_t quad_at(int n, int groups, int y, int x)
+{
+    return ((size_t)y * ((n + 31) >> 5) + (x >> 5)) * groups * 32 + (x & 31);
+}
+
+__device__ __forceinline__ float rsq(float s2)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s2));
+    return r;
+}
+
+// shrink_u and shrink_w of Section 7.2 on one point; t: the threshold (1 unless REG)
+template <int K, int UN, bool REG>
+__device__ __forceinline__ void shrink_u(float (&vx)[K], float (&vy)[K], float t)
+{
+    if (UN == VOMT_U_L12) {
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            const float r = rsq(vx[c] * vx[c] + vy[c] * vy[c]), f = fmaxf(1.0f - (REG ? t * r : r), 0.0f);
+            vx[c] *= f;
+            vy[c] *= f;
+        }
+    } else if (UN == VOMT_U_L2) {
+        float s2 = 0.0f;
+#pragma unroll
+        for (int c = 0; c < K; ++c) s2 += vx[c] * vx[c] + vy[c] * vy[c];
+        const float r = rsq(s2), f = fmaxf(1.0f - (REG ? t * r : r), 0.0f);
+#pragma unroll
+        for (int c = 0; c < K; ++c) { vx[c] *= f; vy[c] *= f; }
+    } else {
+#pragma unroll
+        for (int c = 0; c < K; ++c) { vx[c] = dev::soft(vx[c], t); vy[c] = dev::soft(vy[c], t); }
+    }
+}
+// (w is in units of nu, its threshold alpha may be of any size: the guarded factor)
+template <int L, int WN>
+__device__ __forceinline__ void shrink_w(float (&x)[L], float t)
+{
+    if (WN == VOMT_W_L1) {
+#pragma unroll
+        for (int e = 0; e < L; ++e) x[e] = dev::soft(x[e], t);
+    } else {
+        float s2 = 0.0f;
+#pragma unroll
+        for (int e = 0; e < L; ++e) s2 += x[e] * x[e];
+        const float f = dev::shrink2_factor(s2, t);
+#pragma unroll
+        for (int e = 0; e < L; ++e) x[e] *= f;
+    }
+}
+
+// 16-byte asynchronous copy to shared memory; bytes = 0 writes zeros and reads nothing
+__device__ __forceinline__ void copy16(float4 *dst, const float4 *src, uint32_t bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// One point's values of a row.
+template <int K>
+struct Row {
+    float p[K], x[K], y[K], w[slots(K)], b[K];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int c = 0; c < K; ++c) p[c] = x[c] = y[c] = b[c] = 0.0f;
+#pragma unroll
+        for (int e = 0; e < slots(K); ++e) w[e] = 0.0f;
+    }
+    __device__ __forceinline__ void state_from(const float4 *src)      // groups 32 apart
+    {
+        constexpr int NQ = Quads<K>::NQ;
+        float v[4 * NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            const float4 z = src[i * 32];
+            v[4 * i] = z.x; v[4 * i + 1] = z.y; v[4 * i + 2] = z.z; v[4 * i + 3] = z.w;
+        }
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            p[c] = v[c];
+            x[c] = v[K + c];
+            y[c] = v[2 * K + c];
+        }
+        w[0] = 0.0f;
+#pragma unroll
+        for (int e = 0; e < pairs(K); ++e) w[e] = v[3 * K + e];
+    }
+    __device__ __forceinline__ void b_from(const float4 *src)
+    {
+        constexpr int NB = Quads<K>::NB;
+        float v[4 * NB];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const float4 z = src[i * 32];
+            v[4 * i] = z.x; v[4 * i + 1] = z.y; v[4 * i + 2] = z.z; v[4 * i + 3] = z.w;
+        }
+#pragma unroll
+        for (int c = 0; c < K; ++c) b[c] = v[c];
+    }
+    __device__ __forceinline__ void state_to(float4 *dst) const
+    {
+        constexpr int NQ = Quads<K>::NQ;
+        float v[4 * NQ];
+#pragma unroll
+        for (int i = 0; i < 4 * NQ; ++i) v[i] = 0.0f;
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            v[c] = p[c];
+            v[K + c] = x[c];
+            v[2 * K + c] = y[c];
+        }
+#pragma unroll
+        for (int e = 0; e < pairs(K); ++e) v[3 * K + e] = w[e];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) dst[i * 32] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+};
+
+// ------------------------------------------------------------------ S iterations
+template <int K, int UN, int WN, int S, bool REG>
+__global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_constant__ MarchArgs a,
+                                                                  const __grid_constant__ MarchOp g)
+{
+    constexpr int L = slots(K), W = 32 - 2 * S, NQ = Quads<K>::NQ, NB = Quads<K>::NB, D = depth(K);
+    constexpr int ROW = (NQ + NB) * 32;
+    const int lane = threadIdx.x & 31;
+    const int wi = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    cudaGridDependencySynchronize();      // after the previous kernel (no-op for a normal launch)
+    // the next pass may be scheduled from here on; it waits for this one to finish
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (wi >= a.warps) return;            // whole warps
+    const int n = g.n;
+    const int strip = wi % a.strips, chunk = wi / a.strips;
+    const int x = strip * W - S + lane;
+    const int y0 = chunk * a.rows, y1 = min(n, y0 + a.rows);
+    const int ya = max(y0 - S, 0), yb = y1 + S;          // rows taken in: [ya, yb), zeros from n on
+    const bool in = x >= 0 && x < n;
+    const bool wr = in && lane >= S && lane < S + W;
+    const float ihx = x < n - 1 ? g.ih : 0.0f, mL = x > 0 ? 1.0f : 0.0f;
+    const float tu = REG ? g.su : 1.0f, tw = REG ? g.alpha * g.sw : g.alpha;
+    const int xc = min(max(x, 0), n - 1), blk = (n + 31) >> 5;
+    const float4 *pin = a.in + quad_at(n, NQ, ya, xc), *pb = a.b + quad_at(n, NB, ya, xc);
+    const ptrdiff_t dy = (ptrdiff_t)blk * NQ * 32, dyb = (ptrdiff_t)blk * NB * 32;
+    const ptrdiff_t to_out = a.out - a.in, to_prev = a.prev ? a.prev - a.in : 0;
+
+    // Rows arrive by asynchronous copies into a ring of D rows in shared memory, D - 1 rows
+    // ahead of their use; a lane reads back only what it copied itself, so waiting for its
+    // own copies is all the synchronisation there is.
+    extern __shared__ __align__(16) float4 ring_all[];
+    float4 *const ring = ring_all + (threadIdx.x >> 5) * (D * ROW) + lane;
+    auto fetch = [&](int y) {             // row y, the one pin and pb point at, into its slot
+        float4 *dst = ring + (y & (D - 1)) * ROW;
+        const uint32_t bytes = y < n && in ? 16u : 0u;
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) copy16(dst + i * 32, pin + i * 32, bytes);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) copy16(dst + (NQ + i) * 32, pb + i * 32, bytes);
+        copies_commit();
+        pin += dy;
+        pb += dyb;
+    };
+#pragma unroll
+    for (int q = 0; q < D - 1; ++q) fetch(ya + q);
+    if (a.st->stop) {
+        copies_wait<0>();
+        return;
+    }
+
+    Row<K> d[S];                          // row y - s of stage s, waiting for the row above it
+    float cy[S][K];                       // 2u'_y - u_y of the row below it
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+        d[q].zero();
+#pragma unroll
+        for (int c = 0; c < K; ++c) cy[q][c] = 0.0f;
+    }
+    // unrolled by two: a row's registers move from stage to stage, and the moves that the
+    // rotation costs are paid once per turn of the loop
+#pragma unroll 2
+    for (int y = ya; y < yb; ++y) {
+        fetch(y + D - 1);
+        copies_wait<D - 1>();
+        Row<K> cur;
+        cur.state_from(ring + (y & (D - 1)) * ROW);
+        cur.b_from(ring + (y & (D - 1)) * ROW + NQ * 32);
+#pragma unroll
+        for (int q = 0; q < S; ++q) {
+            if (q == S - 1 && S > 1 && a.prev) {
+                const int yp = y - (S - 1);
+                if (yp >= y0 && yp < y1 && wr) cur.state_to(const_cast<float4 *>(pin) + (to_prev - (D + S - 1) * dy));
+            }
+            // stage q + 1: row r = y - q - 1 from its values dq and the row above, cur
+            Row<K> &dq = d[q];
+            const int r = y - q - 1;
+            const float ihy = r < n - 1 ? g.ih : 0.0f, mD = r > 0 ? 1.0f : 0.0f;
+            Row<K> o;
+            float vx[K], vy[K], ubx[K], div[K];
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                const float right = __shfl_down_sync(0xffffffffu, dq.p[c], 1);
+                vx[c] = dq.x[c] + ihx * (right - dq.p[c]);
+                vy[c] = dq.y[c] + ihy * (cur.p[c] - dq.p[c]);
+                if (REG) { vx[c] *= g.su; vy[c] *= g.su; }
+            }
+            shrink_u<K, UN, REG>(vx, vy, tu);
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                ubx[c] = 2.0f * vx[c] - dq.x[c];
+                const float uby = 2.0f * vy[c] - dq.y[c];
+                div[c] = uby - mD * cy[q][c];
+                cy[q][c] = uby;
+                o.x[c] = vx[c];
+                o.y[c] = vy[c];
+            }
+            float wx[L], rr[K];
+            wx[0] = 0.0f;
+#pragma unroll
+            for (int lo = 0; lo < K; ++lo)
+#pragma unroll
+                for (int hi = lo + 1; hi < K; ++hi) {
+                    const int e = pair_at(K, lo, hi);
+                    wx[e] = dq.w[e] + g.inv[e] * (dq.p[lo] - dq.p[hi]);
+                    if (REG) wx[e] *= g.sw;
+                }
+            if (K > 1) shrink_w<L, WN>(wx, tw);
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                const float left = __shfl_up_sync(0xffffffffu, ubx[c], 1);
+                rr[c] = g.mu * (g.ih * ((ubx[c] - mL * left) + div[c])) + dq.b[c];
+            }
+#pragma unroll
+            for (int lo = 0; lo < K; ++lo)
+#pragma unroll
+                for (int hi = lo + 1; hi < K; ++hi) {
+                    const int e = pair_at(K, lo, hi);
+                    const float v = 2.0f * wx[e] - dq.w[e];
+                    rr[lo] -= g.nuinv[e] * v;
+                    rr[hi] += g.nuinv[e] * v;
+                }
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                o.p[c] = dq.p[c] + g.tau * rr[c];
+                o.b[c] = dq.b[c];
+            }
+#pragma unroll
+            for (int e = 0; e < L; ++e) o.w[e] = wx[e];
+            dq = cur;
+            cur = o;
+        }
+        const int yo = y - S;
+        if (yo >= y0 && yo < y1 && wr) cur.state_to(const_cast<float4 *>(pin) + (to_out - (D + S) * dy));
+    }
+    copies_wait<0>();
+}
+
+// ------------------------------------------------------------------ one check
+// The terms of a convergence check (the sums RED_*) of the iterate cur and its
+// predecessor prv.  The same march: both states' rows once, neighbours along x by
+// shuffles, the row below carried; strips write no columns, so a strip covers 30.  Sums
+// per thread and warp in pairs of FP32 numbers (CheckAcc), per block and grid in FP64.
+template <int K, int UN, int WN>
+__global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ CheckArgs a,
+                                                      const __grid_constant__ MarchOp g)
+{
+    constexpr int L = slots(K), NQ = Quads<K>::NQ, NB = Quads<K>::NB;
+    cudaGridDependencySynchronize();
+    if (a.st->stop) return;
+    const int lane = threadIdx.x & 31, n = g.n;
+    const float ih = g.ih, mu = g.mu, nu = g.nu, alpha = g.alpha;
+    dev::CheckAcc acc;
+    acc.zero();
+    for (int wi = blockIdx.x * WARPS + (threadIdx.x >> 5); wi < a.items; wi += gridDim.x * WARPS) {
+        const int strip = wi % a.strips, chunk = wi / a.strips;
+        const int x = strip * 30 - 1 + lane;
+        const int y0 = chunk * a.rows, y1 = min(n, y0 + a.rows);
+        const bool in = x >= 0 && x < n, own = in && lane >= 1 && lane < 31;
+        const float ihx = x < n - 1 ? ih : 0.0f, mL = x > 0 ? 1.0f : 0.0f;
+        const int xc = min(max(x, 0), n - 1), blk = (n + 31) >> 5;
+        Row<K> c0, p0;                    // row y of cur and prv
+        float dn[K], un_[K];              // u_y and u_y - its predecessor of the row below
+        const int yl = max(y0 - 1, 0);
+        c0.state_from(a.cur + quad_at(n, NQ, yl, xc));
+        p0.state_from(a.prv + quad_at(n, NQ, yl, xc));
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            un_[c] = y0 > 0 ? mu * c0.y[c] : 0.0f;
+            dn[c] = y0 > 0 ? mu * c0.y[c] - mu * p0.y[c] : 0.0f;
+        }
+        if (y0 > 0) {
+            c0.state_from(a.cur + quad_at(n, NQ, y0, xc));
+            p0.state_from(a.prv + quad_at(n, NQ, y0, xc));
+        }
+        for (int y = y0; y < y1; ++y) {
+            Row<K> c1, p1;                // the row above
+            const int yu = min(y + 1, n - 1);
+            c1.state_from(a.cur + quad_at(n, NQ, yu, xc));
+            p1.state_from(a.prv + quad_at(n, NQ, yu, xc));
+            c0.b_from(a.b + quad_at(n, NB, y, xc));
+            const float ihy = y < n - 1 ? ih : 0.0f;
+            float dph[K], ddiv[K], gwb[K], uxs[K], uxl[K], dnn[K], unn[K];
+            float nu_pt = 0.0f, dn_u = 0.0f, fdu = 0.0f, fdp = 0.0f, fd = 0.0f, fbb = 0.0f, fdw = 0.0f, fx = 0.0f;
+            float q2 = 0.0f, dist = 0.0f;
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                const float uxc = mu * c0.x[c], uyc = mu * c0.y[c], bc = c0.b[c], ph = c0.p[c];
+                const float dux = uxc - mu * p0.x[c], duy = uyc - mu * p0.y[c];
+                uxs[c] = uxc;
+                uxl[c] = mL * __shfl_up_sync(0xffffffffu, uxc, 1);
+                const float dxl = mL * __shfl_up_sync(0xffffffffu, dux, 1);
+                const float pr = __shfl_down_sync(0xffffffffu, ph, 1);
+                ddiv[c] = ih * ((dux - dxl) + (duy - dn[c]));
+                dnn[c] = duy;
+                unn[c] = uyc;
+                dph[c] = ph - p0.p[c];
+                gwb[c] = bc;
+                fdu += dux * dux + duy * duy;
+                fdp += dph[c] * dph[c];
+                fd += ph * bc;
+                fbb += bc * bc;
+                q2 += uxc * uxc + uyc * uyc;
+                const float gx = ihx > 0.0f ? ih * (pr - ph) : 0.0f, gy = ihy > 0.0f ? ih * (c1.p[c] - ph) : 0.0f;
+                if (UN == VOMT_U_L12) {
+                    nu_pt += sqrtf(uxc * uxc + uyc * uyc);
+                    const float gn = sqrtf(gx * gx + gy * gy), o = fmaxf(gn - 1.0f, 0.0f);
+                    dn_u = fmaxf(dn_u, gn);
+                    dist += o * o;
+                } else if (UN == VOMT_U_L2) {
+                    nu_pt += uxc * uxc + uyc * uyc;
+                    dn_u += gx * gx + gy * gy;
+                } else {
+                    nu_pt += fabsf(uxc) + fabsf(uyc);
+                    dn_u = fmaxf(dn_u, fmaxf(fabsf(gx), fabsf(gy)));
+                    const float ox = fmaxf(fabsf(gx) - 1.0f, 0.0f), oy = fmaxf(fabsf(gy) - 1.0f, 0.0f);
+                    dist += ox * ox + oy * oy;
+                }
+            }
+            if (UN == VOMT_U_L2) {
+                nu_pt = sqrtf(nu_pt);
+                dn_u = sqrtf(dn_u);
+                const float o = fmaxf(dn_u - 1.0f, 0.0f);
+                dist += o * o;
+            }
+            float nw_pt = 0.0f, dn_w = 0.0f;
+#pragma unroll
+            for (int lo = 0; lo < K; ++lo)
+#pragma unroll
+                for (int hi = lo + 1; hi < K; ++hi) {
+                    const int e = pair_at(K, lo, hi);
+                    const float we = nu * c0.w[e], dwe = we - nu * p0.w[e], ge = g.inv[e] * (c0.p[lo] - c0.p[hi]);
+                    fdw += dwe * dwe;
+                    q2 += we * we;
+                    gwb[lo] -= g.inv[e] * we;
+                    gwb[hi] += g.inv[e] * we;
+                    ddiv[lo] -= g.inv[e] * dwe;
+                    ddiv[hi] += g.inv[e] * dwe;
+                    if (WN == VOMT_W_L1) {
+                        nw_pt += fabsf(we);
+                        dn_w = fmaxf(dn_w, fabsf(ge));
+                        const float o = fmaxf(fabsf(ge) - alpha, 0.0f);
+                        dist += o * o;
+                    } else {
+                        nw_pt += we * we;
+                        dn_w += ge * ge;
+                    }
+                }
+            if (WN == VOMT_W_L2) {
+                nw_pt = sqrtf(nw_pt);
+                dn_w = sqrtf(dn_w);
+                const float o = fmaxf(dn_w - alpha, 0.0f);
+                if (g.l > 0) dist += o * o;
+            }
+            float rr = 0.0f;
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                const float rc = dev::residual_c(ih, uxs[c], uxl[c], unn[c], un_[c], gwb[c]);
+                rr += rc * rc;
+                fx += dph[c] * ddiv[c];
+                un_[c] = unn[c];
+                dn[c] = dnn[c];
+            }
+            if (own) {
+                acc.add(RED_RR, rr);
+                acc.add(RED_P, nu_pt + alpha * nw_pt);
+                if (g.reg) {
+                    acc.add(RED_P, g.eps * q2);
+                    acc.add(RED_DIST, dist);
+                }
+                acc.add(RED_D, fd);
+                acc.add(RED_BB, fbb);
+                acc.add(RED_DU, fdu);
+                acc.add(RED_DW, fdw);
+                acc.add(RED_DP, fdp);
+                acc.add(RED_X, fx);
+                float di = fmaxf(dn_u - 1.0f, 0.0f);
+                if (g.l > 0) di = fmaxf(di, dn_w - alpha);
+                acc.max(RED_MAX, di);
+            }
+            c0 = c1;
+            p0 = p1;
+        }
+    }
+    dev::block_sum_store<NTHR>(acc, a.partials + (size_t)blockIdx.x * NRED);
+}
+
+// ------------------------------------------------------------------ layouts
+// Planar fields <-> the engine's layout (u and w in units of mu and nu); b = rho1 - rho0.
+template <int K>
+__global__ void k_march_in(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g, float4 *state,
+                           float4 *bq)
+{
+    const int n = g.n;
+    const size_t nn = (size_t)n * n;
+    const float imu = 1.0f / g.mu, inu = 1.0f / g.nu;
+    for (int y = blockIdx.y; y < n; y += gridDim.y) {
+        const int x = blockIdx.x * blockDim.x + threadIdx.x;
+        if (x >= n) continue;
+        const size_t q = (size_t)y * n + x;
+        Row<K> r;
+        r.zero();
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            r.b[c] = a.rho1[c * nn + q] - a.rho0[c * nn + q];
+            if (a.warm) {
+                r.p[c] = a.phi[c * nn + q];
+                r.x[c] = x < n - 1 ? imu * a.u[c * nn + q] : 0.0f;
+                r.y[c] = y < n - 1 ? imu * a.u[(K + c) * nn + q] : 0.0f;
+            }
+        }
+        if (a.warm)
+#pragma unroll
+            for (int e = 0; e < pairs(K); ++e)
+                if (g.edge[e] >= 0) r.w[e] = inu * a.w[g.edge[e] * nn + q];
+        r.state_to(state + quad_at(n, Quads<K>::NQ, y, x));
+        float v[4 * Quads<K>::NB];
+#pragma unroll
+        for (int c = 0; c < 4 * Quads<K>::NB; ++c) v[c] = c < K ? r.b[c < K ? c : 0] : 0.0f;
+        float4 *dst = bq + quad_at(n, Quads<K>::NB, y, x);
+#pragma unroll
+        for (int i = 0; i < Quads<K>::NB; ++i)
+            dst[i * 32] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
+}
+
+template <int K>
+__global__ void k_march_out(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g,
+                            const float4 *s0, const float4 *s1, const DevStatus *st)
+{
+    const int n = g.n;
+    const size_t nn = (size_t)n * n;
+    const float4 *state = st->slot ? s1 : s0;
+    for (int y = blockIdx.y; y < n; y += gridDim.y) {
+        const int x = blockIdx.x * blockDim.x + threadIdx.x;
+        if (x >= n) continue;
+        const size_t q = (size_t)y * n + x;
+        Row<K> r;
+        r.state_from(state + quad_at(n, Quads<K>::NQ, y, x));
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            a.phi[c * nn + q] = r.p[c];
+            a.u[c * nn + q] = g.mu * r.x[c];
+            a.u[(K + c) * nn + q] = g.mu * r.y[c];
+        }
+#pragma unroll
+        for (int e = 0; e < pairs(K); ++e)
+            if (g.edge[e] >= 0) a.w[g.edge[e] * nn + q] = g.nu * r.w[e];
+    }
+}
+
+// ------------------------------------------------------------------ dispatch
+template <int K, int UN, int WN, bool REG>
+Kernels kernels_of()
+{
+    Kernels q = {};
+    q.step[0] = k_march<K, UN, WN, 1, REG>;
+    if constexpr (K <= 6) q.step[1] = k_march<K, UN, WN, 2, REG>;
+    if constexpr (K <= 3) q.step[2] = k_march<K, UN, WN, 4, REG>;
+    q.check = k_march_check<K, UN, WN>;
+    q.in = k_march_in<K>;
+    q.out = k_march_out<K>;
+    q.groups = Quads<K>::NQ;
+    q.bgroups = Quads<K>::NB;
+    q.smem = depth(K) * (Quads<K>::NQ + Quads<K>::NB) * 512 * WARPS;
+    return q;
+}
+
+// The plain problem with the default norms has its own kernels; every other one takes
+// those with the regularisation's factors (1 without it).
+template <int K>
+Kernels pick_norms(int un, int wn, bool reg)
+{
+    if (K == 1) wn = VOMT_W_L1;           // no edges
+    if (un == VOMT_U_L12 && wn == VOMT_W_L1) return reg ? kernels_of<K, 0, 0, true>() : kernels_of<K, 0, 0, false>();
+    if constexpr (K > 1) {
+        if (wn == VOMT_W_L2)
+            return un == VOMT_U_L12 ? kernels_of<K, 0, 1, true>()
+                                    : (un == VOMT_U_L2 ? kernels_of<K, 1, 1, true>() : kernels_of<K, 2, 1, true>());
+    }
+    return un == VOMT_U_L2 ? kernels_of<K, 1, 0, true>() : kernels_of<K, 2, 0, true>();
+}
+
+}  // namespace march
+}  // namespace vomt

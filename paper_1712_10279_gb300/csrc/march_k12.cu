@@ -1,0 +1,14 @@
+// Kernels of the marching form for one and two channels (a unit of its own, so that the
+// units compile in parallel).
+#include "march2d.cuh"
+
+namespace vomt {
+namespace march {
+
+Kernels pick_k12(int k, int un, int wn, bool reg)
+{
+    return k == 1 ? pick_norms<1>(un, wn, reg) : pick_norms<2>(un, wn, reg);
+}
+
+}  // namespace march
+}  // namespace vomt

@@ -1,0 +1,11 @@
+// Kernels of the marching form for 5 channels (a unit of its own, so that the units
+// compile in parallel).
+#include "march2d.cuh"
+
+namespace vomt {
+namespace march {
+
+Kernels pick_k5(int, int un, int wn, bool reg) { return pick_norms<5>(un, wn, reg); }
+
+}  // namespace march
+}  // namespace vomt

@@ -1,0 +1,11 @@
+// Kernels of the marching form for 7 channels (a unit of its own, so that the units
+// compile in parallel).
+#include "march2d.cuh"
+
+namespace vomt {
+namespace march {
+
+Kernels pick_k7(int, int un, int wn, bool reg) { return pick_norms<7>(un, wn, reg); }
+
+}  // namespace march
+}  // namespace vomt

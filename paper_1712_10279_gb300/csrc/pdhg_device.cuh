@@ -153,6 +153,23 @@ __device__ __forceinline__ float two_sum(float a, float b, float &e)
     return s;
 }
 
+// ih * ((ux - xl) + (uy - yd)) + gb with the rounding errors of the
+// differences, their sum, the product and the final sum carried along (the
+// compensated evaluation of Ogita, Rump and Oishi, "Accurate sum and dot
+// product", 2005): about twice FP32 precision for the constraint residual,
+// whose terms cancel as the iteration converges.
+__device__ __forceinline__ float residual_c(float ih, float ux, float xl, float uy, float yd, float gb)
+{
+    float e1, e2, e3, e4;
+    const float d1 = two_sum(ux, -xl, e1);
+    const float d2 = two_sum(uy, -yd, e2);
+    const float s = two_sum(d1, d2, e3);
+    const float p = ih * s;
+    const float pe = fmaf(ih, s, -p);
+    const float r = two_sum(p, gb, e4);
+    return r + (e4 + (pe + ih * ((e1 + e2) + e3)));
+}
+
 // One thread's share of a convergence check: each sum slot is a pair of FP32
 // numbers (hi, lo) that TwoSum keeps equal to the exact running sum up to the
 // rounding of lo (about twice FP32 precision); the maximum slot is a plain FP32

@@ -195,23 +195,6 @@ __device__ __forceinline__ void sts(float *p, const float (&v)[K])
     }
 }
 
-// ih * ((ux - xl) + (uy - yd)) + gb with the rounding errors of the
-// differences, their sum, the product and the final sum carried along (the
-// compensated evaluation of Ogita, Rump and Oishi, "Accurate sum and dot
-// product", 2005): about twice FP32 precision for the constraint residual,
-// whose terms cancel as the iteration converges.
-__device__ __forceinline__ float residual_c(float ih, float ux, float xl, float uy, float yd, float gb)
-{
-    float e1, e2, e3, e4;
-    const float d1 = two_sum(ux, -xl, e1);
-    const float d2 = two_sum(uy, -yd, e2);
-    const float s = two_sum(d1, d2, e3);
-    const float p = ih * s;
-    const float pe = fmaf(ih, s, -p);
-    const float r = two_sum(p, gb, e4);
-    return r + (e4 + (pe + ih * ((e1 + e2) + e3)));
-}
-
 // Two tagged words (fields 2j and 2j+1 of one point) in one 16-byte access.
 __device__ __forceinline__ void st_tagged2(unsigned long long *p, float v0, float v1, uint32_t tag)
 {

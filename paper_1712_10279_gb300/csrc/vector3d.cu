@@ -473,15 +473,8 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * (size_t)nblocks * NRED,
                        "partials");
     if (rc) return rc;
-    const int max_checks = p.max_iters / p.check_every + 2;
-    if (ctx->hist_cap < max_checks) {
-        if (ctx->dhist) cudaFree(ctx->dhist);
-        ctx->dhist = nullptr;
-        ctx->hist_cap = 0;
-        e = cudaMalloc(&ctx->dhist, sizeof(double) * NMET * (size_t)max_checks);
-        if (e != cudaSuccess) return set_cuda_error(ctx, e, "history");
-        ctx->hist_cap = max_checks;
-    }
+    rc = ensure_history(ctx, p.max_iters / p.check_every + 2);
+    if (rc) return rc;
     e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "status reset");
     const int pblocks = (int)std::min<size_t>((m + 255) / 256, 4096);
@@ -511,7 +504,7 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
         launch_pdl(L.metrics, dim3(mblocks), dim3(T3), 0, st, si[cur], si[cur ^ 1], (const float *)b, g, s,
                    ctx->partials, (const DevStatus *)ctx->dstatus);
         launch_pdl(k_finalize, dim3(1), dim3(kFinThreads), 0, st, (const double *)ctx->partials, mblocks, cfg, t,
-                   ctx->dstatus, ctx->dhist, ctx->hist_cap);
+                   ctx->dstatus, ctx->dhist, ctx->hist_cap, 0);
         ctx->launches += 2;
     };
     if (p.max_iters == 0) check(0, 0);

@@ -240,15 +240,8 @@ int resident_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveC
     a.rows = (unsigned long long *)(base + xch_bytes);
     a.ctl = (dev::ResCtl *)(base + xch_bytes + rows_bytes);
     a.st = ctx->dstatus;
-    const int max_checks = p.max_iters / p.check_every + 2;
-    if (ctx->hist_cap < max_checks) {
-        if (ctx->dhist) cudaFree(ctx->dhist);
-        ctx->dhist = nullptr;
-        ctx->hist_cap = 0;
-        cudaError_t e = cudaMalloc(&ctx->dhist, sizeof(double) * NMET * (size_t)max_checks);
-        if (e != cudaSuccess) return set_cuda_error(ctx, e, "history");
-        ctx->hist_cap = max_checks;
-    }
+    rc = ensure_history(ctx, p.max_iters / p.check_every + 2);
+    if (rc) return rc;
     a.hist = ctx->dhist;
     a.hist_cap = ctx->hist_cap;
     ctx->hist_raw = true;            // the kernel's check rows hold raw sums (finish_raw_row)

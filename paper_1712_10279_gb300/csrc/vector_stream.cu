@@ -477,7 +477,7 @@ Launchers pick(int k, int un, int wn)
 // Fixed-order sum of the per-block partials, the stopping decision and the
 // history row.  One block of 256 threads.
 __global__ void k_finalize(const double *__restrict__ partials, int nblocks, SolveCfg cfg, int t,
-                           DevStatus *st, double *hist, int hist_cap)
+                           DevStatus *st, double *hist, int hist_cap, int slot)
 {
     cudaGridDependencySynchronize();
     if (st->stop) return;
@@ -519,6 +519,7 @@ __global__ void k_finalize(const double *__restrict__ partials, int nblocks, Sol
             for (int q = 0; q < NMET; ++q) hist[(size_t)st->checks * NMET + q] = m[q];
         st->checks += 1;
         st->iter = t;
+        st->slot = slot;
         if (!finite) { st->error = VOMT_ERR_NONFINITE; st->stop = 1; }
         if (conv) st->stop = 1;
     }
@@ -567,6 +568,9 @@ int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg
                  const vomt_params &p, const float *rho0, const float *rho1,
                  float *u, float *w, float *phi, cudaStream_t st)
 {
+    bool taken = false;
+    const int mrc = march_solve(ctx, g, s, cfg, p, rho0, rho1, u, w, phi, st, &taken);
+    if (mrc || taken) return mrc;
     ctx->hist_raw = false;           // k_finalize writes finished rows
     const int n = s.n, k = g.k, l = g.l;
     const size_t nn = (size_t)n * n;
@@ -590,15 +594,8 @@ int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg
     rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * (size_t)nblocks * NRED,
                        "partials");
     if (rc) return rc;
-    const int max_checks = p.max_iters / p.check_every + 2;
-    if (ctx->hist_cap < max_checks) {
-        if (ctx->dhist) cudaFree(ctx->dhist);
-        ctx->dhist = nullptr;
-        ctx->hist_cap = 0;
-        cudaError_t e = cudaMalloc(&ctx->dhist, sizeof(double) * NMET * (size_t)max_checks);
-        if (e != cudaSuccess) return set_cuda_error(ctx, e, "history");
-        ctx->hist_cap = max_checks;
-    }
+    rc = ensure_history(ctx, p.max_iters / p.check_every + 2);
+    if (rc) return rc;
     cudaError_t e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "status reset");
     const int pblocks = (int)((nn + 255) / 256 < 2048 ? (nn + 255) / 256 : 2048);
@@ -618,12 +615,12 @@ int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg
         launch_pdl(L.metrics, dim3(mblocks), blk, 0, st, si[cur], si[cur ^ 1], (const float *)b, g, s, ctx->partials,
                    (const DevStatus *)ctx->dstatus);
         launch_pdl(k_finalize, dim3(1), dim3(kFinThreads), 0, st, (const double *)ctx->partials, mblocks, cfg, t,
-                   ctx->dstatus, ctx->dhist, ctx->hist_cap);
+                   ctx->dstatus, ctx->dhist, ctx->hist_cap, 0);
         ctx->launches += 2;
     };
     if (p.max_iters == 0) {
         L.metrics<<<mblocks, blk, 0, st>>>(si[0], si[0], b, g, s, ctx->partials, ctx->dstatus);
-        k_finalize<<<1, kFinThreads, 0, st>>>(ctx->partials, mblocks, cfg, 0, ctx->dstatus, ctx->dhist, ctx->hist_cap);
+        k_finalize<<<1, kFinThreads, 0, st>>>(ctx->partials, mblocks, cfg, 0, ctx->dstatus, ctx->dhist, ctx->hist_cap, 0);
         ctx->launches += 2;
     }
     const bool tol_mode = cfg.tol_gap > 0.0;
@@ -649,7 +646,7 @@ int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg
                     launch_pdl(L.metrics, dim3(mblocks), blk, 0, ctx->cap_stream, si[cur], si[cur ^ 1], (const float *)b, g,
                                s, ctx->partials, (const DevStatus *)ctx->dstatus);
                     launch_pdl(k_finalize, dim3(1), dim3(kFinThreads), 0, ctx->cap_stream, (const double *)ctx->partials,
-                               mblocks, cfg, -p.check_every, ctx->dstatus, ctx->dhist, ctx->hist_cap);
+                               mblocks, cfg, -p.check_every, ctx->dstatus, ctx->dhist, ctx->hist_cap, 0);
                 }
             }
             if (cudaStreamEndCapture(ctx->cap_stream, &graph) != cudaSuccess ||
@@ -891,7 +888,7 @@ int noalloc_solve(int n, const float *rho0, const float *rho1, const vomt_graph 
     Launchers L = pick(k, p.u_norm, p.w_norm);
     if (p.max_iters == 0) {
         L.metrics<<<mblocks, blk, 0, st>>>(si[0], si[0], b, g, s, partials, dstatus);
-        k_finalize<<<1, kFinThreads, 0, st>>>(partials, mblocks, cfg, 0, dstatus, nullptr, 0);
+        k_finalize<<<1, kFinThreads, 0, st>>>(partials, mblocks, cfg, 0, dstatus, nullptr, 0, 0);
         launches += 2;
     }
     const bool tol_mode = cfg.tol_gap > 0.0;
@@ -906,7 +903,7 @@ int noalloc_solve(int n, const float *rho0, const float *rho1, const vomt_graph 
             ++launches;
             if (tt % p.check_every == 0 || tt == p.max_iters) {
                 L.metrics<<<mblocks, blk, 0, st>>>(si[cur], si[cur ^ 1], b, g, s, partials, dstatus);
-                k_finalize<<<1, kFinThreads, 0, st>>>(partials, mblocks, cfg, tt, dstatus, nullptr, 0);
+                k_finalize<<<1, kFinThreads, 0, st>>>(partials, mblocks, cfg, tt, dstatus, nullptr, 0, 0);
                 launches += 2;
             }
         }
