@@ -199,6 +199,20 @@ int run_engine(vomt_ctx *ctx, const OpDev &op, const StepDev &s, const SolveCfg 
     if (p.engine != VOMT_ENGINE_STREAM) {
         ResidentPlan plan;
         if (resident_plan(s.n, op.k, ctx->sm_count, p.halo, &plan)) {
+            // Tiles of four points per thread (two from five channels on) spill, and rings of one
+            // cell (two from three channels on) exchange too often; the marching form of the
+            // streaming engine is faster there (us per iteration, k = 1, 352^2: 1.50 against
+            // 1.95; k = 3, 320^2: 2.18 against 2.33, 352^2: 2.25 against 3.85, 512^2: 3.3 against
+            // 8.3; k = 4, 320^2: 3.0 against 3.7; k = 5, 256^2: 3.56 against 3.65; k = 8, 256^2:
+            // 7.4 against 9.6) and slower short of it (k = 1, 320^2: 1.48 against 1.30; k = 3,
+            // 288^2: 1.94 against 1.76; k = 8, 128^2: 5.3 against 3.4).  A ring width asked for
+            // asks for the resident engine.
+            if (p.engine == VOMT_ENGINE_AUTO && p.halo == 0 &&
+                (plan.P > (op.k <= 4 ? 2 : 1) || (plan.Gx * plan.Gy > 1 && plan.H <= (op.k <= 2 ? 1 : 2)))) {
+                bool taken = false;
+                rc = march_solve(ctx, op, s, cfg, p, rho0, rho1, u, w, phi, st, &taken);
+                if (rc || taken) return rc;
+            }
             rc = resident_solve(ctx, op, s, cfg, p, plan, rho0, rho1, u, w, phi, st);
             if (rc == VOMT_OK) {
                 *engine = VOMT_ENGINE_RESIDENT;

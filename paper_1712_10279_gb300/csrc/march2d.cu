@@ -7,33 +7,14 @@
 #include "march2d.h"
 
 namespace vomt {
-namespace {
-
-using namespace march;
-
-constexpr int kWarps = 4;             // warps per block (march2d.cuh)
-
-Kernels pick(int k, int un, int wn, bool reg)
-{
-    switch (k) {
-        case 1:
-        case 2: return pick_k12(k, un, wn, reg);
-        case 3: return pick_k3(k, un, wn, reg);
-        case 4: return pick_k4(k, un, wn, reg);
-        case 5: return pick_k5(k, un, wn, reg);
-        case 6: return pick_k6(k, un, wn, reg);
-        case 7: return pick_k7(k, un, wn, reg);
-        default: return pick_k8(k, un, wn, reg);
-    }
-}
 
 // The pairwise form of a channel graph's operator: every row of G is +1/c_e at one channel
 // and -1/c_e at a later one, Dv its transpose, all weights 1.  False for any other operator
 // (matrix fields).
-bool graph_of(const OpDev &g, const StepDev &s, const SolveCfg &cfg, MarchOp *out)
+bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out)
 {
     if (g.k < 1 || g.k > KVEC || g.l > LVEC) return false;
-    MarchOp m;
+    march::MarchOp m;
     memset(&m, 0, sizeof m);
     for (int e = 0; e < LVEC; ++e) m.edge[e] = -1;
     for (int c = 0; c < g.k; ++c)
@@ -65,15 +46,37 @@ bool graph_of(const OpDev &g, const StepDev &s, const SolveCfg &cfg, MarchOp *ou
     m.eps = s.eps;
     m.su = s.reg ? s.su : 1.0f;
     m.sw = s.reg ? s.sw : 1.0f;
-    (void)cfg;
     *out = m;
     return true;
+}
+
+namespace {
+
+using namespace march;
+
+constexpr int kWarps = 4;             // warps per block (march2d.cuh)
+constexpr int kSmemBlock = 227 * 1024;    // most shared memory of a block
+constexpr int kSmemSM = 228 * 1024;   // shared memory of an SM (each block takes 1 KB besides its own)
+
+Kernels pick(int k, int un, int wn, bool reg)
+{
+    switch (k) {
+        case 1:
+        case 2: return pick_k12(k, un, wn, reg);
+        case 3: return pick_k3(k, un, wn, reg);
+        case 4: return pick_k4(k, un, wn, reg);
+        case 5: return pick_k5(k, un, wn, reg);
+        case 6: return pick_k6(k, un, wn, reg);
+        case 7: return pick_k7(k, un, wn, reg);
+        default: return pick_k8(k, un, wn, reg);
+    }
 }
 
 // One kind of pass: its stages, chunks and estimated time.
 struct Pass {
     int stages = 0, rows = 0, strips = 0, warps = 0, blocks = 0;
     double us = 0.0;
+    int smem = 0;
 };
 
 // Chunk rows of a pass with S stages: those of the least arithmetic time.  A warp takes
@@ -118,7 +121,7 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
 {
     *taken = false;
     MarchOp op;
-    if (p.u_norm > VOMT_U_L1 || p.w_norm > VOMT_W_L2 || !graph_of(g, s, cfg, &op)) return VOMT_OK;
+    if (p.u_norm > VOMT_U_L1 || p.w_norm > VOMT_W_L2 || !march_op(g, s, &op)) return VOMT_OK;
     const int n = s.n, k = g.k;
     const int interval = std::min(p.check_every, std::max(p.max_iters, 0));
     if (k <= 4 && interval < 4) return VOMT_OK;
@@ -128,7 +131,7 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
     int main_pass = 0;
     for (int q = 0; q < 3; ++q) {
         if (!K.step[q]) continue;
-        cudaError_t e = cudaFuncSetAttribute((const void *)K.step[q], cudaFuncAttributeMaxDynamicSharedMemorySize, K.smem);
+        cudaError_t e = cudaFuncSetAttribute((const void *)K.step[q], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBlock);
         int per_sm = 0;
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)K.step[q], 32 * kWarps, K.smem);
@@ -140,6 +143,15 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
             main_pass = q;
     }
     if (pass[0].stages == 0) return VOMT_OK;
+    // A pass starts while the one before it drains, and would fill whatever slots are free
+    // by then, three blocks on some SMs and one on others (2048^2, three channels, two blocks
+    // per SM: 140 us a pass instead of 100).  So each pass asks for the shared memory that
+    // leaves room for just its share of blocks per SM.
+    for (int q = 0; q < 3; ++q) {
+        if (!pass[q].stages) continue;
+        const int share = (pass[q].blocks + ctx->sm_count - 1) / ctx->sm_count;
+        pass[q].smem = std::max(K.smem, kSmemSM / (share + 1));
+    }
 
     // b, two states, and the state one iteration before a check where a pass of several
     // iterations ends on it
@@ -190,7 +202,7 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
         a.rows = ps.rows;
         a.strips = ps.strips;
         a.warps = ps.warps;
-        launch_pdl(K.step[q], dim3(ps.blocks), dim3(32 * kWarps), (size_t)K.smem, st, a, op);
+        launch_pdl(K.step[q], dim3(ps.blocks), dim3(32 * kWarps), (size_t)ps.smem, st, a, op);
         ctx->launches += 1;
         before = a.prev ? a.prev : a.in;
         cur ^= 1;

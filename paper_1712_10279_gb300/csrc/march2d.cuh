@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
         const int y0 = chunk * a.rows, y1 = min(n, y0 + a.rows);
         const bool in = x >= 0 && x < n, own = in && lane >= 1 && lane < 31;
         const float ihx = x < n - 1 ? ih : 0.0f, mL = x > 0 ? 1.0f : 0.0f;
-        const int xc = min(max(x, 0), n - 1), blk = (n + 31) >> 5;
+        const int xc = min(max(x, 0), n - 1);
         Row<K> c0, p0;                    // row y of cur and prv
         float dn[K], un_[K];              // u_y and u_y - its predecessor of the row below
         const int yl = max(y0 - 1, 0);

@@ -57,4 +57,7 @@ Kernels pick_k7(int k, int un, int wn, bool reg);
 Kernels pick_k8(int k, int un, int wn, bool reg);
 
 }  // namespace march
+
+bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out);
+
 }  // namespace vomt
