@@ -206,11 +206,12 @@ int run_engine(vomt_ctx *ctx, const OpDev &op, const StepDev &s, const SolveCfg 
             // 8.3; k = 4, 320^2: 3.0 against 3.7; k = 5, 256^2: 3.56 against 3.65; k = 8, 256^2:
             // 7.4 against 9.6) and slower short of it (k = 1, 320^2: 1.48 against 1.30; k = 3,
             // 288^2: 1.94 against 1.76; k = 8, 128^2: 5.3 against 3.4).  A ring width asked for
-            // asks for the resident engine.
-            if (p.engine == VOMT_ENGINE_AUTO && p.halo == 0 &&
+            // asks for the resident engine.  For the default norms the marching kernels exist in
+            // the resident kernels' order of operations, so results stay what they were.
+            if (p.engine == VOMT_ENGINE_AUTO && p.halo == 0 && p.u_norm == VOMT_U_L12 && p.w_norm == VOMT_W_L1 && !s.reg &&
                 (plan.P > (op.k <= 4 ? 2 : 1) || (plan.Gx * plan.Gy > 1 && plan.H <= (op.k <= 2 ? 1 : 2)))) {
                 bool taken = false;
-                rc = march_solve(ctx, op, s, cfg, p, rho0, rho1, u, w, phi, st, &taken);
+                rc = march_solve(ctx, op, s, cfg, p, true, rho0, rho1, u, w, phi, st, &taken);
                 if (rc || taken) return rc;
             }
             rc = resident_solve(ctx, op, s, cfg, p, plan, rho0, rho1, u, w, phi, st);

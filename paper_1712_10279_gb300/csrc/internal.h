@@ -230,8 +230,9 @@ int ensure_buffer(vomt_ctx *ctx, void **p, size_t *cap, size_t bytes, const char
 int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg,
                  const vomt_params &p, const float *rho0, const float *rho1,
                  float *u, float *w, float *phi, cudaStream_t st);
-// its marching form for vector problems (march2d.cu); *taken: whether it ran the solve
-int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg, const vomt_params &p,
+// its marching form for vector problems (march2d.cu), in the order of operations of the
+// resident engine (res) or of the one-iteration kernels; *taken: whether it ran the solve
+int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg, const vomt_params &p, bool res,
                 const float *rho0, const float *rho1, float *u, float *w, float *phi, cudaStream_t st, bool *taken);
 // rows of the check history on the device
 int ensure_history(vomt_ctx *ctx, int rows);

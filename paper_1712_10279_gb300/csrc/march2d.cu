@@ -33,7 +33,6 @@ bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out)
         if (m.edge[q] >= 0) return false;
         m.edge[q] = e;
         m.inv[q] = g.G[e][lo];
-        m.nuinv[q] = s.nu * g.G[e][lo];
     }
     m.n = s.n;
     m.l = g.l;
@@ -44,6 +43,10 @@ bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out)
     m.tau = s.tau;
     m.alpha = s.alpha;
     m.eps = s.eps;
+    m.g1 = s.ih;
+    m.g2 = s.mu;
+    m.tu = s.reg ? s.mu * s.su : s.mu;
+    m.tw = s.reg ? s.alpha * s.nu * s.sw : s.alpha * s.nu;
     m.su = s.reg ? s.su : 1.0f;
     m.sw = s.reg ? s.sw : 1.0f;
     *out = m;
@@ -58,17 +61,17 @@ constexpr int kWarps = 4;             // warps per block (march2d.cuh)
 constexpr int kSmemBlock = 227 * 1024;    // most shared memory of a block
 constexpr int kSmemSM = 228 * 1024;   // shared memory of an SM (each block takes 1 KB besides its own)
 
-Kernels pick(int k, int un, int wn, bool reg)
+Kernels pick(int k, int un, int wn, bool reg, bool res)
 {
     switch (k) {
         case 1:
-        case 2: return pick_k12(k, un, wn, reg);
-        case 3: return pick_k3(k, un, wn, reg);
-        case 4: return pick_k4(k, un, wn, reg);
-        case 5: return pick_k5(k, un, wn, reg);
-        case 6: return pick_k6(k, un, wn, reg);
-        case 7: return pick_k7(k, un, wn, reg);
-        default: return pick_k8(k, un, wn, reg);
+        case 2: return pick_k12(k, un, wn, reg, res);
+        case 3: return pick_k3(k, un, wn, reg, res);
+        case 4: return pick_k4(k, un, wn, reg, res);
+        case 5: return pick_k5(k, un, wn, reg, res);
+        case 6: return pick_k6(k, un, wn, reg, res);
+        case 7: return pick_k7(k, un, wn, reg, res);
+        default: return pick_k8(k, un, wn, reg, res);
     }
 }
 
@@ -116,7 +119,7 @@ Pass plan_pass(int n, int k, int groups, int S, int blocks_per_sm, int sms)
 // device's memory, and up to four channels with fewer than four iterations between checks,
 // where the one-iteration kernels need no second layout and are as fast (2048^2, three
 // channels: 79 us against 84 with one stage).
-int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg, const vomt_params &p,
+int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg &cfg, const vomt_params &p, bool res,
                 const float *rho0, const float *rho1, float *u, float *w, float *phi, cudaStream_t st, bool *taken)
 {
     *taken = false;
@@ -125,7 +128,14 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
     const int n = s.n, k = g.k;
     const int interval = std::min(p.check_every, std::max(p.max_iters, 0));
     if (k <= 4 && interval < 4) return VOMT_OK;
-    const Kernels K = pick(k, p.u_norm, p.w_norm, s.reg != 0);
+    // the kernels' reciprocal square root takes sums of squares below 1.2e-38 for zero, which
+    // is right where the threshold is above their root
+    if (op.tu < 2e-19f || (g.l > 0 && op.tw < 2e-19f)) return VOMT_OK;
+    if (res) {
+        op.g1 = 1.0f;
+        op.g2 = s.mu * s.ih;
+    }
+    const Kernels K = pick(k, p.u_norm, p.w_norm, s.reg != 0, res);
 
     Pass pass[3];
     int main_pass = 0;

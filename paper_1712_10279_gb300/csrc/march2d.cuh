@@ -19,11 +19,12 @@
 // is bound by HBM alone; 1024^2 with one channel 3.4 us (was 9.2), 512^2 with eight
 // channels 21 us (118 us: the recomputed shrinks of the one-iteration kernel spill).
 //
-// The state is kept in units of the thresholds: u / mu and w / nu.  The shrinks then have
-// the thresholds 1 and alpha, the gradients enter without mu and nu, and a sum of squares
-// that underflows belongs to a flux that shrinks to zero anyway, so the reciprocal square
-// root needs no denormal handling (at three channels about 30 of 142 instructions per
-// point and stage less than with u and w themselves).
+// Every value is rounded as the one-iteration kernels (or, RES, the resident kernels) round
+// it, operation by operation, so that the iterates are theirs bit for bit: after hundreds
+// of iterations w, which is zero except where a difference of phi passes its threshold,
+// differs by 1e-5 and more of its norm between two roundings of phi.  The sums over
+// channels of the graph gradient reduce to the two channels of a pair (the other terms are
+// exact zeros), which keeps its matrix out of the registers.
 //
 // Rows and columns outside the grid hold finite values that never reach a stored point:
 // the differences across the grid's edge are multiplied by 0.
@@ -76,14 +77,18 @@ __device__ __forceinline__ float rsq(float s2)
     return r;
 }
 
-// shrink_u and shrink_w of Section 7.2 on one point; t: the threshold (1 unless REG)
-template <int K, int UN, bool REG>
+// shrink_2 factor of Appendix B (dev::shrink2_factor) where sums of squares that flush to
+// zero are below the squared threshold
+__device__ __forceinline__ float factor(float s2, float t) { return fmaxf(1.0f - t * rsq(s2), 0.0f); }
+
+// shrink_u and shrink_w of Section 7.2 on one point, threshold t
+template <int K, int UN>
 __device__ __forceinline__ void shrink_u(float (&vx)[K], float (&vy)[K], float t)
 {
     if (UN == VOMT_U_L12) {
 #pragma unroll
         for (int c = 0; c < K; ++c) {
-            const float r = rsq(vx[c] * vx[c] + vy[c] * vy[c]), f = fmaxf(1.0f - (REG ? t * r : r), 0.0f);
+            const float f = factor(vx[c] * vx[c] + vy[c] * vy[c], t);
             vx[c] *= f;
             vy[c] *= f;
         }
@@ -91,7 +96,7 @@ __device__ __forceinline__ void shrink_u(float (&vx)[K], float (&vy)[K], float t
         float s2 = 0.0f;
 #pragma unroll
         for (int c = 0; c < K; ++c) s2 += vx[c] * vx[c] + vy[c] * vy[c];
-        const float r = rsq(s2), f = fmaxf(1.0f - (REG ? t * r : r), 0.0f);
+        const float f = factor(s2, t);
 #pragma unroll
         for (int c = 0; c < K; ++c) { vx[c] *= f; vy[c] *= f; }
     } else {
@@ -99,7 +104,6 @@ __device__ __forceinline__ void shrink_u(float (&vx)[K], float (&vy)[K], float t
         for (int c = 0; c < K; ++c) { vx[c] = dev::soft(vx[c], t); vy[c] = dev::soft(vy[c], t); }
     }
 }
-// (w is in units of nu, its threshold alpha may be of any size: the guarded factor)
 template <int L, int WN>
 __device__ __forceinline__ void shrink_w(float (&x)[L], float t)
 {
@@ -110,7 +114,7 @@ __device__ __forceinline__ void shrink_w(float (&x)[L], float t)
         float s2 = 0.0f;
 #pragma unroll
         for (int e = 0; e < L; ++e) s2 += x[e] * x[e];
-        const float f = dev::shrink2_factor(s2, t);
+        const float f = factor(s2, t);
 #pragma unroll
         for (int e = 0; e < L; ++e) x[e] *= f;
     }
@@ -192,7 +196,7 @@ struct Row {
 };
 
 // ------------------------------------------------------------------ S iterations
-template <int K, int UN, int WN, int S, bool REG>
+template <int K, int UN, int WN, int S, bool REG, bool RES>
 __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_constant__ MarchArgs a,
                                                                   const __grid_constant__ MarchOp g)
 {
@@ -211,8 +215,7 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_c
     const int ya = max(y0 - S, 0), yb = y1 + S;          // rows taken in: [ya, yb), zeros from n on
     const bool in = x >= 0 && x < n;
     const bool wr = in && lane >= S && lane < S + W;
-    const float ihx = x < n - 1 ? g.ih : 0.0f, mL = x > 0 ? 1.0f : 0.0f;
-    const float tu = REG ? g.su : 1.0f, tw = REG ? g.alpha * g.sw : g.alpha;
+    const float g1x = x < n - 1 ? g.g1 : 0.0f, mL = x > 0 ? 1.0f : 0.0f;
     const int xc = min(max(x, 0), n - 1), blk = (n + 31) >> 5;
     const float4 *pin = a.in + quad_at(n, NQ, ya, xc), *pb = a.b + quad_at(n, NB, ya, xc);
     const ptrdiff_t dy = (ptrdiff_t)blk * NQ * 32, dyb = (ptrdiff_t)blk * NB * 32;
@@ -267,17 +270,18 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_c
             // stage q + 1: row r = y - q - 1 from its values dq and the row above, cur
             Row<K> &dq = d[q];
             const int r = y - q - 1;
-            const float ihy = r < n - 1 ? g.ih : 0.0f, mD = r > 0 ? 1.0f : 0.0f;
+            const float g1y = r < n - 1 ? g.g1 : 0.0f, mD = r > 0 ? 1.0f : 0.0f;
             Row<K> o;
             float vx[K], vy[K], ubx[K], div[K];
 #pragma unroll
             for (int c = 0; c < K; ++c) {
                 const float right = __shfl_down_sync(0xffffffffu, dq.p[c], 1);
-                vx[c] = dq.x[c] + ihx * (right - dq.p[c]);
-                vy[c] = dq.y[c] + ihy * (cur.p[c] - dq.p[c]);
+                const float sx = g1x * (right - dq.p[c]), sy = g1y * (cur.p[c] - dq.p[c]);
+                vx[c] = RES ? fmaf(g.g2, sx, dq.x[c]) : __fadd_rn(dq.x[c], __fmul_rn(g.g2, sx));
+                vy[c] = RES ? fmaf(g.g2, sy, dq.y[c]) : __fadd_rn(dq.y[c], __fmul_rn(g.g2, sy));
                 if (REG) { vx[c] *= g.su; vy[c] *= g.su; }
             }
-            shrink_u<K, UN, REG>(vx, vy, tu);
+            shrink_u<K, UN>(vx, vy, g.tu);
 #pragma unroll
             for (int c = 0; c < K; ++c) {
                 ubx[c] = 2.0f * vx[c] - dq.x[c];
@@ -294,14 +298,18 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_c
 #pragma unroll
                 for (int hi = lo + 1; hi < K; ++hi) {
                     const int e = pair_at(K, lo, hi);
-                    wx[e] = dq.w[e] + g.inv[e] * (dq.p[lo] - dq.p[hi]);
+                    float ge = g.inv[e] * dq.p[lo];
+                    ge += -g.inv[e] * dq.p[hi];
+                    wx[e] = dq.w[e] + g.nu * ge;
                     if (REG) wx[e] *= g.sw;
                 }
-            if (K > 1) shrink_w<L, WN>(wx, tw);
+            if (K > 1) shrink_w<L, WN>(wx, g.tw);
+            float dx[K];
 #pragma unroll
             for (int c = 0; c < K; ++c) {
                 const float left = __shfl_up_sync(0xffffffffu, ubx[c], 1);
-                rr[c] = g.mu * (g.ih * ((ubx[c] - mL * left) + div[c])) + dq.b[c];
+                dx[c] = (ubx[c] - mL * left) + div[c];
+                rr[c] = RES ? 0.0f : g.ih * dx[c] + dq.b[c];
             }
 #pragma unroll
             for (int lo = 0; lo < K; ++lo)
@@ -309,11 +317,12 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_c
                 for (int hi = lo + 1; hi < K; ++hi) {
                     const int e = pair_at(K, lo, hi);
                     const float v = 2.0f * wx[e] - dq.w[e];
-                    rr[lo] -= g.nuinv[e] * v;
-                    rr[hi] += g.nuinv[e] * v;
+                    rr[lo] -= g.inv[e] * v;
+                    rr[hi] += g.inv[e] * v;
                 }
 #pragma unroll
             for (int c = 0; c < K; ++c) {
+                if (RES) rr[c] = g.ih * dx[c] + (rr[c] + dq.b[c]);
                 o.p[c] = dq.p[c] + g.tau * rr[c];
                 o.b[c] = dq.b[c];
             }
@@ -341,7 +350,7 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
     cudaGridDependencySynchronize();
     if (a.st->stop) return;
     const int lane = threadIdx.x & 31, n = g.n;
-    const float ih = g.ih, mu = g.mu, nu = g.nu, alpha = g.alpha;
+    const float ih = g.ih, alpha = g.alpha;
     dev::CheckAcc acc;
     acc.zero();
     for (int wi = blockIdx.x * WARPS + (threadIdx.x >> 5); wi < a.items; wi += gridDim.x * WARPS) {
@@ -358,8 +367,8 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
         p0.state_from(a.prv + quad_at(n, NQ, yl, xc));
 #pragma unroll
         for (int c = 0; c < K; ++c) {
-            un_[c] = y0 > 0 ? mu * c0.y[c] : 0.0f;
-            dn[c] = y0 > 0 ? mu * c0.y[c] - mu * p0.y[c] : 0.0f;
+            un_[c] = y0 > 0 ? c0.y[c] : 0.0f;
+            dn[c] = y0 > 0 ? c0.y[c] - p0.y[c] : 0.0f;
         }
         if (y0 > 0) {
             c0.state_from(a.cur + quad_at(n, NQ, y0, xc));
@@ -377,8 +386,8 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
             float q2 = 0.0f, dist = 0.0f;
 #pragma unroll
             for (int c = 0; c < K; ++c) {
-                const float uxc = mu * c0.x[c], uyc = mu * c0.y[c], bc = c0.b[c], ph = c0.p[c];
-                const float dux = uxc - mu * p0.x[c], duy = uyc - mu * p0.y[c];
+                const float uxc = c0.x[c], uyc = c0.y[c], bc = c0.b[c], ph = c0.p[c];
+                const float dux = uxc - p0.x[c], duy = uyc - p0.y[c];
                 uxs[c] = uxc;
                 uxl[c] = mL * __shfl_up_sync(0xffffffffu, uxc, 1);
                 const float dxl = mL * __shfl_up_sync(0xffffffffu, dux, 1);
@@ -421,7 +430,7 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
 #pragma unroll
                 for (int hi = lo + 1; hi < K; ++hi) {
                     const int e = pair_at(K, lo, hi);
-                    const float we = nu * c0.w[e], dwe = we - nu * p0.w[e], ge = g.inv[e] * (c0.p[lo] - c0.p[hi]);
+                    const float we = c0.w[e], dwe = we - p0.w[e], ge = g.inv[e] * (c0.p[lo] - c0.p[hi]);
                     fdw += dwe * dwe;
                     q2 += we * we;
                     gwb[lo] -= g.inv[e] * we;
@@ -478,14 +487,13 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
 }
 
 // ------------------------------------------------------------------ layouts
-// Planar fields <-> the engine's layout (u and w in units of mu and nu); b = rho1 - rho0.
+// Planar fields <-> the engine's layout; b = rho1 - rho0.
 template <int K>
 __global__ void k_march_in(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g, float4 *state,
                            float4 *bq)
 {
     const int n = g.n;
     const size_t nn = (size_t)n * n;
-    const float imu = 1.0f / g.mu, inu = 1.0f / g.nu;
     for (int y = blockIdx.y; y < n; y += gridDim.y) {
         const int x = blockIdx.x * blockDim.x + threadIdx.x;
         if (x >= n) continue;
@@ -497,14 +505,14 @@ __global__ void k_march_in(const __grid_constant__ PlanarArgs a, const __grid_co
             r.b[c] = a.rho1[c * nn + q] - a.rho0[c * nn + q];
             if (a.warm) {
                 r.p[c] = a.phi[c * nn + q];
-                r.x[c] = x < n - 1 ? imu * a.u[c * nn + q] : 0.0f;
-                r.y[c] = y < n - 1 ? imu * a.u[(K + c) * nn + q] : 0.0f;
+                r.x[c] = x < n - 1 ? a.u[c * nn + q] : 0.0f;
+                r.y[c] = y < n - 1 ? a.u[(K + c) * nn + q] : 0.0f;
             }
         }
         if (a.warm)
 #pragma unroll
             for (int e = 0; e < pairs(K); ++e)
-                if (g.edge[e] >= 0) r.w[e] = inu * a.w[g.edge[e] * nn + q];
+                if (g.edge[e] >= 0) r.w[e] = a.w[g.edge[e] * nn + q];
         r.state_to(state + quad_at(n, Quads<K>::NQ, y, x));
         float v[4 * Quads<K>::NB];
 #pragma unroll
@@ -532,23 +540,23 @@ __global__ void k_march_out(const __grid_constant__ PlanarArgs a, const __grid_c
 #pragma unroll
         for (int c = 0; c < K; ++c) {
             a.phi[c * nn + q] = r.p[c];
-            a.u[c * nn + q] = g.mu * r.x[c];
-            a.u[(K + c) * nn + q] = g.mu * r.y[c];
+            a.u[c * nn + q] = r.x[c];
+            a.u[(K + c) * nn + q] = r.y[c];
         }
 #pragma unroll
         for (int e = 0; e < pairs(K); ++e)
-            if (g.edge[e] >= 0) a.w[g.edge[e] * nn + q] = g.nu * r.w[e];
+            if (g.edge[e] >= 0) a.w[g.edge[e] * nn + q] = r.w[e];
     }
 }
 
 // ------------------------------------------------------------------ dispatch
-template <int K, int UN, int WN, bool REG>
+template <int K, int UN, int WN, bool REG, bool RES = false>
 Kernels kernels_of()
 {
     Kernels q = {};
-    q.step[0] = k_march<K, UN, WN, 1, REG>;
-    if constexpr (K <= 6) q.step[1] = k_march<K, UN, WN, 2, REG>;
-    if constexpr (K <= 3) q.step[2] = k_march<K, UN, WN, 4, REG>;
+    q.step[0] = k_march<K, UN, WN, 1, REG, RES>;
+    if constexpr (K <= 6) q.step[1] = k_march<K, UN, WN, 2, REG, RES>;
+    if constexpr (K <= 3) q.step[2] = k_march<K, UN, WN, 4, REG, RES>;
     q.check = k_march_check<K, UN, WN>;
     q.in = k_march_in<K>;
     q.out = k_march_out<K>;
@@ -561,9 +569,10 @@ Kernels kernels_of()
 // The plain problem with the default norms has its own kernels; every other one takes
 // those with the regularisation's factors (1 without it).
 template <int K>
-Kernels pick_norms(int un, int wn, bool reg)
+Kernels pick_norms(int un, int wn, bool reg, bool res)
 {
     if (K == 1) wn = VOMT_W_L1;           // no edges
+    if (res) return kernels_of<K, 0, 0, false, true>();      // default norms, eps = 0 only (run_engine)
     if (un == VOMT_U_L12 && wn == VOMT_W_L1) return reg ? kernels_of<K, 0, 0, true>() : kernels_of<K, 0, 0, false>();
     if constexpr (K > 1) {
         if (wn == VOMT_W_L2)

@@ -10,8 +10,10 @@ namespace march {
 struct MarchOp {
     int n, l, reg;
     float ih, mu, nu, tau, alpha;
+    float g1, g2;                     // the primal step takes g2 (g1 (difference)): (ih, mu) or (1, mu ih)
+    float tu, tw;                     // thresholds of the shrinks
     float eps, su, sw;
-    float inv[LVEC], nuinv[LVEC];     // 1 / c_e and nu / c_e (0: no edge)
+    float inv[LVEC];                  // 1 / c_e (0: no edge)
     int edge[LVEC];                   // the caller's edge number (-1: no edge)
 };
 
@@ -48,13 +50,13 @@ struct Kernels {
     int smem;                         // shared memory of a step
 };
 
-Kernels pick_k12(int k, int un, int wn, bool reg);
-Kernels pick_k3(int k, int un, int wn, bool reg);
-Kernels pick_k4(int k, int un, int wn, bool reg);
-Kernels pick_k5(int k, int un, int wn, bool reg);
-Kernels pick_k6(int k, int un, int wn, bool reg);
-Kernels pick_k7(int k, int un, int wn, bool reg);
-Kernels pick_k8(int k, int un, int wn, bool reg);
+Kernels pick_k12(int k, int un, int wn, bool reg, bool res);
+Kernels pick_k3(int k, int un, int wn, bool reg, bool res);
+Kernels pick_k4(int k, int un, int wn, bool reg, bool res);
+Kernels pick_k5(int k, int un, int wn, bool reg, bool res);
+Kernels pick_k6(int k, int un, int wn, bool reg, bool res);
+Kernels pick_k7(int k, int un, int wn, bool reg, bool res);
+Kernels pick_k8(int k, int un, int wn, bool reg, bool res);
 
 }  // namespace march
 

@@ -5,9 +5,9 @@
 namespace vomt {
 namespace march {
 
-Kernels pick_k12(int k, int un, int wn, bool reg)
+Kernels pick_k12(int k, int un, int wn, bool reg, bool res)
 {
-    return k == 1 ? pick_norms<1>(un, wn, reg) : pick_norms<2>(un, wn, reg);
+    return k == 1 ? pick_norms<1>(un, wn, reg, res) : pick_norms<2>(un, wn, reg, res);
 }
 
 }  // namespace march

@@ -5,7 +5,7 @@
 namespace vomt {
 namespace march {
 
-Kernels pick_k7(int, int un, int wn, bool reg) { return pick_norms<7>(un, wn, reg); }
+Kernels pick_k7(int, int un, int wn, bool reg, bool res) { return pick_norms<7>(un, wn, reg, res); }
 
 }  // namespace march
 }  // namespace vomt

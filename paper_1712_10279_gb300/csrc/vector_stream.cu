@@ -569,7 +569,7 @@ int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg
                  float *u, float *w, float *phi, cudaStream_t st)
 {
     bool taken = false;
-    const int mrc = march_solve(ctx, g, s, cfg, p, rho0, rho1, u, w, phi, st, &taken);
+    const int mrc = march_solve(ctx, g, s, cfg, p, false, rho0, rho1, u, w, phi, st, &taken);
     if (mrc || taken) return mrc;
     ctx->hist_raw = false;           // k_finalize writes finished rows
     const int n = s.n, k = g.k, l = g.l;
