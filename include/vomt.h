@@ -139,7 +139,9 @@ typedef struct {
     int blocks;          /* thread blocks of the main launch (resident: one tile each) */
     int halo;            /* resident engine: iterations between halo exchanges (0 otherwise) */
     int variant;         /* form of the main step kernel: 1 = inputs staged by TMA tiles,
-                            0 = per-thread loads (streaming and 3-D solves); for
+                            0 = per-thread loads (streaming and 3-D solves; 3-D
+                            grids with n not a multiple of 4 report 0 also where their padded
+                            rows are staged by tiles); for
                             vomt_solve_batched: 1 = the solve ran as one CUDA graph launch */
 } vomt_result;
 
@@ -195,7 +197,7 @@ int vomt_solve_host(vomt_ctx *ctx, int n, const float *rho0, const float *rho1,
  * {L1, L2}; p->eps must be 0; p->engine is ignored; p->halo > 0 sets the
  * number of z planes each thread block marches through (0: the library's
  * choice, about four blocks per SM).  result->variant tells whether the TMA
- * form of the step ran (n a multiple of 4, n >= 40, k <= 4).  Default mu
+ * form of the step ran on unpadded rows (n a multiple of 4, n >= 40, k <= 6).  Default mu
  * is 1/(48 tau (n-1)^2) (1/(24 tau (n-1)^2) without edges), since
  * ||grad||^2 <= 12 (n-1)^2 in 3-D; user mu, nu must satisfy
  * tau mu 12 (n-1)^2 + tau nu lambda_max(-Delta_G) < 1.  The history is that of

@@ -10,8 +10,8 @@
 // neighbours, so the step marches blocks up z: u' is computed once per point,
 // the x and y components meet their neighbours through shared memory and the z
 // component is carried to the next plane.  Two forms of that step: inputs staged
-// by TMA tiles (vector3d_tma.cu; n a multiple of 4, n >= 40, k <= 6) and, for
-// every other case, the form below with per-thread loads.  Step rule:
+// by TMA tiles (vector3d_tma.cu; n >= 40, k <= 6; rows padded to a multiple of
+// four floats) and, for every other case, the form below with per-thread loads.  Step rule:
 // ||grad||^2 <= 12 / h^2 in 3-D, so mu = 1/(48 tau (n-1)^2) (1/(24 tau (n-1)^2)
 // without edges) keeps the 2-D rule's share of the bound.
 #include <math.h>
@@ -245,18 +245,19 @@ __global__ void __launch_bounds__(MT, K <= 4 ? 2 : 1) k_step3m(S3In in, S3Out ou
 template <int K, int UN, int WN>
 __global__ void __launch_bounds__(T3) k_metrics3(S3In cur, S3In prv, const float *__restrict__ b, OpDev g,
                                                  StepDev s, double *__restrict__ partials,
-                                                 const DevStatus *__restrict__ st)
+                                                 const DevStatus *__restrict__ st, int np)
 {
     cudaGridDependencySynchronize();      // after the previous kernel (no-op for a normal launch)
     if (st->stop) return;
     constexpr int LK = LK3<K>::v;
     const int n = s.n;
-    const size_t m = (size_t)n * n * n;
+    const size_t points = (size_t)n * n * n, m = (size_t)n * n * np;
     CheckAcc acc;
     acc.zero();
-    for (size_t p = (size_t)blockIdx.x * T3 + threadIdx.x; p < m; p += (size_t)gridDim.x * T3) {
-        const int x = (int)(p % n), y = (int)((p / n) % n), z = (int)(p / ((size_t)n * n));
-        const long SX = 1, SY = n, SZ = (long)n * n;
+    for (size_t r = (size_t)blockIdx.x * T3 + threadIdx.x; r < points; r += (size_t)gridDim.x * T3) {
+        const int x = (int)(r % n), y = (int)((r / n) % n), z = (int)(r / ((size_t)n * n));
+        const size_t p = (r / n) * np + x;
+        const long SX = 1, SY = np, SZ = (long)n * np;
         const bool hx = x < n - 1, hy = y < n - 1, hz = z < n - 1, lx = x > 0, ly = y > 0, lz = z > 0;
         const float ih = s.ih, alpha = s.alpha;
         const double dih = (double)(n - 1);
@@ -367,40 +368,45 @@ __global__ void __launch_bounds__(T3) k_metrics3(S3In cur, S3In prv, const float
     block_sum_store<T3>(acc, partials + (size_t)blockIdx.x * NRED);
 }
 
-__global__ void k_prepare3(size_t m, int k, int l, const float *__restrict__ rho0, const float *__restrict__ rho1,
+// (rows of the volumes that the engine works on may be padded: np floats each)
+__global__ void k_prepare3(int n, int np, int k, int l, const float *__restrict__ rho0, const float *__restrict__ rho1,
                            float *__restrict__ b, int warm, const float *__restrict__ u_in,
                            const float *__restrict__ w_in, const float *__restrict__ phi_in, S3Out s0)
 {
+    const size_t m = (size_t)n * n * n, mp = (size_t)n * n * np;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < m; q += (size_t)gridDim.x * blockDim.x) {
+        const size_t o = q / n * np + q % n;
         for (int c = 0; c < k; ++c) {
-            b[c * m + q] = rho1[c * m + q] - rho0[c * m + q];
-            s0.phi[c * m + q] = warm ? phi_in[c * m + q] : 0.0f;
-            s0.ux[c * m + q] = warm ? u_in[c * m + q] : 0.0f;
-            s0.uy[c * m + q] = warm ? u_in[(k + c) * m + q] : 0.0f;
-            s0.uz[c * m + q] = warm ? u_in[(2 * k + c) * m + q] : 0.0f;
+            b[c * mp + o] = rho1[c * m + q] - rho0[c * m + q];
+            s0.phi[c * mp + o] = warm ? phi_in[c * m + q] : 0.0f;
+            s0.ux[c * mp + o] = warm ? u_in[c * m + q] : 0.0f;
+            s0.uy[c * mp + o] = warm ? u_in[(k + c) * m + q] : 0.0f;
+            s0.uz[c * mp + o] = warm ? u_in[(2 * k + c) * m + q] : 0.0f;
         }
-        for (int e = 0; e < l; ++e) s0.w[e * m + q] = warm ? w_in[e * m + q] : 0.0f;
+        for (int e = 0; e < l; ++e) s0.w[e * mp + o] = warm ? w_in[e * m + q] : 0.0f;
     }
 }
 
-__global__ void k_copy_out3(size_t m, int k, int l, S3In s0, S3In s1, const DevStatus *st, float *u, float *w,
+__global__ void k_copy_out3(int n, int np, int k, int l, S3In s0, S3In s1, const DevStatus *st, float *u, float *w,
                             float *phi)
 {
     const S3In &s = (st->iter & 1) ? s1 : s0;
+    const size_t m = (size_t)n * n * n, mp = (size_t)n * n * np;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < m; q += (size_t)gridDim.x * blockDim.x) {
+        const size_t o = q / n * np + q % n;
         for (int c = 0; c < k; ++c) {
-            phi[c * m + q] = s.phi[c * m + q];
-            u[c * m + q] = s.ux[c * m + q];
-            u[(k + c) * m + q] = s.uy[c * m + q];
-            u[(2 * k + c) * m + q] = s.uz[c * m + q];
+            phi[c * m + q] = s.phi[c * mp + o];
+            u[c * m + q] = s.ux[c * mp + o];
+            u[(k + c) * m + q] = s.uy[c * mp + o];
+            u[(2 * k + c) * m + q] = s.uz[c * mp + o];
         }
-        for (int e = 0; e < l; ++e) w[e * m + q] = s.w[e * m + q];
+        for (int e = 0; e < l; ++e) w[e * m + q] = s.w[e * mp + o];
     }
 }
 
 struct L3 {
     void (*step)(S3In, S3Out, const float *, OpDev, StepDev, const DevStatus *, int);
-    void (*metrics)(S3In, S3In, const float *, OpDev, StepDev, double *, const DevStatus *);
+    void (*metrics)(S3In, S3In, const float *, OpDev, StepDev, double *, const DevStatus *, int);
     size_t smem;
 };
 
@@ -451,14 +457,27 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
 {
     ctx->hist_raw = false;           // k_finalize writes finished rows
     const int k = g.k, l = g.l;
-    const size_t m = (size_t)n * n * n;
     cudaError_t e;
     int rc;
+    // inputs by TMA tiles where they apply (n >= 40, k <= 6).  The tiles want rows of a
+    // multiple of 16 bytes, so rows of other lengths are padded (3 x 3 tensors at 75^3:
+    // 120 us an iteration with per-thread loads)
+    bool tma = tma3_supported(n, k, l, p.u_norm, p.w_norm);
+    int np = tma ? (n + 3) / 4 * 4 : n;
     // workspace: b, then two states {phi, u_x, u_y, u_z, w}
-    const size_t per_state = (size_t)(4 * k + l) * m;
-    rc = ensure_buffer(ctx, (void **)&ctx->ws, &ctx->ws_floats, ((size_t)k * m + 2 * per_state) * sizeof(float),
-                       "workspace");
+    auto workspace = [&]() {
+        return ensure_buffer(ctx, (void **)&ctx->ws, &ctx->ws_floats,
+                             (size_t)(9 * k + 2 * l) * n * n * np * sizeof(float), "workspace");
+    };
+    rc = workspace();
+    if (rc && np != n) {              // no room for the padding
+        tma = false;
+        np = n;
+        rc = workspace();
+        if (!rc) ctx->err.clear();
+    }
     if (rc) return rc;
+    const size_t points = (size_t)n * n * n, m = (size_t)n * n * np, per_state = (size_t)(4 * k + l) * m;
     float *b = ctx->ws;
     S3Out so[2];
     S3In si[2];
@@ -468,7 +487,7 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
                       base + (size_t)4 * k * m};
         si[q] = S3In{so[q].phi, so[q].ux, so[q].uy, so[q].uz, so[q].w};
     }
-    const int nblocks = (int)((m + T3 - 1) / T3);
+    const int nblocks = (int)((points + T3 - 1) / T3);
     const int mblocks = nblocks < kMetricBlocks ? nblocks : kMetricBlocks;     // blocks of a check
     rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * (size_t)nblocks * NRED,
                        "partials");
@@ -477,17 +496,15 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     if (rc) return rc;
     e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "status reset");
-    const int pblocks = (int)std::min<size_t>((m + 255) / 256, 4096);
-    k_prepare3<<<pblocks, 256, 0, st>>>(m, k, l, rho0, rho1, b, p.warm_start, u, w, phi, so[0]);
+    const int pblocks = (int)std::min<size_t>((points + 255) / 256, 4096);
+    k_prepare3<<<pblocks, 256, 0, st>>>(n, np, k, l, rho0, rho1, b, p.warm_start, u, w, phi, so[0]);
     ctx->launches += 1;
     L3 L = pick3(k, p.u_norm, p.w_norm);
     e = cudaFuncSetAttribute((const void *)L.step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "3-D step shared memory");
-    // inputs by TMA tiles where they apply (n a multiple of 4, n >= 40, k <= 6)
-    Tma3Plan *tp = tma3_supported(n, k, l, p.u_norm, p.w_norm)
-                       ? tma3_plan_create(n, k, l, p.u_norm, p.w_norm, so[0].phi, so[1].phi, b)
-                       : nullptr;
-    ctx->last_variant = tp ? 1 : 0;
+    Tma3Plan *tp = tma ? tma3_plan_create(n, np, k, l, p.u_norm, p.w_norm, so[0].phi, so[1].phi, b) : nullptr;
+    if (!tp && np != n) return fail(ctx, VOMT_ERR_CUDA, "tensor maps of the padded volumes");
+    ctx->last_variant = tp && np == n ? 1 : 0;
     // z chunk: the longest of 32, 16, 8, 4 planes that still gives 1.5 blocks per SM
     // (TMA form; longer chunks amortise the pipeline fill, but fewer blocks than SMs
     // leave HBM idle; 32 measured best at 128^3 and 256^3) or four blocks per SM
@@ -502,7 +519,7 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     ctx->last_blocks = (int)(mgrid.x * mgrid.y * mgrid.z);
     auto check = [&](int t, int cur) {
         launch_pdl(L.metrics, dim3(mblocks), dim3(T3), 0, st, si[cur], si[cur ^ 1], (const float *)b, g, s,
-                   ctx->partials, (const DevStatus *)ctx->dstatus);
+                   ctx->partials, (const DevStatus *)ctx->dstatus, np);
         launch_pdl(k_finalize, dim3(1), dim3(kFinThreads), 0, st, (const double *)ctx->partials, mblocks, cfg, t,
                    ctx->dstatus, ctx->dhist, ctx->hist_cap, 0);
         ctx->launches += 2;
@@ -539,7 +556,7 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
             ++nchunk;
         }
     }
-    k_copy_out3<<<pblocks, 256, 0, st>>>(m, k, l, si[0], si[1], ctx->dstatus, u, w, phi);
+    k_copy_out3<<<pblocks, 256, 0, st>>>(n, np, k, l, si[0], si[1], ctx->dstatus, u, w, phi);
     ctx->launches += 1;
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&ctx->hstatus[0], ctx->dstatus, sizeof(DevStatus),

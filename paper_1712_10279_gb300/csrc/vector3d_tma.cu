@@ -15,9 +15,9 @@
 // shared memory, the z component is carried in a register to the next plane
 // (the chunk's first plane recomputes it from global memory).
 //
-// TMA rules honoured here: the tensors are 4-D (x, y, z, volume) with strides
-// 4n, 4n^2, 4n^3 bytes, so n must be a multiple of 4; every box starts at an x
-// that is a multiple of 4; loads may start at negative or out-of-range
+// TMA rules honoured here: the tensors are 4-D (x, y, z, volume) with rows of np
+// floats, np >= n a multiple of 4 (strides 4 np, 4 np n, 4 np n^2 bytes); every box
+// starts at an x that is a multiple of 4; loads may start at negative or out-of-range
 // coordinates and then read zeros, which the stencil masks anyway.  Every wait
 // on an mbarrier is bounded: one that runs out marks the solve failed, the
 // block drains its copies in flight (again bounded) and returns.
@@ -126,7 +126,8 @@ __device__ __forceinline__ bool wait_phase(uint32_t mb, uint32_t parity, uint32_
 
 template <int K, int UN, int WN>
 __global__ void __launch_bounds__(NT3, blocks_per_sm(K)) k_step3t(const __grid_constant__ Maps3 maps, const float *__restrict__ in,
-                                                 S3Out out, OpDev g, StepDev s, DevStatus *st, int zc)
+                                                 S3Out out, OpDev g, StepDev s, DevStatus *st, int zc,
+                                                 int np)
 {
     constexpr int NS = nstages(K), LK = LK3<K>::v;
     constexpr int PL = BYP * BXH, UL = BYU * BXU, WL = MY * MX;
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(NT3, blocks_per_sm(K)) k_step3t(const __grid_c
     const int n = s.n, l = g.l;
     const Stage3 SL = stage3(K, l);
     float *const sb0 = (float *)(smem + NS * SL.size);
-    const size_t m = (size_t)n * n * n, nn = (size_t)n * n;
+    const size_t m = (size_t)n * n * np, nn = (size_t)n * np;      // a volume, a plane (rows of np floats)
     const int tid = threadIdx.x, tx = tid % MX, ty = tid / MX;
     const bool tile = tid < MT;                 // else a halo thread: ht < MX row, < MX + MY column
     const int ht = tid - MT;
@@ -186,12 +187,12 @@ __global__ void __launch_bounds__(NT3, blocks_per_sm(K)) k_step3t(const __grid_c
 #pragma unroll
     for (int c = 0; c < K; ++c) cz[c] = 0.0f;
     if (z0 > 0 && inb) {
-        const size_t p = (size_t)(z0 - 1) * nn + (size_t)y * n + x;
+        const size_t p = (size_t)(z0 - 1) * nn + (size_t)y * np + x;
         float ax[K], ay[K], az[K], az0[K];
 #pragma unroll
         for (int c = 0; c < K; ++c) {
             const float *P = in + c * m + p;
-            const float pc = __ldg(P), px = hx ? __ldg(P + 1) : 0.0f, py = hy ? __ldg(P + n) : 0.0f;
+            const float pc = __ldg(P), px = hx ? __ldg(P + 1) : 0.0f, py = hy ? __ldg(P + np) : 0.0f;
             const float pz = __ldg(P + nn);
             az0[c] = __ldg(in + (3 * K + c) * m + p);
             ax[c] = upre(__ldg(in + (K + c) * m + p), px, pc, hx, mi);
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(NT3, blocks_per_sm(K)) k_step3t(const __grid_c
             for (int c = 0; c < K; ++c) r[c] -= g.Dv[c][e] * v;
         }
         if (inb) {
-            const size_t p = (size_t)z * nn + (size_t)y * n + x;
+            const size_t p = (size_t)z * nn + (size_t)y * np + x;
 #pragma unroll
             for (int c = 0; c < K; ++c) {
                 const size_t q = c * m + p;
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(NT3, blocks_per_sm(K)) k_step3t(const __grid_c
     }
 }
 
-using Kern3 = void (*)(const Maps3, const float *, S3Out, OpDev, StepDev, DevStatus *, int);
+using Kern3 = void (*)(const Maps3, const float *, S3Out, OpDev, StepDev, DevStatus *, int, int);
 
 template <int K>
 Kern3 pick_norms3t(int un, int wn)
@@ -388,14 +389,15 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn3()
     return fn;
 }
 
-// 4-D map (x, y, z, volume) over `vols` n^3 volumes at base; box bx x by x 1 x bv
-bool encode4(CUtensorMap *map, const float *base, int n, int vols, int bx, int by, int bv)
+// 4-D map (x, y, z, volume) over `vols` n^3 volumes at base, rows np floats apart; box
+// bx x by x 1 x bv
+bool encode4(CUtensorMap *map, const float *base, int n, int np, int vols, int bx, int by, int bv)
 {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn3();
     if (!fn) return false;
-    const cuuint64_t nn = (cuuint64_t)n;
+    const cuuint64_t nn = (cuuint64_t)n, row = (cuuint64_t)np * 4;
     const cuuint64_t dims[4] = {nn, nn, nn, (cuuint64_t)vols};
-    const cuuint64_t strides[3] = {nn * 4, nn * nn * 4, nn * nn * nn * 4};
+    const cuuint64_t strides[3] = {row, nn * row, nn * nn * row};
     const cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, 1, (cuuint32_t)bv};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (void *)base, dims, strides, box, estr,
@@ -409,19 +411,19 @@ struct Tma3Plan {
     Maps3 maps[2];       // reading state 0 / state 1
     const float *in[2];
     Kern3 kern;
-    int smem;
+    int smem, np;
 };
 
 bool tma3_supported(int n, int k, int l, int un, int wn)
 {
-    if (n < BXH || n % 4 != 0 || n > 1024) return false;
+    if (n < BXH || n > 1024) return false;
     if (!pick3t(k, un, wn)) return false;
     // the ring fits blocks_per_sm blocks of one SM's 228 KB (1 KB reserved per block)
     if (smem3(k, l) > (k <= 4 ? 110 : 224) * 1024) return false;
     return encode_fn3() != nullptr;
 }
 
-Tma3Plan *tma3_plan_create(int n, int k, int l, int un, int wn, const float *state0, const float *state1,
+Tma3Plan *tma3_plan_create(int n, int np, int k, int l, int un, int wn, const float *state0, const float *state1,
                            const float *b)
 {
     Tma3Plan *pl = new Tma3Plan();
@@ -430,14 +432,15 @@ Tma3Plan *tma3_plan_create(int n, int k, int l, int un, int wn, const float *sta
     bool ok = true;
     for (int q = 0; q < 2 && ok; ++q) {
         pl->in[q] = st[q];
-        ok = encode4(&pl->maps[q].phi, st[q], n, vols, BXH, BYP, k) &&
-             encode4(&pl->maps[q].u, st[q], n, vols, BXU, BYU, k) &&
-             (l == 0 || encode4(&pl->maps[q].w, st[q], n, vols, MX, MY, l)) &&
-             encode4(&pl->maps[q].b, b, n, k, MX, MY, k);
+        ok = encode4(&pl->maps[q].phi, st[q], n, np, vols, BXH, BYP, k) &&
+             encode4(&pl->maps[q].u, st[q], n, np, vols, BXU, BYU, k) &&
+             (l == 0 || encode4(&pl->maps[q].w, st[q], n, np, vols, MX, MY, l)) &&
+             encode4(&pl->maps[q].b, b, n, np, k, MX, MY, k);
         if (l == 0) memset(&pl->maps[q].w, 0, sizeof(CUtensorMap));
     }
     pl->kern = pick3t(k, un, wn);
     pl->smem = smem3(k, l);
+    pl->np = np;
     if (ok && pl->kern)
         ok = cudaFuncSetAttribute((const void *)pl->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->smem) ==
              cudaSuccess;
@@ -455,7 +458,7 @@ void tma3_launch_step(const Tma3Plan *pl, int in_state, S3Out out, const OpDev &
 {
     const int n = s.n;
     const dim3 grd((n + MX - 1) / MX, (n + MY - 1) / MY, (n + zc - 1) / zc);
-    launch_pdl(pl->kern, grd, dim3(NT3), pl->smem, stream, pl->maps[in_state], pl->in[in_state], out, g, s, st, zc);
+    launch_pdl(pl->kern, grd, dim3(NT3), pl->smem, stream, pl->maps[in_state], pl->in[in_state], out, g, s, st, zc, pl->np);
 }
 
 }  // namespace vomt
