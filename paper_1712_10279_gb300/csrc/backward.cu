@@ -21,14 +21,18 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "internal.h"
+#include "march2d.h"
+#include "pdhg_device.cuh"
 
 namespace vomt {
 namespace {
 
 constexpr int AX = 32, AY = 8, AT = AX * AY;
+constexpr size_t kKeepBytes = (size_t)1 << 30;      // most memory for keeping every iterate of an unrolled solve
 
 __global__ void __launch_bounds__(1024) k_envelope(int n, int pitch, int k, int l, int wn, const float *__restrict__ phi,
                                                    const float *__restrict__ w, const float *__restrict__ gscale,
@@ -150,113 +154,140 @@ __global__ void __launch_bounds__(AT) k_adj_init(int n, int l, int wn, float alp
 // write the adjoint of s^t (A0), add tau * (adjoint of phi^{t+1}) to grho (the
 // derivative with respect to rho1; rho0 gets its negative) and add this block's
 // contribution to dJ/dalpha to apart[blk].  ||u||_{1,2} (per channel shrink_2).
+//
+// A warp marches up `rows` rows of a strip of 30 columns, one column per lane: the shrink's
+// adjoint is formed once per point, its x component reaches the right neighbour by a
+// shuffle and its y component the row above in a register, and every value is read once.
+// Bound by the latency of a launch at the sizes that are unrolled in practice (256^2, three
+// channels: 27 planes, 7 MB, all in L2), so launches overlap (launch_pdl).
 template <int K>
-__global__ void __launch_bounds__(AT) k_adj_step(OpDev g, StepDev s, int wn, const float *__restrict__ S,
-                                                 const float *__restrict__ A1, float *__restrict__ A0,
-                                                 float *__restrict__ grho, double *__restrict__ apart)
+__global__ void __launch_bounds__(AT) k_adj_step(const __grid_constant__ march::MarchOp g, int wn,
+                                                 const float *__restrict__ S, const float *__restrict__ A1,
+                                                 float *__restrict__ A0, float *__restrict__ grho,
+                                                 double *__restrict__ apart, int rows, int strips, int warps)
 {
+    cudaGridDependencySynchronize();      // after the previous kernel (no-op for a normal launch)
     constexpr int LK = ALK<K>::v;
-    const int n = s.n, l = g.l;
-    const int i = blockIdx.x * AX + threadIdx.x, j = blockIdx.y * AY + threadIdx.y;
-    double ga = 0.0;
-    if (i < n && j < n) {
-        const size_t nn = (size_t)n * n, p = (size_t)j * n + i;
-        const bool hR = i < n - 1, hU = j < n - 1, hL = i > 0, hD = j > 0;
-        const float mu = s.mu, nu = s.nu, tau = s.tau, ih = s.ih, muih = mu * ih;
+    const int n = g.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int wi = blockIdx.x * (AT / 32) + wid;
+    float ga = 0.0f, gl = 0.0f;           // this thread's share of dJ/dalpha, a pair kept by TwoSum
+    if (wi < warps) {
+        const int i = (wi % strips) * 30 - 1 + lane, y0 = (wi / strips) * rows, y1 = min(n, y0 + rows);
+        const bool in = i >= 0 && i < n, own = in && lane >= 1 && lane < 31;
+        const bool hR = i < n - 1, hL = i > 0;
+        const size_t nn = (size_t)n * n;
+        const float mu = g.mu, nu = g.nu, tau = g.tau, ih = g.ih, muih = mu * ih;
         const float *phi = S, *ux = S + (size_t)K * nn, *uy = S + (size_t)2 * K * nn, *w = S + (size_t)3 * K * nn;
-        const float *Gp = A1, *Gx = A1 + (size_t)K * nn, *Gy = A1 + (size_t)2 * K * nn, *Gw = A1 + (size_t)3 * K * nn;
-        float qc[K], dvg[K];
+        const float *Gx = A1 + (size_t)K * nn, *Gy = A1 + (size_t)2 * K * nn, *Gw = A1 + (size_t)3 * K * nn;
+        const int jb = y0 > 0 ? y0 - 1 : 0;
+        float pc[K], qc[K], gd[K];        // phi and its adjoint in the row, the y component of the row below
 #pragma unroll
         for (int c = 0; c < K; ++c) {
-            const size_t o = c * nn + p;
-            const float pc = phi[o], pr = hR ? phi[o + 1] : 0.0f, pu = hU ? phi[o + n] : 0.0f;
-            const float pl = hL ? phi[o - 1] : 0.0f, plu = (hL && hU) ? phi[o - 1 + n] : 0.0f;
-            const float pd = hD ? phi[o - n] : 0.0f, prd = (hR && hD) ? phi[o + 1 - n] : 0.0f;
-            qc[c] = Gp[o];
-            const float qr = hR ? Gp[o + 1] : 0.0f, qu = hU ? Gp[o + n] : 0.0f;
-            const float ql = hL ? Gp[o - 1] : 0.0f, qlu = (hL && hU) ? Gp[o - 1 + n] : 0.0f;
-            const float qd = hD ? Gp[o - n] : 0.0f, qrd = (hR && hD) ? Gp[o + 1 - n] : 0.0f;
-            // at p
-            const float ax = hR ? ih * (qr - qc[c]) : 0.0f, ay = hU ? ih * (qu - qc[c]) : 0.0f;
-            const float vx = ux[o] + (hR ? muih * (pr - pc) : 0.0f), vy = uy[o] + (hU ? muih * (pu - pc) : 0.0f);
-            float gvx, gvy;
-            vjp_shrink2(vx, vy, mu, Gx[o] - 2.0f * tau * ax, Gy[o] - 2.0f * tau * ay, gvx, gvy);
-            A0[(K + c) * nn + p] = gvx + tau * ax;
-            A0[(2 * K + c) * nn + p] = gvy + tau * ay;
-            // x component of the same quantity at (i-1, j)
-            float glx = 0.0f;
-            if (hL) {
-                const float lax = ih * (qc[c] - ql), lay = hU ? ih * (qlu - ql) : 0.0f;
-                const float lvx = ux[o - 1] + muih * (pc - pl), lvy = uy[o - 1] + (hU ? muih * (plu - pl) : 0.0f);
-                float t_;
-                vjp_shrink2(lvx, lvy, mu, Gx[o - 1] - 2.0f * tau * lax, Gy[o - 1] - 2.0f * tau * lay, glx, t_);
-            }
-            // y component at (i, j-1)
-            float gdy = 0.0f;
-            if (hD) {
-                const float dax = hR ? ih * (qrd - qd) : 0.0f, day = ih * (qc[c] - qd);
-                const float dvx = ux[o - n] + (hR ? muih * (prd - pd) : 0.0f), dvy = uy[o - n] + muih * (pc - pd);
-                float t_;
-                vjp_shrink2(dvx, dvy, mu, Gx[o - n] - 2.0f * tau * dax, Gy[o - n] - 2.0f * tau * day, t_, gdy);
-            }
-            dvg[c] = ih * ((gvx - glx) + (gvy - gdy));      // div of the shrink adjoint at p
+            const size_t o = c * nn + (size_t)jb * n + i;
+            pc[c] = in ? phi[o] : 0.0f;
+            qc[c] = in ? A1[o] : 0.0f;
+            gd[c] = 0.0f;
         }
-        // graph part at p
-        float xw[LK], hw[LK], gxw[LK];
-#pragma unroll
-        for (int e = 0; e < LK; ++e) {
-            float ge = 0.0f, dq = 0.0f;
+        for (int j = jb; j < y1; ++j) {
+            const bool hU = j < n - 1, hD = j > 0, wr = own && j >= y0;
+            const size_t p = (size_t)j * n + i;
+            float pu[K], qu[K], dvg[K];
 #pragma unroll
             for (int c = 0; c < K; ++c) {
-                ge += g.G[e][c] * phi[c * nn + p];
-                dq += g.Dv[c][e] * qc[c];
-            }
-            xw[e] = (e < l) ? w[e * nn + p] + nu * ge : 0.0f;
-            hw[e] = (e < l) ? Gw[e * nn + p] - 2.0f * tau * dq : 0.0f;
-            gxw[e] = 0.0f;
-            if (e < l) A0[(3 * K + e) * nn + p] = tau * dq;
-        }
-        const float th = s.alpha * nu;
-        if (wn == VOMT_W_L1) {
-#pragma unroll
-            for (int e = 0; e < LK; ++e)
-                if (e < l && fabsf(xw[e]) > th) {
-                    gxw[e] = hw[e];
-                    ga += -(double)nu * (xw[e] > 0.0f ? 1.0 : -1.0) * (double)hw[e];
+                const size_t o = c * nn + p;
+                pu[c] = in && hU ? phi[o + n] : 0.0f;
+                qu[c] = in && hU ? A1[o + n] : 0.0f;
+                const float pr = __shfl_down_sync(0xffffffffu, pc[c], 1), qr = __shfl_down_sync(0xffffffffu, qc[c], 1);
+                const float x0 = in ? ux[o] : 0.0f, yy0 = in ? uy[o] : 0.0f;
+                const float hx = in ? Gx[o] : 0.0f, hy = in ? Gy[o] : 0.0f;
+                const float ax = hR ? ih * (qr - qc[c]) : 0.0f, ay = hU ? ih * (qu[c] - qc[c]) : 0.0f;
+                const float vx = x0 + (hR ? muih * (pr - pc[c]) : 0.0f);
+                const float vy = yy0 + (hU ? muih * (pu[c] - pc[c]) : 0.0f);
+                float gvx, gvy;
+                vjp_shrink2(vx, vy, mu, hx - 2.0f * tau * ax, hy - 2.0f * tau * ay, gvx, gvy);
+                const float left = __shfl_up_sync(0xffffffffu, gvx, 1), glx = hL ? left : 0.0f;
+                dvg[c] = ih * ((gvx - glx) + (gvy - (hD ? gd[c] : 0.0f)));      // div of the shrink adjoint
+                gd[c] = gvy;
+                if (wr) {
+                    A0[(K + c) * nn + p] = gvx + tau * ax;
+                    A0[(2 * K + c) * nn + p] = gvy + tau * ay;
                 }
-        } else {
-            float s2 = 0.0f, xh = 0.0f;
+            }
+            if (wr) {
+                // graph part
+                float xw[LK], hw[LK], dq[LK], gxw[LK];
+                const float th = g.alpha * nu;
+                float s2 = 0.0f, xh = 0.0f;
 #pragma unroll
-            for (int e = 0; e < LK; ++e) { s2 += xw[e] * xw[e]; xh += xw[e] * hw[e]; }
-            if (s2 > th * th) {
-                const float r = rsqrtf(s2);
-                const float a = 1.0f - th * r, c3 = th * xh * r * r * r;
+                for (int lo = 0; lo < K; ++lo)
 #pragma unroll
-                for (int e = 0; e < LK; ++e) gxw[e] = a * hw[e] + c3 * xw[e];
-                ga += -(double)nu * (double)(xh * r);
+                    for (int hi = lo + 1; hi < K; ++hi) {
+                        const int e = lo * (2 * K - lo - 1) / 2 + hi - lo - 1, ed = g.edge[e];
+                        dq[e] = g.inv[e] * (qc[lo] - qc[hi]);
+                        xw[e] = ed >= 0 ? w[ed * nn + p] + nu * (g.inv[e] * (pc[lo] - pc[hi])) : 0.0f;
+                        hw[e] = ed >= 0 ? Gw[ed * nn + p] - 2.0f * tau * dq[e] : 0.0f;
+                        gxw[e] = 0.0f;
+                        s2 += xw[e] * xw[e];
+                        xh += xw[e] * hw[e];
+                    }
+                float da = 0.0f;
+                if (wn == VOMT_W_L1) {
+#pragma unroll
+                    for (int e = 0; e < K * (K - 1) / 2; ++e)
+                        if (fabsf(xw[e]) > th) {
+                            gxw[e] = hw[e];
+                            da -= nu * (xw[e] > 0.0f ? hw[e] : -hw[e]);
+                        }
+                } else if (s2 > th * th) {
+                    const float r = rsqrtf(s2), a = 1.0f - th * r, c3 = th * xh * r * r * r;
+#pragma unroll
+                    for (int e = 0; e < K * (K - 1) / 2; ++e) gxw[e] = a * hw[e] + c3 * xw[e];
+                    da = -nu * (xh * r);
+                }
+                float err;
+                ga = dev::two_sum(ga, da, err);
+                gl += err;
+                float gg[K];
+#pragma unroll
+                for (int c = 0; c < K; ++c) gg[c] = 0.0f;
+#pragma unroll
+                for (int lo = 0; lo < K; ++lo)
+#pragma unroll
+                    for (int hi = lo + 1; hi < K; ++hi) {
+                        const int e = lo * (2 * K - lo - 1) / 2 + hi - lo - 1, ed = g.edge[e];
+                        if (ed >= 0) A0[(3 * K + ed) * nn + p] = tau * dq[e] + gxw[e];
+                        gg[lo] += g.inv[e] * gxw[e];
+                        gg[hi] -= g.inv[e] * gxw[e];
+                    }
+#pragma unroll
+                for (int c = 0; c < K; ++c) {
+                    A0[c * nn + p] = qc[c] - mu * dvg[c] + nu * gg[c];
+                    grho[c * nn + p] += tau * qc[c];
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
+                pc[c] = pu[c];
+                qc[c] = qu[c];
             }
         }
-#pragma unroll
-        for (int e = 0; e < LK; ++e)
-            if (e < l) A0[(3 * K + e) * nn + p] += gxw[e];
-#pragma unroll
-        for (int c = 0; c < K; ++c) {
-            float gg = 0.0f;
-#pragma unroll
-            for (int e = 0; e < LK; ++e) gg += g.G[e][c] * gxw[e];
-            A0[c * nn + p] = qc[c] - mu * dvg[c] + nu * gg;
-            grho[c * nn + p] += tau * qc[c];
-        }
     }
-    __shared__ double sh[AT];
-    const int t = threadIdx.y * AX + threadIdx.x;
-    sh[t] = ga;
+    // the block's sum: pairs over a warp, FP64 over the warps
+    __shared__ double sh[AT / 32];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const float oh = __shfl_down_sync(0xffffffffu, ga, off), ol = __shfl_down_sync(0xffffffffu, gl, off);
+        float err;
+        ga = dev::two_sum(ga, oh, err);
+        gl += ol + err;
+    }
+    if (lane == 0) sh[wid] = (double)ga + (double)gl;
     __syncthreads();
-    for (int off = AT / 2; off > 0; off >>= 1) {
-        if (t < off) sh[t] += sh[t + off];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int q = 0; q < AT / 32; ++q) t += sh[q];
+        apart[blockIdx.x] += t;
     }
-    if (t == 0) apart[blockIdx.y * gridDim.x + blockIdx.x] += sh[0];
 }
 
 __global__ void k_sub(size_t cnt, const float *__restrict__ r0, const float *__restrict__ r1, float *__restrict__ b)
@@ -275,7 +306,8 @@ __global__ void k_finish_grad(size_t cnt, float scale, const float *__restrict__
 }
 
 using AdjInit = void (*)(int, int, int, float, const float *, float *, double *);
-using AdjStep = void (*)(OpDev, StepDev, int, const float *, const float *, float *, float *, double *);
+using AdjStep = void (*)(const march::MarchOp, int, const float *, const float *, float *, float *, double *, int, int,
+                         int);
 
 template <int K>
 void pick_adj_k(AdjInit *ai, AdjStep *as)
@@ -346,32 +378,50 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         rc = check_vector_densities(ctx, op.k, n, rho0, rho1, st);
         if (rc) return rc;
         const int K = op.k, l = op.l;
+        march::MarchOp mop;
+        if (!march_op(op, s, &mop)) return fail(ctx, VOMT_ERR_BAD_ARG, "unrolled gradient: not a channel graph");
         const size_t nn = (size_t)n * n, SZ = (size_t)(3 * K + l) * nn;
+        // Every iterate is kept where that takes at most kKeepBytes: nothing is computed twice
+        // then (256^2, three channels, 200 iterations: 0.6 GB and 190 launches fewer).  Beyond, or
+        // where the memory is not to be had, checkpoints every `ckpt` iterations.
+        bool keep = ((size_t)T + 1) * SZ * sizeof(float) <= kKeepBytes;
         const int nck = T / ckpt + 1;
-        const size_t floats = (size_t)2 * K * nn + ((size_t)nck + ckpt + 1 + 2) * SZ;
-        rc = ensure_buffer(ctx, (void **)&ctx->gbuf, &ctx->gbuf_bytes, floats * sizeof(float), "gradient scratch");
+        auto floats = [&]() {
+            return (size_t)2 * K * nn + 2 * SZ + (keep ? (size_t)T + 1 : (size_t)nck + ckpt + 1) * SZ;
+        };
+        rc = ensure_buffer(ctx, (void **)&ctx->gbuf, &ctx->gbuf_bytes, floats() * sizeof(float), "gradient scratch");
+        if (rc && keep) {
+            keep = false;
+            rc = ensure_buffer(ctx, (void **)&ctx->gbuf, &ctx->gbuf_bytes, floats() * sizeof(float), "gradient scratch");
+            if (!rc) ctx->err.clear();
+        }
         if (rc) return rc;
         const dim3 blk(AX, AY), grd((n + AX - 1) / AX, (n + AY - 1) / AY);
         const int nb = (int)(grd.x * grd.y);
-        rc = ensure_buffer(ctx, (void **)&ctx->gpart, &ctx->gpart_bytes, sizeof(double) * 3 * (size_t)nb, "gradient sums");
+        // reverse steps: chunks of rows that give every scheduler a warp or two
+        const int strips = (n + 29) / 30;
+        const int rows = std::max(2, (int)(((long)strips * n + 8 * ctx->sm_count - 1) / (8 * ctx->sm_count)));
+        const int warps = strips * ((n + rows - 1) / rows), rb = (warps + AT / 32 - 1) / (AT / 32);
+        rc = ensure_buffer(ctx, (void **)&ctx->gpart, &ctx->gpart_bytes, sizeof(double) * (2 * (size_t)nb + rb), "gradient sums");
         if (rc) return rc;
         float *b = ctx->gbuf, *grho = b + (size_t)K * nn;
-        float *ck = grho + (size_t)K * nn;                  // nck checkpoints
+        float *adj = grho + (size_t)K * nn;                 // 2 adjoint states
+        float *ck = adj + 2 * SZ;                           // the iterates kept (all, or nck checkpoints)
         float *seg = ck + (size_t)nck * SZ;                 // ckpt + 1 recompute slots
-        float *adj = seg + (size_t)(ckpt + 1) * SZ;         // 2 adjoint states
         double *part = ctx->gpart, *apart = part + 2 * (size_t)nb;
         const int pb = (int)(((size_t)K * nn + 255) / 256 < 2048 ? ((size_t)K * nn + 255) / 256 : 2048);
         e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(ck, 0, SZ * sizeof(float), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(grho, 0, (size_t)K * nn * sizeof(float), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(apart, 0, sizeof(double) * nb, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(apart, 0, sizeof(double) * rb, st);
         if (e != cudaSuccess) return set_cuda_error(ctx, e, "gradient reset");
         k_sub<<<pb, 256, 0, st>>>((size_t)K * nn, rho0, rho1, b);
         ++ctx->launches;
-        // forward, keeping every ckpt-th iterate
+        // forward, keeping every iterate or every ckpt-th
         const float *cur = ck;
         for (int t = 1; t <= T; ++t) {
-            float *out = (t % ckpt == 0) ? ck + (size_t)(t / ckpt) * SZ : seg + (size_t)(t & 1) * SZ;
+            float *out = keep ? ck + (size_t)t * SZ
+                              : (t % ckpt == 0 ? ck + (size_t)(t / ckpt) * SZ : seg + (size_t)(t & 1) * SZ);
             launch_step(op, s, p.u_norm, p.w_norm, cur, out, b, ctx->dstatus, st);
             ++ctx->launches;
             cur = out;
@@ -381,27 +431,31 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         pick_adj(K, &ai, &as);
         ai<<<grd, blk, 0, st>>>(n, l, p.w_norm, s.alpha, cur, adj, part);
         ++ctx->launches;
-        // reverse, one checkpoint segment at a time
         int a_in = 0;
-        for (int sg = (T - 1) / ckpt; sg >= 0; --sg) {
-            const int t0 = sg * ckpt, t1 = (t0 + ckpt < T) ? t0 + ckpt : T;
-            const float *base = ck + (size_t)sg * SZ;
-            for (int m = 1; m < t1 - t0; ++m) {
-                const float *in = (m == 1) ? base : seg + (size_t)(m - 1) * SZ;
-                launch_step(op, s, p.u_norm, p.w_norm, in, seg + (size_t)m * SZ, b, ctx->dstatus, st);
-                ++ctx->launches;
-            }
-            for (int t = t1 - 1; t >= t0; --t) {
-                const float *St = (t == t0) ? base : seg + (size_t)(t - t0) * SZ;
-                as<<<grd, blk, 0, st>>>(op, s, p.w_norm, St, adj + (size_t)a_in * SZ, adj + (size_t)(1 - a_in) * SZ,
-                                        grho, apart);
-                ++ctx->launches;
-                a_in = 1 - a_in;
+        auto reverse = [&](const float *St) {
+            launch_pdl(as, dim3(rb), dim3(AT), 0, st, mop, p.w_norm, St, (const float *)(adj + (size_t)a_in * SZ),
+                       adj + (size_t)(1 - a_in) * SZ, grho, apart, rows, strips, warps);
+            ++ctx->launches;
+            a_in = 1 - a_in;
+        };
+        if (keep) {
+            for (int t = T - 1; t >= 0; --t) reverse(ck + (size_t)t * SZ);
+        } else {
+            // one checkpoint segment at a time
+            for (int sg = (T - 1) / ckpt; sg >= 0; --sg) {
+                const int t0 = sg * ckpt, t1 = (t0 + ckpt < T) ? t0 + ckpt : T;
+                const float *base = ck + (size_t)sg * SZ;
+                for (int m = 1; m < t1 - t0; ++m) {
+                    const float *in = (m == 1) ? base : seg + (size_t)(m - 1) * SZ;
+                    launch_step(op, s, p.u_norm, p.w_norm, in, seg + (size_t)m * SZ, b, ctx->dstatus, st);
+                    ++ctx->launches;
+                }
+                for (int t = t1 - 1; t >= t0; --t) reverse(t == t0 ? base : seg + (size_t)(t - t0) * SZ);
             }
         }
         k_finish_grad<<<pb, 256, 0, st>>>((size_t)K * nn, (float)scale, grho, d_rho0, d_rho1);
         ++ctx->launches;
-        std::vector<double> hp((size_t)3 * nb);
+        std::vector<double> hp((size_t)2 * nb + rb);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(hp.data(), part, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -410,8 +464,8 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         for (int q = 0; q < nb; ++q) {
             jv += hp[2 * q];
             ws += hp[2 * q + 1];
-            ga += hp[2 * nb + q];
         }
+        for (int q = 0; q < rb; ++q) ga += hp[2 * (size_t)nb + q];
         if (J) *J = jv;
         if (d_alpha) *d_alpha = scale * (ws + ga);
         if (!isfinite(jv)) return fail(ctx, VOMT_ERR_NONFINITE, "unrolled objective is not finite");

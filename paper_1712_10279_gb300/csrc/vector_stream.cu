@@ -535,7 +535,7 @@ void launch_step(const OpDev &g, const StepDev &s, int un, int wn, const float *
     const StateIn si{in, in + (size_t)k * nn, in + (size_t)2 * k * nn, in + (size_t)3 * k * nn};
     const StateOut so{out, out + (size_t)k * nn, out + (size_t)2 * k * nn, out + (size_t)3 * k * nn};
     const dim3 blk(BX, BY), grd((s.n + BX - 1) / BX, (s.n + BY - 1) / BY);
-    pick(k, un, wn).step<<<grd, blk, 0, stream>>>(si, so, b, g, s, st);
+    launch_pdl(pick(k, un, wn).step, grd, blk, 0, stream, si, so, b, g, s, st);
 }
 
 int validate_densities(vomt_ctx *ctx, int planes, int n, const float *rho0, const float *rho1,
