@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pdhg_device.cuh"
 
 namespace vomt {
 namespace {
@@ -43,46 +44,68 @@ PairTable make_pairs(int k)
     return t;
 }
 
-// per block: sum tr Lam0, sum tr Lam1, min diagonal entry, max |X_ab - X_ba|,
-// max |X_ab|, count of non-finite entries
-__global__ void k_mat_validate(size_t nn, int k, const float *__restrict__ L0, const float *__restrict__ L1,
-                               double *__restrict__ out)
+// What a block of 256 threads has seen of matrix densities: sum tr Lam0, sum tr Lam1 (FP32
+// pairs per thread and warp, FP64 where those overflow), min diagonal entry, max asymmetry, max |X_ab|, count of
+// non-finite entries.
+template <typename Sum>
+struct MatrixCheck {
+    Sum t[2];
+    float mind = INFINITY, asym = 0.0f, mabs = 0.0f;
+    int bad = 0;
+    __device__ __forceinline__ void store(double *out)
+    {
+        __shared__ double sh[8][6];
+        t[0].warp();
+        t[1].warp();
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            mind = fminf(mind, __shfl_down_sync(0xffffffffu, mind, off));
+            asym = fmaxf(asym, __shfl_down_sync(0xffffffffu, asym, off));
+            mabs = fmaxf(mabs, __shfl_down_sync(0xffffffffu, mabs, off));
+            bad += __shfl_down_sync(0xffffffffu, bad, off);
+        }
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        if (lane == 0) {
+            sh[wid][0] = t[0].value();
+            sh[wid][1] = t[1].value();
+            sh[wid][2] = mind;
+            sh[wid][3] = asym;
+            sh[wid][4] = mabs;
+            sh[wid][5] = bad;
+        }
+        __syncthreads();
+        const int q = threadIdx.x;
+        if (q < 6) {
+            double v = sh[0][q];
+            for (int w = 1; w < 8; ++w) v = q == 2 ? fmin(v, sh[w][q]) : (q == 3 || q == 4 ? fmax(v, sh[w][q]) : v + sh[w][q]);
+            out[q] = v;
+        }
+    }
+};
+
+template <typename Sum>
+__global__ void __launch_bounds__(256) k_mat_validate(size_t nn, int k, const float *__restrict__ L0,
+                                                      const float *__restrict__ L1, double *__restrict__ out)
 {
-    double t0 = 0.0, t1 = 0.0, mind = 1e300, asym = 0.0, mabs = 0.0, bad = 0.0;
+    MatrixCheck<Sum> m;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < nn; q += (size_t)gridDim.x * blockDim.x) {
         for (int side = 0; side < 2; ++side) {
             const float *X = side ? L1 : L0;
             for (int a = 0; a < k; ++a)
                 for (int b = 0; b < k; ++b) {
                     const float v = X[(a * k + b) * nn + q];
-                    if (!isfinite(v)) { bad += 1.0; continue; }
-                    mabs = fmax(mabs, (double)fabsf(v));
+                    if (!(fabsf(v) < INFINITY)) { ++m.bad; continue; }
+                    m.mabs = fmaxf(m.mabs, fabsf(v));
                     if (a == b) {
-                        if (side) t1 += v; else t0 += v;
-                        mind = fmin(mind, (double)v);
+                        m.t[side].add(v);
+                        m.mind = fminf(m.mind, v);
                     } else if (a < b) {
-                        asym = fmax(asym, (double)fabsf(v - X[(b * k + a) * nn + q]));
+                        m.asym = fmaxf(m.asym, fabsf(v - X[(b * k + a) * nn + q]));
                     }
                 }
         }
     }
-    __shared__ double sh[6][256];
-    sh[0][threadIdx.x] = t0; sh[1][threadIdx.x] = t1; sh[2][threadIdx.x] = mind;
-    sh[3][threadIdx.x] = asym; sh[4][threadIdx.x] = mabs; sh[5][threadIdx.x] = bad;
-    __syncthreads();
-    for (int off = 128; off > 0; off >>= 1) {
-        if (threadIdx.x < off) {
-            const int o = threadIdx.x + off;
-            sh[0][threadIdx.x] += sh[0][o];
-            sh[1][threadIdx.x] += sh[1][o];
-            sh[2][threadIdx.x] = fmin(sh[2][threadIdx.x], sh[2][o]);
-            sh[3][threadIdx.x] = fmax(sh[3][threadIdx.x], sh[3][o]);
-            sh[4][threadIdx.x] = fmax(sh[4][threadIdx.x], sh[4][o]);
-            sh[5][threadIdx.x] += sh[5][o];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 6) out[blockIdx.x * 6 + threadIdx.x] = sh[threadIdx.x][0];
+    m.store(out + (size_t)blockIdx.x * 6);
 }
 
 // full symmetric planes -> compact channels (the symmetric part), `groups` fields
@@ -150,49 +173,34 @@ double default_tau_matrix(int n) { return n <= 64 ? 10.0 : (n <= 128 ? 30.0 : 60
 // coordinates of hermitian_to_op (diagonal; Re, Im above it), padded to K
 // channels with zeros.  `full` holds `groups` fields of [re: k*k planes][im: k*k planes].
 
-// per block: sum Re tr Lam0, sum Re tr Lam1, min Re diagonal, max |X_ab - conj X_ba|
-// (and |Im X_aa|), max |X|, count of non-finite entries
-__global__ void k_herm_validate(size_t nn, int k, const float *__restrict__ L0, const float *__restrict__ L1,
-                                double *__restrict__ out)
+// the same for Hermitian fields: traces and diagonal of the real part, max |X_ab - conj X_ba|
+// and |Im X_aa|
+template <typename Sum>
+__global__ void __launch_bounds__(256) k_herm_validate(size_t nn, int k, const float *__restrict__ L0,
+                                                       const float *__restrict__ L1, double *__restrict__ out)
 {
     const int kk = k * k;
-    double t0 = 0.0, t1 = 0.0, mind = 1e300, asym = 0.0, mabs = 0.0, bad = 0.0;
+    MatrixCheck<Sum> m;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < nn; q += (size_t)gridDim.x * blockDim.x) {
         for (int side = 0; side < 2; ++side) {
             const float *re = side ? L1 : L0, *im = re + (size_t)kk * nn;
             for (int a = 0; a < k; ++a)
                 for (int b = 0; b < k; ++b) {
                     const float xr = re[(a * k + b) * nn + q], xi = im[(a * k + b) * nn + q];
-                    if (!isfinite(xr) || !isfinite(xi)) { bad += 1.0; continue; }
-                    mabs = fmax(mabs, (double)fmaxf(fabsf(xr), fabsf(xi)));
+                    if (!(fabsf(xr) < INFINITY) || !(fabsf(xi) < INFINITY)) { ++m.bad; continue; }
+                    m.mabs = fmaxf(m.mabs, fmaxf(fabsf(xr), fabsf(xi)));
                     if (a == b) {
-                        if (side) t1 += xr; else t0 += xr;
-                        mind = fmin(mind, (double)xr);
-                        asym = fmax(asym, (double)fabsf(xi));
+                        m.t[side].add(xr);
+                        m.mind = fminf(m.mind, xr);
+                        m.asym = fmaxf(m.asym, fabsf(xi));
                     } else if (a < b) {
                         const float yr = re[(b * k + a) * nn + q], yi = im[(b * k + a) * nn + q];
-                        asym = fmax(asym, (double)fmaxf(fabsf(xr - yr), fabsf(xi + yi)));
+                        m.asym = fmaxf(m.asym, fmaxf(fabsf(xr - yr), fabsf(xi + yi)));
                     }
                 }
         }
     }
-    __shared__ double sh[6][256];
-    sh[0][threadIdx.x] = t0; sh[1][threadIdx.x] = t1; sh[2][threadIdx.x] = mind;
-    sh[3][threadIdx.x] = asym; sh[4][threadIdx.x] = mabs; sh[5][threadIdx.x] = bad;
-    __syncthreads();
-    for (int off = 128; off > 0; off >>= 1) {
-        if (threadIdx.x < off) {
-            const int o = threadIdx.x + off;
-            sh[0][threadIdx.x] += sh[0][o];
-            sh[1][threadIdx.x] += sh[1][o];
-            sh[2][threadIdx.x] = fmin(sh[2][threadIdx.x], sh[2][o]);
-            sh[3][threadIdx.x] = fmax(sh[3][threadIdx.x], sh[3][o]);
-            sh[4][threadIdx.x] = fmax(sh[4][threadIdx.x], sh[4][o]);
-            sh[5][threadIdx.x] += sh[5][o];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 6) out[blockIdx.x * 6 + threadIdx.x] = sh[threadIdx.x][0];
+    m.store(out + (size_t)blockIdx.x * 6);
 }
 
 // Hermitian part of full complex fields -> compact channels
@@ -395,20 +403,28 @@ static int momt_any(int dim, vomt_ctx *ctx, int n, int k, const float *Lam0, con
         const int vb = (int)((nn + 255) / 256 < 512 ? (nn + 255) / 256 : 512);
         rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * 6 * (size_t)vb, "partials");
         if (rc) return rc;
-        k_mat_validate<<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
-        ++ctx->launches;
         std::vector<double> hv((size_t)vb * 6);
-        e = cudaMemcpyAsync(hv.data(), ctx->partials, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return set_cuda_error(ctx, e, "matrix validate");
         double tr0 = 0.0, tr1 = 0.0, mind = 1e300, asym = 0.0, mabs = 0.0, bad = 0.0;
-        for (int q = 0; q < vb; ++q) {
-            tr0 += hv[q * 6 + 0];
-            tr1 += hv[q * 6 + 1];
-            mind = fmin(mind, hv[q * 6 + 2]);
-            asym = fmax(asym, hv[q * 6 + 3]);
-            mabs = fmax(mabs, hv[q * 6 + 4]);
-            bad += hv[q * 6 + 5];
+        for (int wide = 0; wide < 2; ++wide) {
+            if (wide)
+                k_mat_validate<dev::WideSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
+            else
+                k_mat_validate<dev::PairSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
+            ++ctx->launches;
+            e = cudaMemcpyAsync(hv.data(), ctx->partials, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return set_cuda_error(ctx, e, "matrix validate");
+            tr0 = tr1 = asym = mabs = bad = 0.0;
+            mind = 1e300;
+            for (int q = 0; q < vb; ++q) {
+                tr0 += hv[q * 6 + 0];
+                tr1 += hv[q * 6 + 1];
+                mind = fmin(mind, hv[q * 6 + 2]);
+                asym = fmax(asym, hv[q * 6 + 3]);
+                mabs = fmax(mabs, hv[q * 6 + 4]);
+                bad += hv[q * 6 + 5];
+            }
+            if (isfinite(tr0) && isfinite(tr1)) break;
         }
         if (bad > 0.0) return fail(ctx, VOMT_ERR_NONFINITE, "density has NaN or Inf entries");
         if (mind < 0.0) return fail(ctx, VOMT_ERR_NEGATIVE_DENSITY, "density has a negative diagonal entry");
@@ -526,20 +542,28 @@ extern "C" int momt_solve_complex(vomt_ctx *ctx, int n, int k, const float *Lam0
         const int vb = (int)((nn + 255) / 256 < 512 ? (nn + 255) / 256 : 512);
         rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * 6 * (size_t)vb, "partials");
         if (rc) return rc;
-        k_herm_validate<<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
-        ++ctx->launches;
         std::vector<double> hv((size_t)vb * 6);
-        e = cudaMemcpyAsync(hv.data(), ctx->partials, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return set_cuda_error(ctx, e, "complex validate");
         double tr0 = 0.0, tr1 = 0.0, mind = 1e300, asym = 0.0, mabs = 0.0, bad = 0.0;
-        for (int q = 0; q < vb; ++q) {
-            tr0 += hv[q * 6 + 0];
-            tr1 += hv[q * 6 + 1];
-            mind = fmin(mind, hv[q * 6 + 2]);
-            asym = fmax(asym, hv[q * 6 + 3]);
-            mabs = fmax(mabs, hv[q * 6 + 4]);
-            bad += hv[q * 6 + 5];
+        for (int wide = 0; wide < 2; ++wide) {
+            if (wide)
+                k_herm_validate<dev::WideSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
+            else
+                k_herm_validate<dev::PairSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
+            ++ctx->launches;
+            e = cudaMemcpyAsync(hv.data(), ctx->partials, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return set_cuda_error(ctx, e, "complex validate");
+            tr0 = tr1 = asym = mabs = bad = 0.0;
+            mind = 1e300;
+            for (int q = 0; q < vb; ++q) {
+                tr0 += hv[q * 6 + 0];
+                tr1 += hv[q * 6 + 1];
+                mind = fmin(mind, hv[q * 6 + 2]);
+                asym = fmax(asym, hv[q * 6 + 3]);
+                mabs = fmax(mabs, hv[q * 6 + 4]);
+                bad += hv[q * 6 + 5];
+            }
+            if (isfinite(tr0) && isfinite(tr1)) break;
         }
         if (bad > 0.0) return fail(ctx, VOMT_ERR_NONFINITE, "density has NaN or Inf entries");
         if (mind < 0.0) return fail(ctx, VOMT_ERR_NEGATIVE_DENSITY, "density has a negative diagonal entry");

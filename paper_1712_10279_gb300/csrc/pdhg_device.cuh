@@ -170,6 +170,94 @@ __device__ __forceinline__ float residual_c(float ih, float ux, float xl, float 
     return r + (e4 + (pe + ih * ((e1 + e2) + e3)));
 }
 
+// A running sum kept as a pair of FP32 numbers by TwoSum (about twice FP32 precision).  FP64
+// additions run at a sixty-fourth of the FP32 rate on this GPU, so a pass that adds every
+// value it reads in FP64 is bound by them.
+struct PairSum {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x)
+    {
+        float e;
+        hi = two_sum(hi, x, e);
+        lo += e;
+    }
+    __device__ __forceinline__ void merge(float oh, float ol)
+    {
+        float e;
+        hi = two_sum(hi, oh, e);
+        lo += ol + e;
+    }
+    __device__ __forceinline__ void warp()          // lane 0 ends with the warp's sum
+    {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+            merge(__shfl_down_sync(0xffffffffu, hi, off), __shfl_down_sync(0xffffffffu, lo, off));
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// The same in FP64, for sums beyond FP32's range.
+struct WideSum {
+    double v = 0.0;
+    __device__ __forceinline__ void add(float x) { v += x; }
+    __device__ __forceinline__ void warp()
+    {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    }
+    __device__ __forceinline__ double value() const { return v; }
+};
+
+// Input checks of densities: what a block of 256 threads has seen, stored as five FP64
+// values (sum rho0, sum rho1, min rho0, min rho1, count of non-finite entries).  Where a sum
+// of pairs comes back non-finite, the caller runs the check again with WideSum.
+template <typename Sum>
+struct DensityCheck {
+    Sum s0, s1;
+    float m0 = INFINITY, m1 = INFINITY;
+    int bad = 0;
+    __device__ __forceinline__ void add(float a, float c)
+    {
+        if (!(fabsf(a) < INFINITY) || !(fabsf(c) < INFINITY)) {
+            ++bad;
+            return;
+        }
+        s0.add(a);
+        s1.add(c);
+        m0 = fminf(m0, a);
+        m1 = fminf(m1, c);
+    }
+    __device__ __forceinline__ void store(double *out)
+    {
+        __shared__ double sh[8][5];
+        s0.warp();
+        s1.warp();
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            m0 = fminf(m0, __shfl_down_sync(0xffffffffu, m0, off));
+            m1 = fminf(m1, __shfl_down_sync(0xffffffffu, m1, off));
+            bad += __shfl_down_sync(0xffffffffu, bad, off);
+        }
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        if (lane == 0) {
+            sh[wid][0] = s0.value();
+            sh[wid][1] = s1.value();
+            sh[wid][2] = m0;
+            sh[wid][3] = m1;
+            sh[wid][4] = bad;
+        }
+        __syncthreads();
+        if (threadIdx.x < 5) {
+            double t = sh[0][threadIdx.x];
+            for (int w = 1; w < 8; ++w) {
+                const double x = sh[w][threadIdx.x];
+                t = threadIdx.x == 2 || threadIdx.x == 3 ? fmin(t, x) : t + x;
+            }
+            out[threadIdx.x] = t;
+        }
+    }
+};
+
 // One thread's share of a convergence check: each sum slot is a pair of FP32
 // numbers (hi, lo) that TwoSum keeps equal to the exact running sum up to the
 // rounding of lo (about twice FP32 precision); the maximum slot is a plain FP32
