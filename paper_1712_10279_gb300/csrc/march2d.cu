@@ -3,6 +3,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "march2d.h"
 
@@ -28,11 +29,22 @@ bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out)
             else if (hi < 0) hi = c;
             else return false;
         }
+        if (lo < 0) continue;                     // 1 / cost is 0 in FP32: any free pair, below
         if (hi < 0 || g.we[e] != 1.0f || !(g.G[e][lo] > 0.0f) || g.G[e][hi] != -g.G[e][lo]) return false;
         const int q = lo * (2 * g.k - lo - 1) / 2 + hi - lo - 1;
         if (m.edge[q] >= 0) return false;
         m.edge[q] = e;
         m.inv[q] = g.G[e][lo];
+    }
+    for (int e = 0; e < g.l; ++e) {
+        bool set = false;
+        for (int q = 0; q < LVEC; ++q) set = set || m.edge[q] == e;
+        for (int q = 0; !set && q < g.k * (g.k - 1) / 2; ++q)
+            if (m.edge[q] < 0) {
+                m.edge[q] = e;
+                set = true;
+            }
+        if (!set) return false;
     }
     m.n = s.n;
     m.l = g.l;
@@ -50,6 +62,17 @@ bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out)
     m.su = s.reg ? s.su : 1.0f;
     m.sw = s.reg ? s.sw : 1.0f;
     *out = m;
+    return true;
+}
+
+bool edges_in_order(const march::MarchOp &m)
+{
+    int last = -1;
+    for (int q = 0; q < LVEC; ++q)
+        if (m.edge[q] >= 0) {
+            if (m.edge[q] < last) return false;
+            last = m.edge[q];
+        }
     return true;
 }
 
@@ -124,7 +147,7 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
 {
     *taken = false;
     MarchOp op;
-    if (p.u_norm > VOMT_U_L1 || p.w_norm > VOMT_W_L2 || !march_op(g, s, &op)) return VOMT_OK;
+    if (p.u_norm > VOMT_U_L1 || p.w_norm > VOMT_W_L2 || !march_op(g, s, &op) || !edges_in_order(op)) return VOMT_OK;
     const int n = s.n, k = g.k;
     const int interval = std::min(p.check_every, std::max(p.max_iters, 0));
     if (k <= 4 && interval < 4) return VOMT_OK;
@@ -269,6 +292,291 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
     for (int q = 0; q < 2; ++q)
         if (ev[q]) cudaEventDestroy(ev[q]);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "solve");
+    return VOMT_OK;
+}
+
+// ------------------------------------------------------------------ batches
+__global__ void k_finalize_many(const march::BatchItem *__restrict__ items, int nblocks, int t, int slot);
+
+void march_scratch_free(BatchMarchScratch *s)
+{
+    cudaFree(s->items);
+    cudaFree(s->maps);
+    cudaFree(s->data);
+    cudaFree(s->stat);
+    if (s->hstat) cudaFreeHost(s->hstat);
+    *s = BatchMarchScratch();
+}
+
+namespace {
+
+constexpr int kCheckBlocks = 8;       // blocks of a problem's check
+
+// The problems of one channel count: passes over all of them at once, with chunks of the
+// same number of rows in every problem.
+struct Group {
+    int k = 0, main_pass = 0;
+    std::vector<int> probs;
+    Kernels K;
+    Pass pass[3];                     // blocks: of the whole group
+};
+
+// plan_pass for a group: the chunk length of the least arithmetic time
+Pass plan_group(const std::vector<BatchProblem> &probs, const Group &gr, int S, int blocks_per_sm, int sms)
+{
+    const int k = gr.k, W = 32 - 2 * S;
+    const double issue = 20.0 + 40.0 * k + 4.0 * k * (k - 1), lat = 180.0, ghz = 1.95;
+    const long cap = (long)blocks_per_sm * sms;
+    int top = 0;
+    double pts = 0.0;
+    for (int q : gr.probs) {
+        top = std::max(top, probs[q].g.n);
+        pts += (double)probs[q].g.n * probs[q].g.n;
+    }
+    Pass best;
+    for (int rows = 1; rows <= top; rows += rows < 32 ? 1 : rows / 16) {
+        long blocks = 0, warps = 0;
+        for (int q : gr.probs) {
+            const int n = probs[q].g.n;
+            const long w = (long)((n + W - 1) / W) * ((n + rows - 1) / rows);
+            warps += w;
+            blocks += (w + kWarps - 1) / kWarps;
+        }
+        if (blocks > (1l << 30)) continue;
+        const long full = blocks / cap, rest = blocks % cap;
+        double cycles = (double)full * std::max(lat, issue * blocks_per_sm);
+        if (rest) cycles += std::max(lat, issue * ceil((double)rest / sms));
+        const double us = cycles * S * (rows + 2 * S) / (ghz * 1e3);
+        if (best.stages == 0 || us < best.us) best = Pass{S, rows, 0, (int)warps, (int)blocks, us};
+    }
+    const double mb = 16e-6 * pts * (2 * gr.K.groups + (k + 3) / 4);
+    best.us = 3.5 + std::max(best.us, mb / (mb > 110.0 ? 6.3 : 12.0));
+    return best;
+}
+
+int plan_groups(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p, std::vector<Group> *out)
+{
+    out->clear();
+    const int interval = std::max(1, std::min(p.check_every, p.max_iters));
+    for (int k = 1; k <= 5; ++k) {
+        Group g;
+        g.k = k;
+        for (int q = 0; q < (int)probs.size(); ++q)
+            if (probs[q].k == k) g.probs.push_back(q);
+        if (g.probs.empty()) continue;
+        g.K = pick(k, VOMT_U_L12, VOMT_W_L1, false, true);
+        for (int q = 0; q < 3; ++q) {
+            if (!g.K.many[q]) continue;
+            int per_sm = 0;
+            cudaError_t e = cudaFuncSetAttribute((const void *)g.K.many[q], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 kSmemBlock);
+            if (e == cudaSuccess)
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)g.K.many[q], 32 * kWarps,
+                                                                  g.K.smem);
+            if (e != cudaSuccess) return set_cuda_error(ctx, e, "marching kernel");
+            if (per_sm < 1) continue;
+            Pass &ps = g.pass[q];
+            ps = plan_group(probs, g, kStages[q], per_sm, ctx->sm_count);
+            const int share = (ps.blocks + ctx->sm_count - 1) / ctx->sm_count;      // see march_solve
+            ps.smem = std::max(g.K.smem, kSmemSM / (share + 1));
+            if (kStages[q] <= interval && (g.pass[g.main_pass].stages == 0 ||
+                                           ps.us / kStages[q] < g.pass[g.main_pass].us / kStages[g.main_pass]))
+                g.main_pass = q;
+        }
+        if (g.pass[0].stages == 0) return VOMT_ERR_TOO_LARGE;
+        out->push_back(g);
+    }
+    return VOMT_OK;
+}
+
+}  // namespace
+
+double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p)
+{
+    std::vector<Group> groups;
+    if (plan_groups(ctx, probs, p, &groups)) return 1e30;
+    double us = 0.0;
+    for (const Group &g : groups) us += g.pass[g.main_pass].us / kStages[g.main_pass];
+    return us;
+}
+
+// The problems of a channel count advance together, a pass over all of them per launch; a
+// problem that has stopped costs its blocks a look at its status.  Eight pairs at 256^2
+// with three channels take about 5 us per iteration together, where one after another on
+// every SM (the grouped resident form) they take 8 x 1.6.
+int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
+                cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)
+{
+    *taken = false;
+    const int count = (int)probs.size();
+    if (count > 65535) return VOMT_OK;                // a launch's third dimension
+    std::vector<Group> groups;
+    int rc = plan_groups(ctx, probs, p, &groups);
+    if (rc) return rc == VOMT_ERR_TOO_LARGE ? VOMT_OK : rc;
+    // scratch: per problem b, two states, the state before a check; check sums; tables
+    std::vector<BatchItem> items(count);
+    std::vector<int> maps, slot_of(count);            // items are stored group by group
+    size_t floats4 = 0;
+    std::vector<size_t> off(count);
+    for (const Group &g : groups)
+        for (int q : g.probs) {
+            const size_t tile = (size_t)probs[q].g.n * ((probs[q].g.n + 31) / 32) * 32;
+            off[q] = floats4;
+            floats4 += tile * (3 * (size_t)g.K.groups + g.K.bgroups);
+        }
+    const size_t sums = sizeof(double) * NRED * kCheckBlocks * (size_t)count;
+    rc = ensure_buffer(ctx, &scr->data, &scr->data_cap, sizeof(float4) * floats4 + sums, "batch states");
+    if (rc) {
+        ctx->err.clear();
+        return VOMT_OK;
+    }
+    rc = ensure_buffer(ctx, &scr->items, &scr->items_cap, sizeof(BatchItem) * count, "batch tables");
+    if (!rc) rc = ensure_buffer(ctx, &scr->stat, &scr->stat_cap, sizeof(DevStatus) * count, "batch status");
+    if (rc) return rc;
+    if (scr->hstat_cap < 2 * sizeof(DevStatus) * count) {
+        if (scr->hstat) cudaFreeHost(scr->hstat);
+        scr->hstat = nullptr;
+        scr->hstat_cap = 0;
+        cudaError_t e = cudaMallocHost(&scr->hstat, 2 * sizeof(DevStatus) * count);
+        if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch status");
+        scr->hstat_cap = 2 * sizeof(DevStatus) * count;
+    }
+    float4 *data = (float4 *)scr->data;
+    double *dsums = (double *)(data + floats4);
+    DevStatus *dstat = (DevStatus *)scr->stat, *hstat = (DevStatus *)scr->hstat;
+    blocks->assign(count, 1);
+    int at = 0;
+    std::vector<size_t> map_at(groups.size() * 3, 0);
+    std::vector<int> first_item(groups.size()), top(groups.size(), 0);
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+        const Group &g = groups[gi];
+        first_item[gi] = at;
+        int next[3] = {0, 0, 0};
+        std::vector<int> gm[3];
+        for (size_t i = 0; i < g.probs.size(); ++i, ++at) {
+            const int q = g.probs[i], n = probs[q].g.n;
+            const size_t tile = (size_t)n * ((n + 31) / 32) * 32;
+            BatchItem &d = items[at];
+            memset(&d, 0, sizeof d);
+            d.g = probs[q].g;
+            d.g.g1 = 1.0f;
+            d.g.g2 = d.g.mu * d.g.ih;
+            d.cfg = probs[q].cfg;
+            d.planar = probs[q].planar;
+            d.b = data + off[q];
+            for (int c = 0; c < 3; ++c) d.S[c] = d.b + tile * (g.K.bgroups + (size_t)c * g.K.groups);
+            d.st = dstat + at;
+            d.partials = dsums + (size_t)at * NRED * kCheckBlocks;
+            for (int c = 0; c < 3; ++c) {
+                if (!g.pass[c].stages) continue;
+                const int W = 32 - 2 * kStages[c];
+                d.pass[c].rows = std::min(g.pass[c].rows, n);
+                d.pass[c].strips = (n + W - 1) / W;
+                d.pass[c].warps = d.pass[c].strips * ((n + d.pass[c].rows - 1) / d.pass[c].rows);
+                d.pass[c].first = next[c];
+                const int nb = (d.pass[c].warps + kWarps - 1) / kWarps;
+                gm[c].insert(gm[c].end(), nb, (int)i);
+                next[c] += nb;
+                if (c == g.main_pass) (*blocks)[q] = nb;
+            }
+            d.check_strips = (n + 29) / 30;
+            d.check_rows = std::max(2, (d.check_strips * n + kCheckBlocks * kWarps - 1) / (kCheckBlocks * kWarps));
+            d.check_items = d.check_strips * ((n + d.check_rows - 1) / d.check_rows);
+            slot_of[q] = at;
+            top[gi] = std::max(top[gi], n);
+        }
+        for (int c = 0; c < 3; ++c) {
+            map_at[gi * 3 + c] = maps.size();
+            maps.insert(maps.end(), gm[c].begin(), gm[c].end());
+            groups[gi].pass[c].blocks = next[c];
+        }
+    }
+    rc = ensure_buffer(ctx, &scr->maps, &scr->maps_cap, sizeof(int) * maps.size(), "batch tables");
+    if (rc) return rc;
+    cudaError_t e = cudaMemcpyAsync(scr->items, items.data(), sizeof(BatchItem) * count, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scr->maps, maps.data(), sizeof(int) * maps.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(dstat, 0, sizeof(DevStatus) * count, st);
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch tables");
+    *taken = true;
+    const BatchItem *ditems = (const BatchItem *)scr->items;
+    const int *dmaps = (const int *)scr->maps;
+    auto layout_grid = [&](size_t gi) {
+        return dim3((top[gi] + 127) / 128, std::min(top[gi], 256), (unsigned)groups[gi].probs.size());
+    };
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+        groups[gi].K.in_many<<<layout_grid(gi), 128, 0, st>>>(ditems + first_item[gi]);
+        ctx->launches += 1;
+    }
+    std::vector<int> cur(groups.size(), 0), before(groups.size(), 0);
+    auto one = [&](size_t gi, int q, bool last) {
+        const Group &g = groups[gi];
+        const int prev = last && kStages[q] > 1 ? 1 : 0;
+        launch_pdl(g.K.many[q], dim3(g.pass[q].blocks), dim3(32 * kWarps), (size_t)g.pass[q].smem, st,
+                   ditems + first_item[gi], dmaps + map_at[gi * 3 + q], cur[gi], prev);
+        ctx->launches += 1;
+        before[gi] = prev ? 2 : cur[gi];
+        cur[gi] ^= 1;
+    };
+    auto advance = [&](size_t gi, int m) {        // m iterations, fewer-stage passes first
+        const Group &g = groups[gi];
+        const int q = g.main_pass;
+        int odd = m % kStages[q];
+        for (int r = q - 1; r >= 0; --r)
+            for (; g.pass[r].stages && odd >= kStages[r]; odd -= kStages[r], m -= kStages[r]) one(gi, r, m == kStages[r]);
+        for (; m > 0; m -= kStages[q]) one(gi, q, m == kStages[q]);
+    };
+    auto check = [&](size_t gi, int t) {
+        const Group &g = groups[gi];
+        const unsigned np = (unsigned)g.probs.size();
+        launch_pdl(g.K.check_many, dim3(kCheckBlocks, np), dim3(32 * kWarps), 0, st, ditems + first_item[gi], cur[gi],
+                   before[gi]);
+        launch_pdl(k_finalize_many, dim3(np), dim3(kFinThreads), 0, st, ditems + first_item[gi], kCheckBlocks, t, cur[gi]);
+        ctx->launches += 2;
+    };
+    if (p.max_iters == 0)
+        for (size_t gi = 0; gi < groups.size(); ++gi) check(gi, 0);
+    const bool tol_mode = p.tol_gap > 0.0;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    if (tol_mode)
+        for (int q = 0; q < 2; ++q) cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming);
+    const int chunk = p.check_every * ((2048 + p.check_every - 1) / p.check_every);
+    int t = 0, nchunk = 0;
+    bool stopped = false;
+    while (t < p.max_iters && !stopped) {
+        const int end = p.max_iters - t > chunk ? t + chunk : p.max_iters;
+        while (t < end) {
+            const int m = std::min(p.check_every, p.max_iters - t);
+            t += m;
+            for (size_t gi = 0; gi < groups.size(); ++gi) {
+                advance(gi, m);
+                check(gi, t);
+            }
+        }
+        if (tol_mode) {
+            const int slot = nchunk & 1;
+            cudaMemcpyAsync(hstat + (size_t)slot * count, dstat, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
+            cudaEventRecord(ev[slot], st);
+            if (nchunk >= 1) {
+                // the previous chunk's flags: the GPU keeps running the chunk just queued
+                cudaEventSynchronize(ev[slot ^ 1]);
+                stopped = true;
+                for (int q = 0; q < count; ++q) stopped = stopped && hstat[(size_t)(slot ^ 1) * count + q].stop;
+            }
+            ++nchunk;
+        }
+    }
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+        groups[gi].K.out_many<<<layout_grid(gi), 128, 0, st>>>(ditems + first_item[gi]);
+        ctx->launches += 1;
+    }
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hstat, dstat, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    for (int q = 0; q < 2; ++q)
+        if (ev[q]) cudaEventDestroy(ev[q]);
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch solve");
+    status->resize(count);
+    for (int q = 0; q < count; ++q) (*status)[q] = hstat[slot_of[q]];
     return VOMT_OK;
 }
 

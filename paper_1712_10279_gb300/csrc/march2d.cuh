@@ -20,7 +20,7 @@
 // channels 21 us (118 us: the recomputed shrinks of the one-iteration kernel spill).
 //
 // Every value is rounded as the one-iteration kernels (or, RES, the resident kernels) round
-// it, operation by operation, so that the iterates are theirs bit for bit: after hundreds
+// it, operation by operation (edges listed in the order of the pairs), so that the iterates are theirs bit for bit: after hundreds
 // of iterations w, which is zero except where a difference of phi passes its threshold,
 // differs by 1e-5 and more of its norm between two roundings of phi.  The sums over
 // channels of the graph gradient reduce to the two channels of a pair (the other terms are
@@ -81,6 +81,9 @@ __device__ __forceinline__ float rsq(float s2)
 // zero are below the squared threshold
 __device__ __forceinline__ float factor(float s2, float t) { return fmaxf(1.0f - t * rsq(s2), 0.0f); }
 
+// x x + y y in the two roundings the one-iteration kernels have
+__device__ __forceinline__ float sq2(float x, float y) { return __fmaf_rn(x, x, __fmul_rn(y, y)); }
+
 // shrink_u and shrink_w of Section 7.2 on one point, threshold t
 template <int K, int UN>
 __device__ __forceinline__ void shrink_u(float (&vx)[K], float (&vy)[K], float t)
@@ -88,14 +91,14 @@ __device__ __forceinline__ void shrink_u(float (&vx)[K], float (&vy)[K], float t
     if (UN == VOMT_U_L12) {
 #pragma unroll
         for (int c = 0; c < K; ++c) {
-            const float f = factor(vx[c] * vx[c] + vy[c] * vy[c], t);
+            const float f = factor(sq2(vx[c], vy[c]), t);
             vx[c] *= f;
             vy[c] *= f;
         }
     } else if (UN == VOMT_U_L2) {
         float s2 = 0.0f;
 #pragma unroll
-        for (int c = 0; c < K; ++c) s2 += vx[c] * vx[c] + vy[c] * vy[c];
+        for (int c = 0; c < K; ++c) s2 += sq2(vx[c], vy[c]);
         const float f = factor(s2, t);
 #pragma unroll
         for (int c = 0; c < K; ++c) { vx[c] *= f; vy[c] *= f; }
@@ -113,7 +116,7 @@ __device__ __forceinline__ void shrink_w(float (&x)[L], float t)
     } else {
         float s2 = 0.0f;
 #pragma unroll
-        for (int e = 0; e < L; ++e) s2 += x[e] * x[e];
+        for (int e = 0; e < L; ++e) s2 = __fmaf_rn(x[e], x[e], s2);
         const float f = factor(s2, t);
 #pragma unroll
         for (int e = 0; e < L; ++e) x[e] *= f;
@@ -196,18 +199,13 @@ struct Row {
 };
 
 // ------------------------------------------------------------------ S iterations
+// What warp wi of a pass does.
 template <int K, int UN, int WN, int S, bool REG, bool RES>
-__global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_constant__ MarchArgs a,
-                                                                  const __grid_constant__ MarchOp g)
+__device__ __forceinline__ void march_warp(const MarchArgs &a, const MarchOp &g, const int wi)
 {
     constexpr int L = slots(K), W = 32 - 2 * S, NQ = Quads<K>::NQ, NB = Quads<K>::NB, D = depth(K);
     constexpr int ROW = (NQ + NB) * 32;
     const int lane = threadIdx.x & 31;
-    const int wi = blockIdx.x * WARPS + (threadIdx.x >> 5);
-    cudaGridDependencySynchronize();      // after the previous kernel (no-op for a normal launch)
-    // the next pass may be scheduled from here on; it waits for this one to finish
-    cudaTriggerProgrammaticLaunchCompletion();
-    if (wi >= a.warps) return;            // whole warps
     const int n = g.n;
     const int strip = wi % a.strips, chunk = wi / a.strips;
     const int x = strip * W - S + lane;
@@ -298,8 +296,7 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_c
 #pragma unroll
                 for (int hi = lo + 1; hi < K; ++hi) {
                     const int e = pair_at(K, lo, hi);
-                    float ge = g.inv[e] * dq.p[lo];
-                    ge += -g.inv[e] * dq.p[hi];
+                    const float ge = __fmaf_rn(-g.inv[e], dq.p[hi], __fmul_rn(g.inv[e], dq.p[lo]));
                     wx[e] = dq.w[e] + g.nu * ge;
                     if (REG) wx[e] *= g.sw;
                 }
@@ -337,23 +334,56 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_c
     copies_wait<0>();
 }
 
+template <int K, int UN, int WN, int S, bool REG, bool RES>
+__global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march(const __grid_constant__ MarchArgs a,
+                                                                  const __grid_constant__ MarchOp g)
+{
+    const int wi = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    cudaGridDependencySynchronize();      // after the previous kernel (no-op for a normal launch)
+    // the next pass may be scheduled from here on; it waits for this one to finish
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (wi < a.warps) march_warp<K, UN, WN, S, REG, RES>(a, g, wi);       // whole warps
+}
+
+// The same pass over many problems of K channels and any sides (default norms): block q
+// works on problem map[q].  state 0 or 1 holds the iterates; prev: state 2 takes the
+// iterate before the last.
+template <int K, int S>
+__global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march_many(const BatchItem *__restrict__ items,
+                                                                       const int *__restrict__ map, int state, int prev)
+{
+    const BatchItem &d = items[map[blockIdx.x]];
+    constexpr int q = S == 4 ? 2 : S - 1;
+    const int wi = ((int)blockIdx.x - d.pass[q].first) * WARPS + (threadIdx.x >> 5);
+    MarchArgs a;
+    a.in = d.S[state];
+    a.out = d.S[state ^ 1];
+    a.prev = prev ? d.S[2] : nullptr;
+    a.b = d.b;
+    a.st = d.st;
+    a.rows = d.pass[q].rows;
+    a.strips = d.pass[q].strips;
+    a.warps = d.pass[q].warps;
+    const MarchOp g = d.g;
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (wi < a.warps) march_warp<K, VOMT_U_L12, VOMT_W_L1, S, false, true>(a, g, wi);
+}
+
 // ------------------------------------------------------------------ one check
 // The terms of a convergence check (the sums RED_*) of the iterate cur and its
 // predecessor prv.  The same march: both states' rows once, neighbours along x by
 // shuffles, the row below carried; strips write no columns, so a strip covers 30.  Sums
 // per thread and warp in pairs of FP32 numbers (CheckAcc), per block and grid in FP64.
 template <int K, int UN, int WN>
-__global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ CheckArgs a,
-                                                      const __grid_constant__ MarchOp g)
+__device__ __forceinline__ void check_block(const CheckArgs &a, const MarchOp &g, const int block, const int blocks)
 {
-    constexpr int L = slots(K), NQ = Quads<K>::NQ, NB = Quads<K>::NB;
-    cudaGridDependencySynchronize();
-    if (a.st->stop) return;
+    constexpr int NQ = Quads<K>::NQ, NB = Quads<K>::NB;
     const int lane = threadIdx.x & 31, n = g.n;
     const float ih = g.ih, alpha = g.alpha;
     dev::CheckAcc acc;
     acc.zero();
-    for (int wi = blockIdx.x * WARPS + (threadIdx.x >> 5); wi < a.items; wi += gridDim.x * WARPS) {
+    for (int wi = block * WARPS + (threadIdx.x >> 5); wi < a.items; wi += blocks * WARPS) {
         const int strip = wi % a.strips, chunk = wi / a.strips;
         const int x = strip * 30 - 1 + lane;
         const int y0 = chunk * a.rows, y1 = min(n, y0 + a.rows);
@@ -483,14 +513,41 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
             p0 = p1;
         }
     }
-    dev::block_sum_store<NTHR>(acc, a.partials + (size_t)blockIdx.x * NRED);
+    dev::block_sum_store<NTHR>(acc, a.partials + (size_t)block * NRED);
+}
+
+template <int K, int UN, int WN>
+__global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ CheckArgs a,
+                                                      const __grid_constant__ MarchOp g)
+{
+    cudaGridDependencySynchronize();
+    if (a.st->stop) return;
+    check_block<K, UN, WN>(a, g, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// many problems: blockIdx.y is the problem; cur, prv: which states
+template <int K>
+__global__ void __launch_bounds__(NTHR) k_check_many(const BatchItem *__restrict__ items, int cur, int prv)
+{
+    const BatchItem &d = items[blockIdx.y];
+    cudaGridDependencySynchronize();
+    if (d.st->stop) return;
+    CheckArgs a;
+    a.cur = d.S[cur];
+    a.prv = d.S[prv];
+    a.b = d.b;
+    a.partials = d.partials;
+    a.rows = d.check_rows;
+    a.strips = d.check_strips;
+    a.items = d.check_items;
+    const MarchOp g = d.g;
+    check_block<K, VOMT_U_L12, VOMT_W_L1>(a, g, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // ------------------------------------------------------------------ layouts
 // Planar fields <-> the engine's layout; b = rho1 - rho0.
 template <int K>
-__global__ void k_march_in(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g, float4 *state,
-                           float4 *bq)
+__device__ __forceinline__ void layout_in(const PlanarArgs &a, const MarchOp &g, float4 *state, float4 *bq)
 {
     const int n = g.n;
     const size_t nn = (size_t)n * n;
@@ -525,12 +582,23 @@ __global__ void k_march_in(const __grid_constant__ PlanarArgs a, const __grid_co
 }
 
 template <int K>
-__global__ void k_march_out(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g,
-                            const float4 *s0, const float4 *s1, const DevStatus *st)
+__global__ void k_march_in(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g, float4 *state,
+                           float4 *bq)
+{
+    layout_in<K>(a, g, state, bq);
+}
+template <int K>
+__global__ void k_in_many(const BatchItem *__restrict__ items)
+{
+    const BatchItem &d = items[blockIdx.z];
+    layout_in<K>(d.planar, d.g, d.S[0], d.b);
+}
+
+template <int K>
+__device__ __forceinline__ void layout_out(const PlanarArgs &a, const MarchOp &g, const float4 *state)
 {
     const int n = g.n;
     const size_t nn = (size_t)n * n;
-    const float4 *state = st->slot ? s1 : s0;
     for (int y = blockIdx.y; y < n; y += gridDim.y) {
         const int x = blockIdx.x * blockDim.x + threadIdx.x;
         if (x >= n) continue;
@@ -549,6 +617,19 @@ __global__ void k_march_out(const __grid_constant__ PlanarArgs a, const __grid_c
     }
 }
 
+template <int K>
+__global__ void k_march_out(const __grid_constant__ PlanarArgs a, const __grid_constant__ MarchOp g,
+                            const float4 *s0, const float4 *s1, const DevStatus *st)
+{
+    layout_out<K>(a, g, st->slot ? s1 : s0);
+}
+template <int K>
+__global__ void k_out_many(const BatchItem *__restrict__ items)
+{
+    const BatchItem &d = items[blockIdx.z];
+    layout_out<K>(d.planar, d.g, d.S[d.st->slot ? 1 : 0]);
+}
+
 // ------------------------------------------------------------------ dispatch
 template <int K, int UN, int WN, bool REG, bool RES = false>
 Kernels kernels_of()
@@ -557,6 +638,14 @@ Kernels kernels_of()
     q.step[0] = k_march<K, UN, WN, 1, REG, RES>;
     if constexpr (K <= 6) q.step[1] = k_march<K, UN, WN, 2, REG, RES>;
     if constexpr (K <= 3) q.step[2] = k_march<K, UN, WN, 4, REG, RES>;
+    if constexpr (RES && K <= 5) {
+        q.many[0] = k_march_many<K, 1>;
+        q.many[1] = k_march_many<K, 2>;
+        if constexpr (K <= 3) q.many[2] = k_march_many<K, 4>;
+        q.check_many = k_check_many<K>;
+        q.in_many = k_in_many<K>;
+        q.out_many = k_out_many<K>;
+    }
     q.check = k_march_check<K, UN, WN>;
     q.in = k_march_in<K>;
     q.out = k_march_out<K>;

@@ -39,6 +39,20 @@ struct PlanarArgs {
     int warm;
 };
 
+// One problem of a batch.
+struct BatchItem {
+    MarchOp g;
+    float4 *S[3], *b;                 // two states, the state before a check, rho1 - rho0
+    double *partials;
+    DevStatus *st;
+    SolveCfg cfg;
+    PlanarArgs planar;
+    struct {
+        int rows, strips, warps, first;      // of a pass of 1, 2, 4 iterations; its first block
+    } pass[3];
+    int check_rows, check_strips, check_items;
+};
+
 constexpr int kStages[3] = {1, 2, 4};   // iterations per pass of Kernels::step
 
 struct Kernels {
@@ -46,6 +60,11 @@ struct Kernels {
     void (*check)(const CheckArgs, const MarchOp);
     void (*in)(const PlanarArgs, const MarchOp, float4 *, float4 *);
     void (*out)(const PlanarArgs, const MarchOp, const float4 *, const float4 *, const DevStatus *);
+    // many problems at once (default norms, up to five channels, resident engine's order)
+    void (*many[3])(const BatchItem *, const int *, int, int);
+    void (*check_many)(const BatchItem *, int, int);
+    void (*in_many)(const BatchItem *);
+    void (*out_many)(const BatchItem *);
     int groups, bgroups;              // groups of four values of a point: state, b
     int smem;                         // shared memory of a step
 };
@@ -61,5 +80,28 @@ Kernels pick_k8(int k, int un, int wn, bool reg, bool res);
 }  // namespace march
 
 bool march_op(const OpDev &g, const StepDev &s, march::MarchOp *out);
+// whether its edges are listed in the order of the pairs: the marching form sums over the
+// edges at a channel in that order, the other kernels in the listed one
+bool edges_in_order(const march::MarchOp &m);
+
+// A batch of vector problems (default norms, eps = 0, k <= 5) in the marching form, in the
+// resident engine's order of operations (march2d.cu).
+struct BatchProblem {
+    march::MarchOp g;
+    int k;
+    SolveCfg cfg;
+    march::PlanarArgs planar;
+};
+struct BatchMarchScratch {            // device and pinned memory of march_batch, kept by the caller
+    void *items = nullptr, *maps = nullptr, *data = nullptr, *stat = nullptr, *hstat = nullptr;
+    size_t items_cap = 0, maps_cap = 0, data_cap = 0, stat_cap = 0, hstat_cap = 0;
+};
+void march_scratch_free(BatchMarchScratch *s);
+// microseconds an iteration of the batch takes by estimate
+double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p);
+// *taken = false where the memory is not to be had; status[q]: the host copy of each problem's
+// final status block, blocks[q]: the blocks of its main pass
+int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
+                cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken);
 
 }  // namespace vomt

@@ -10,6 +10,7 @@
 #include <math.h>
 
 #include "internal.h"
+#include "march2d.h"
 #include "matrix_norms.cuh"
 #include "pdhg_device.cuh"
 #include "stream_tma.h"
@@ -470,10 +471,9 @@ Launchers pick(int k, int un, int wn)
 
 // Fixed-order sum of the per-block partials, the stopping decision and the
 // history row.  One block of 256 threads.
-__global__ void k_finalize(const double *__restrict__ partials, int nblocks, SolveCfg cfg, int t,
-                           DevStatus *st, double *hist, int hist_cap, int slot)
+__device__ __forceinline__ void finalize(const double *__restrict__ partials, int nblocks, const SolveCfg &cfg, int t,
+                                         DevStatus *st, double *hist, int hist_cap, int slot)
 {
-    cudaGridDependencySynchronize();
     if (st->stop) return;
     __shared__ double S[NRED];
     // warp q sums slot q: lane j takes rows j, j + 32, ..., then a butterfly over
@@ -517,6 +517,21 @@ __global__ void k_finalize(const double *__restrict__ partials, int nblocks, Sol
         if (!finite) { st->error = VOMT_ERR_NONFINITE; st->stop = 1; }
         if (conv) st->stop = 1;
     }
+}
+
+__global__ void k_finalize(const double *__restrict__ partials, int nblocks, SolveCfg cfg, int t,
+                           DevStatus *st, double *hist, int hist_cap, int slot)
+{
+    cudaGridDependencySynchronize();
+    finalize(partials, nblocks, cfg, t, st, hist, hist_cap, slot);
+}
+
+// a block per problem of a batch
+__global__ void k_finalize_many(const march::BatchItem *__restrict__ items, int nblocks, int t, int slot)
+{
+    const march::BatchItem &d = items[blockIdx.x];
+    cudaGridDependencySynchronize();
+    finalize(d.partials, nblocks, d.cfg, t, d.st, nullptr, 0, slot);
 }
 
 // One fused iteration (Section 7.2) from the state at `in` to the state at

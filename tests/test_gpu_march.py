@@ -107,3 +107,89 @@ def test_warm_start_continues_and_a_met_tolerance_stops():
     assert a.result["rel_gap"] <= 1e-3 and a.result["rel_res"] <= 1e-3
     fixed = V.solve(_t(r0), _t(r1), edges, 1.0, max_iters=a.result["iters"], **kw)
     assert torch.equal(fixed.u, a.u) and torch.equal(fixed.phi, a.phi) and torch.equal(fixed.w, a.w)
+
+
+def _batch(shapes, seed, turn=False):
+    rng = np.random.default_rng(seed)
+    probs, r0, r1 = [], [], []
+    for n, k in shapes:
+        edges = S.random_connected_graph(rng, k, 0.6)
+        edges = edges[::-1] if turn else edges
+        a, b = S.blob_pair(n, k, seed=int(rng.integers(1 << 30)))
+        probs.append(dict(n=n, k=k, edges=edges, alpha=float(rng.uniform(0.1, 1.0)), tau=0.003 * k * n * n,
+                          cost=rng.uniform(0.5, 2.0, len(edges)) if edges else None))
+        r0.append(a.astype(np.float32))
+        r1.append(b.astype(np.float32))
+    return V.Batch(probs, r0, r1), V.Batch(probs, r0, r1)
+
+
+@pytest.mark.parametrize("shapes", [
+    [(256, 3)] * 6,
+    [(256, 1), (255, 3), (192, 5), (97, 5), (256, 3), (33, 1), (128, 3), (250, 5), (200, 2), (180, 4), (2, 1), (9, 3)],
+])
+@pytest.mark.parametrize("kw", [dict(max_iters=57, check_every=20), dict(max_iters=6, check_every=6),
+                                dict(max_iters=2400, check_every=100, tol_gap=3e-2, tol_res=3e-2)])
+def test_marching_batch_equals_the_grouped_batch(shapes, kw):
+    """AUTO's marching form of a batch against the grouped resident form: the same iterates
+    bit for bit (the kernels round alike), each problem stopped at the same check."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    auto, grouped = _batch(shapes, 5)
+    auto.solve(**kw)
+    grouped.solve(path="grouped", **kw)
+    assert all(r["variant"] == 0 and r["blocks"] >= 1 for r in auto.results)      # the marching form ran
+    assert all(r["variant"] == 1 for r in grouped.results)
+    if "tol_gap" in kw:
+        assert len({r["iters"] for r in grouped.results}) > 1 or len(set(shapes)) == 1
+    for q in range(len(shapes)):
+        a, g = auto.results[q], grouped.results[q]
+        assert a["iters"] == g["iters"] and a["status"] == g["status"] and a["checks"] == g["checks"]
+        assert torch.equal(auto.phi(q), grouped.phi(q)) and torch.equal(auto.u(q), grouped.u(q))
+        assert torch.equal(auto.w(q), grouped.w(q))
+        for key in ("primal", "dual", "rel_res"):
+            assert a[key] == pytest.approx(g[key], rel=1e-5)
+    auto.solve(warm_start=True, **kw)
+    grouped.solve(path="grouped", warm_start=True, **kw)
+    for q in range(len(shapes)):
+        assert torch.equal(auto.phi(q), grouped.phi(q)) and torch.equal(auto.w(q), grouped.w(q))
+
+
+def test_edges_out_of_order_keep_the_listed_sums():
+    """Edges that are not listed in the order of the pairs: the kernels that sum as listed."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kw = dict(max_iters=57, check_every=20)
+    auto, grouped = _batch([(256, 3)] * 4 + [(128, 4)], 7, turn=True)
+    auto.solve(**kw)
+    grouped.solve(path="grouped", **kw)
+    assert all(r["variant"] == 1 for r in auto.results)
+    for q in range(5):
+        assert torch.equal(auto.phi(q), grouped.phi(q)) and torch.equal(auto.w(q), grouped.w(q))
+    r0, r1 = _fields(80, 4, 8)
+    a, b = (V.solve(_t(r0), _t(r1), S.complete_graph(4)[::-1], 0.6, engine="stream", max_iters=40, check_every=c,
+                    tau=0.7) for c in (2, 20))
+    assert torch.equal(a.u, b.u) and torch.equal(a.w, b.w) and torch.equal(a.phi, b.phi)
+
+
+@pytest.mark.parametrize("n,k", [(352, 3), (330, 4), (256, 5), (200, 8), (400, 1)])
+def test_auto_keeps_the_resident_results(n, k):
+    """Where AUTO leaves the resident engine for the marching form, the iterates are the
+    resident engine's bit for bit."""
+    edges = S.complete_graph(k) if k > 1 else []
+    r0, r1 = _fields(n, k, n)
+    kw = dict(max_iters=47, check_every=20, tau=0.7)
+    a = V.solve(_t(r0), _t(r1), edges, 0.6, **kw)
+    b = V.solve(_t(r0), _t(r1), edges, 0.6, engine="resident", **kw)
+    assert a.result["engine"] == "stream" and b.result["engine"] == "resident"
+    assert torch.equal(a.u, b.u) and torch.equal(a.w, b.w) and torch.equal(a.phi, b.phi)
+
+
+def test_marching_keeps_the_one_iteration_results():
+    """check_every = 2 takes the one-iteration kernels, 20 the marching form: the same
+    iterates bit for bit, for every norm pair and with eps (three channels)."""
+    n, k = 75, 3
+    r0, r1 = _fields(n, k, 4)
+    for un, wn, eps in ((0, 0, 0.0), (1, 1, 0.0), (2, 0, 0.0), (0, 1, 0.4)):
+        a, b = (V.solve(_t(r0), _t(r1), S.COMPLETE_K3, 0.6, engine="stream", max_iters=40, check_every=c, tau=0.7,
+                        u_norm=un, w_norm=wn, eps=eps) for c in (2, 20))
+        assert torch.equal(a.u, b.u) and torch.equal(a.w, b.w) and torch.equal(a.phi, b.phi)
