@@ -113,17 +113,23 @@ __global__ void __launch_bounds__(1024) k_envelope(int n, int pitch, int k, int 
     if (threadIdx.x == 0 && rank == 0 && d_alpha) d_alpha[problem] = (float)(g * wtotal);
 }
 
+// The reverse step's sums, each rounded in a fixed way: the shrink's derivative jumps where
+// |v| crosses the threshold, so at a point that lies on it another rounding moves the
+// gradient (one such point of 256^2 moved dJ/dalpha by 1.7e-5).
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float madd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul_add(float a, float b, float c) { return __fadd_rn(__fmul_rn(a, b), c); }
+
 // transpose of the Jacobian of shrink_2(.; t) at v (a 2-vector), applied to H:
 // (1 - t/s) H + t (v.H) v / s^3 for s = |v| > t, else 0
 __device__ __forceinline__ void vjp_shrink2(float vx, float vy, float t, float hx, float hy, float &ox, float &oy)
 {
-    const float s2 = vx * vx + vy * vy;
+    const float s2 = dot2(vx, vx, vy, vy);
     if (s2 > t * t) {
-        const float r = rsqrtf(s2), s = s2 * r;
-        const float a = 1.0f - t * r, c = t * (vx * hx + vy * hy) * r * r * r;
-        (void)s;
-        ox = a * hx + c * vx;
-        oy = a * hy + c * vy;
+        const float r = rsqrtf(s2);
+        const float a = madd(-t, r, 1.0f), c = t * dot2(vx, hx, vy, hy) * r * r * r;
+        ox = dot2(a, hx, c, vx);
+        oy = dot2(a, hy, c, vy);
     } else {
         ox = 0.0f;
         oy = 0.0f;
@@ -190,138 +196,143 @@ __global__ void __launch_bounds__(AT) k_adj_init(int n, int l, int wn, float alp
 // derivative with respect to rho1; rho0 gets its negative) and add this block's
 // contribution to dJ/dalpha to apart[blk].  ||u||_{1,2} (per channel shrink_2).
 //
-// A warp marches up `rows` rows of a strip of 30 columns, one column per lane: the shrink's
-// adjoint is formed once per point, its x component reaches the right neighbour by a
-// shuffle and its y component the row above in a register, and every value is read once.
-// Bound by the latency of a launch at the sizes that are unrolled in practice (256^2, three
-// channels: 27 planes, 7 MB, all in L2), so launches overlap (launch_pdl).
+// A warp takes a row of a strip of 30 columns, one column per lane, and reads everything it
+// needs at once: the shrink's adjoint is formed in the row (its x component reaches the
+// right neighbour by a shuffle) and once more in the row below, whose y component enters.
+// At the sizes that are unrolled in practice a step is bound by latency (256^2, three
+// channels: 27 planes, 7 MB, all in L2): one round trip to L2 and the launch, which
+// overlaps the previous step's end (launch_pdl).
 template <int K>
 __global__ void __launch_bounds__(AT) k_adj_step(const __grid_constant__ march::MarchOp g, int wn,
                                                  const float *__restrict__ S, const float *__restrict__ A1,
                                                  float *__restrict__ A0, float *__restrict__ grho,
-                                                 double *__restrict__ apart, int rows, int strips, int warps)
+                                                 double *__restrict__ apart)
 {
     cudaGridDependencySynchronize();      // after the previous kernel (no-op for a normal launch)
     constexpr int LK = ALK<K>::v;
     const int n = g.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int wi = blockIdx.x * (AT / 32) + wid;
-    float ga = 0.0f, gl = 0.0f;           // this thread's share of dJ/dalpha, a pair kept by TwoSum
-    if (wi < warps) {
-        const int i = (wi % strips) * 30 - 1 + lane, y0 = (wi / strips) * rows, y1 = min(n, y0 + rows);
+    const int i = blockIdx.x * 30 - 1 + lane, j = blockIdx.y * AY + wid;
+    float da = 0.0f;                      // this thread's share of dJ/dalpha
+    if (j < n) {                          // whole warps
         const bool in = i >= 0 && i < n, own = in && lane >= 1 && lane < 31;
-        const bool hR = i < n - 1, hL = i > 0;
-        const size_t nn = (size_t)n * n;
+        const bool hR = i < n - 1, hL = i > 0, hU = j < n - 1, hD = j > 0;
+        const size_t nn = (size_t)n * n, p = (size_t)j * n + (in ? i : 0);
         const float mu = g.mu, nu = g.nu, tau = g.tau, ih = g.ih, muih = mu * ih;
-        const float *phi = S, *ux = S + (size_t)K * nn, *uy = S + (size_t)2 * K * nn, *w = S + (size_t)3 * K * nn;
+        const float *ux = S + (size_t)K * nn, *uy = S + (size_t)2 * K * nn, *w = S + (size_t)3 * K * nn;
         const float *Gx = A1 + (size_t)K * nn, *Gy = A1 + (size_t)2 * K * nn, *Gw = A1 + (size_t)3 * K * nn;
-        const int jb = y0 > 0 ? y0 - 1 : 0;
-        float pc[K], qc[K], gd[K];        // phi and its adjoint in the row, the y component of the row below
+        const bool iu = in && hU, id = in && hD;
+        float pc[K], qc[K], pu[K], qu[K], pd[K], qd[K], x[K], y[K], hx[K], hy[K], xd[K], yd[K], hxd[K], hyd[K], gr[K];
+        float w0[LK], hw[LK];
 #pragma unroll
         for (int c = 0; c < K; ++c) {
-            const size_t o = c * nn + (size_t)jb * n + i;
-            pc[c] = in ? phi[o] : 0.0f;
+            const size_t o = c * nn + p;
+            pc[c] = in ? S[o] : 0.0f;
             qc[c] = in ? A1[o] : 0.0f;
-            gd[c] = 0.0f;
+            pu[c] = iu ? S[o + n] : 0.0f;
+            qu[c] = iu ? A1[o + n] : 0.0f;
+            pd[c] = id ? S[o - n] : 0.0f;
+            qd[c] = id ? A1[o - n] : 0.0f;
+            x[c] = in ? ux[o] : 0.0f;
+            y[c] = in ? uy[o] : 0.0f;
+            hx[c] = in ? Gx[o] : 0.0f;
+            hy[c] = in ? Gy[o] : 0.0f;
+            xd[c] = id ? ux[o - n] : 0.0f;
+            yd[c] = id ? uy[o - n] : 0.0f;
+            hxd[c] = id ? Gx[o - n] : 0.0f;
+            hyd[c] = id ? Gy[o - n] : 0.0f;
+            gr[c] = own ? grho[o] : 0.0f;
         }
-        for (int j = jb; j < y1; ++j) {
-            const bool hU = j < n - 1, hD = j > 0, wr = own && j >= y0;
-            const size_t p = (size_t)j * n + i;
-            float pu[K], qu[K], dvg[K];
+#pragma unroll
+        for (int e = 0; e < K * (K - 1) / 2; ++e) {
+            const int ed = g.edge[e];
+            w0[e] = ed >= 0 && own ? w[ed * nn + p] : 0.0f;
+            hw[e] = ed >= 0 && own ? Gw[ed * nn + p] : 0.0f;
+        }
+        float dvg[K];
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            const float pr = __shfl_down_sync(0xffffffffu, pc[c], 1), qr = __shfl_down_sync(0xffffffffu, qc[c], 1);
+            const float prd = __shfl_down_sync(0xffffffffu, pd[c], 1), qrd = __shfl_down_sync(0xffffffffu, qd[c], 1);
+            const float ax = hR ? ih * (qr - qc[c]) : 0.0f, ay = hU ? ih * (qu[c] - qc[c]) : 0.0f;
+            const float ex = hR ? pr - pc[c] : 0.0f, ey = hU ? pu[c] - pc[c] : 0.0f;
+            const float kx = madd(-2.0f * tau, ax, hx[c]), ky = madd(-2.0f * tau, ay, hy[c]);
+            float gvx, gvy, glx, gdy = 0.0f, t_;
+            vjp_shrink2(mul_add(muih, ex, x[c]), mul_add(muih, ey, y[c]), mu, kx, ky, gvx, gvy);
+            // its x component as the right neighbour has it
+            vjp_shrink2(madd(muih, ex, x[c]), mul_add(muih, ey, y[c]), mu, kx, ky, glx, t_);
+            if (hD) {                     // the y component in the row below
+                const float dax = hR ? ih * (qrd - qd[c]) : 0.0f, day = ih * (qc[c] - qd[c]);
+                const float edx = hR ? prd - pd[c] : 0.0f;
+                vjp_shrink2(mul_add(muih, edx, xd[c]), madd(muih, pc[c] - pd[c], yd[c]), mu,
+                            madd(-2.0f * tau, dax, hxd[c]), madd(-2.0f * tau, day, hyd[c]), t_, gdy);
+            }
+            const float left = __shfl_up_sync(0xffffffffu, glx, 1);
+            dvg[c] = ih * ((gvx - (hL ? left : 0.0f)) + (gvy - gdy));      // div of the shrink adjoint
+            if (own) {
+                A0[(K + c) * nn + p] = madd(tau, ax, gvx);
+                A0[(2 * K + c) * nn + p] = madd(tau, ay, gvy);
+            }
+        }
+        if (own) {
+            // graph part
+            float xw[LK], dq[LK], gxw[LK];
+            const float th = g.alpha * nu;
+            float s2 = 0.0f, xh = 0.0f;
+#pragma unroll
+            for (int lo = 0; lo < K; ++lo)
+#pragma unroll
+                for (int hi = lo + 1; hi < K; ++hi) {
+                    const int e = lo * (2 * K - lo - 1) / 2 + hi - lo - 1;
+                    dq[e] = dot2(-g.inv[e], qc[hi], g.inv[e], qc[lo]);
+                    xw[e] = madd(nu, dot2(-g.inv[e], pc[hi], g.inv[e], pc[lo]), w0[e]);    // 0 where there is no edge
+                    hw[e] = madd(-2.0f * tau, dq[e], hw[e]);
+                    gxw[e] = 0.0f;
+                    s2 = madd(xw[e], xw[e], s2);
+                    xh = madd(xw[e], hw[e], xh);
+                }
+            if (wn == VOMT_W_L1) {
+#pragma unroll
+                for (int e = 0; e < K * (K - 1) / 2; ++e)
+                    if (fabsf(xw[e]) > th) {
+                        gxw[e] = hw[e];
+                        da -= nu * (xw[e] > 0.0f ? hw[e] : -hw[e]);
+                    }
+            } else if (s2 > th * th) {
+                const float r = rsqrtf(s2), a = madd(-th, r, 1.0f), c3 = th * xh * r * r * r;
+#pragma unroll
+                for (int e = 0; e < K * (K - 1) / 2; ++e) gxw[e] = dot2(a, hw[e], c3, xw[e]);
+                da = -nu * (xh * r);
+            }
+            float gg[K];
+#pragma unroll
+            for (int c = 0; c < K; ++c) gg[c] = 0.0f;
+#pragma unroll
+            for (int lo = 0; lo < K; ++lo)
+#pragma unroll
+                for (int hi = lo + 1; hi < K; ++hi) {
+                    const int e = lo * (2 * K - lo - 1) / 2 + hi - lo - 1, ed = g.edge[e];
+                    if (ed >= 0) A0[(3 * K + ed) * nn + p] = mul_add(tau, dq[e], gxw[e]);
+                    gg[lo] = madd(g.inv[e], gxw[e], gg[lo]);
+                    gg[hi] = madd(-g.inv[e], gxw[e], gg[hi]);
+                }
 #pragma unroll
             for (int c = 0; c < K; ++c) {
-                const size_t o = c * nn + p;
-                pu[c] = in && hU ? phi[o + n] : 0.0f;
-                qu[c] = in && hU ? A1[o + n] : 0.0f;
-                const float pr = __shfl_down_sync(0xffffffffu, pc[c], 1), qr = __shfl_down_sync(0xffffffffu, qc[c], 1);
-                const float x0 = in ? ux[o] : 0.0f, yy0 = in ? uy[o] : 0.0f;
-                const float hx = in ? Gx[o] : 0.0f, hy = in ? Gy[o] : 0.0f;
-                const float ax = hR ? ih * (qr - qc[c]) : 0.0f, ay = hU ? ih * (qu[c] - qc[c]) : 0.0f;
-                const float vx = x0 + (hR ? muih * (pr - pc[c]) : 0.0f);
-                const float vy = yy0 + (hU ? muih * (pu[c] - pc[c]) : 0.0f);
-                float gvx, gvy;
-                vjp_shrink2(vx, vy, mu, hx - 2.0f * tau * ax, hy - 2.0f * tau * ay, gvx, gvy);
-                const float left = __shfl_up_sync(0xffffffffu, gvx, 1), glx = hL ? left : 0.0f;
-                dvg[c] = ih * ((gvx - glx) + (gvy - (hD ? gd[c] : 0.0f)));      // div of the shrink adjoint
-                gd[c] = gvy;
-                if (wr) {
-                    A0[(K + c) * nn + p] = gvx + tau * ax;
-                    A0[(2 * K + c) * nn + p] = gvy + tau * ay;
-                }
-            }
-            if (wr) {
-                // graph part
-                float xw[LK], hw[LK], dq[LK], gxw[LK];
-                const float th = g.alpha * nu;
-                float s2 = 0.0f, xh = 0.0f;
-#pragma unroll
-                for (int lo = 0; lo < K; ++lo)
-#pragma unroll
-                    for (int hi = lo + 1; hi < K; ++hi) {
-                        const int e = lo * (2 * K - lo - 1) / 2 + hi - lo - 1, ed = g.edge[e];
-                        dq[e] = g.inv[e] * (qc[lo] - qc[hi]);
-                        xw[e] = ed >= 0 ? w[ed * nn + p] + nu * (g.inv[e] * (pc[lo] - pc[hi])) : 0.0f;
-                        hw[e] = ed >= 0 ? Gw[ed * nn + p] - 2.0f * tau * dq[e] : 0.0f;
-                        gxw[e] = 0.0f;
-                        s2 += xw[e] * xw[e];
-                        xh += xw[e] * hw[e];
-                    }
-                float da = 0.0f;
-                if (wn == VOMT_W_L1) {
-#pragma unroll
-                    for (int e = 0; e < K * (K - 1) / 2; ++e)
-                        if (fabsf(xw[e]) > th) {
-                            gxw[e] = hw[e];
-                            da -= nu * (xw[e] > 0.0f ? hw[e] : -hw[e]);
-                        }
-                } else if (s2 > th * th) {
-                    const float r = rsqrtf(s2), a = 1.0f - th * r, c3 = th * xh * r * r * r;
-#pragma unroll
-                    for (int e = 0; e < K * (K - 1) / 2; ++e) gxw[e] = a * hw[e] + c3 * xw[e];
-                    da = -nu * (xh * r);
-                }
-                float err;
-                ga = dev::two_sum(ga, da, err);
-                gl += err;
-                float gg[K];
-#pragma unroll
-                for (int c = 0; c < K; ++c) gg[c] = 0.0f;
-#pragma unroll
-                for (int lo = 0; lo < K; ++lo)
-#pragma unroll
-                    for (int hi = lo + 1; hi < K; ++hi) {
-                        const int e = lo * (2 * K - lo - 1) / 2 + hi - lo - 1, ed = g.edge[e];
-                        if (ed >= 0) A0[(3 * K + ed) * nn + p] = tau * dq[e] + gxw[e];
-                        gg[lo] += g.inv[e] * gxw[e];
-                        gg[hi] -= g.inv[e] * gxw[e];
-                    }
-#pragma unroll
-                for (int c = 0; c < K; ++c) {
-                    A0[c * nn + p] = qc[c] - mu * dvg[c] + nu * gg[c];
-                    grho[c * nn + p] += tau * qc[c];
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < K; ++c) {
-                pc[c] = pu[c];
-                qc[c] = qu[c];
+                A0[c * nn + p] = madd(nu, gg[c], madd(-mu, dvg[c], qc[c]));
+                grho[c * nn + p] = madd(tau, qc[c], gr[c]);
             }
         }
     }
-    // the block's sum: pairs over a warp, FP64 over the warps
-    __shared__ double sh[AT / 32];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const float oh = __shfl_down_sync(0xffffffffu, ga, off), ol = __shfl_down_sync(0xffffffffu, gl, off);
-        float err;
-        ga = dev::two_sum(ga, oh, err);
-        gl += ol + err;
-    }
-    if (lane == 0) sh[wid] = (double)ga + (double)gl;
+    // the block's sum: FP32 pairs over a warp, FP64 over the warps
+    __shared__ double sh[AY];
+    dev::PairSum sum;
+    sum.add(da);
+    sum.warp();
+    if (lane == 0) sh[wid] = sum.value();
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int q = 0; q < AT / 32; ++q) t += sh[q];
-        apart[blockIdx.x] += t;
+        for (int q = 0; q < AY; ++q) t += sh[q];
+        apart[blockIdx.y * gridDim.x + blockIdx.x] += t;
     }
 }
 
@@ -341,8 +352,7 @@ __global__ void k_finish_grad(size_t cnt, float scale, const float *__restrict__
 }
 
 using AdjInit = void (*)(int, int, int, float, const float *, float *, double *);
-using AdjStep = void (*)(const march::MarchOp, int, const float *, const float *, float *, float *, double *, int, int,
-                         int);
+using AdjStep = void (*)(const march::MarchOp, int, const float *, const float *, float *, float *, double *);
 
 template <int K>
 void pick_adj_k(AdjInit *ai, AdjStep *as)
@@ -442,10 +452,8 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         if (rc) return rc;
         const dim3 blk(AX, AY), grd((n + AX - 1) / AX, (n + AY - 1) / AY);
         const int nb = (int)(grd.x * grd.y);
-        // reverse steps: chunks of rows that give every scheduler a warp or two
-        const int strips = (n + 29) / 30;
-        const int rows = std::max(2, (int)(((long)strips * n + 8 * ctx->sm_count - 1) / (8 * ctx->sm_count)));
-        const int warps = strips * ((n + rows - 1) / rows), rb = (warps + AT / 32 - 1) / (AT / 32);
+        const dim3 rgrd((n + 29) / 30, (n + AY - 1) / AY);        // reverse steps: strips of 30 columns
+        const int rb = (int)(rgrd.x * rgrd.y);
         rc = ensure_buffer(ctx, (void **)&ctx->gpart, &ctx->gpart_bytes, sizeof(double) * (2 * (size_t)nb + rb), "gradient sums");
         if (rc) return rc;
         float *b = ctx->gbuf, *grho = b + (size_t)K * nn;
@@ -477,8 +485,8 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         ++ctx->launches;
         int a_in = 0;
         auto reverse = [&](const float *St) {
-            launch_pdl(as, dim3(rb), dim3(AT), 0, st, mop, p.w_norm, St, (const float *)(adj + (size_t)a_in * SZ),
-                       adj + (size_t)(1 - a_in) * SZ, grho, apart, rows, strips, warps);
+            launch_pdl(as, rgrd, dim3(AT), 0, st, mop, p.w_norm, St, (const float *)(adj + (size_t)a_in * SZ),
+                       adj + (size_t)(1 - a_in) * SZ, grho, apart);
             ++ctx->launches;
             a_in = 1 - a_in;
         };
