@@ -88,6 +88,24 @@ double plan_cost(int TX, int TY, int H, int G, int rt = RES_THREADS, bool heavy 
     return per_pt * spill(ext) * pts / H + 3100.0 / H;
 }
 
+// Estimated nanoseconds per iteration of a single problem with up to four channels (the
+// grouped waves keep plan_cost, which their choice of path is fitted to): a step's floor
+// (two barriers and the chain through a point) plus its points, an exchange every H steps.
+// Against all plans measured at k = 1 and 3, n = 32 .. 256, it picks within 3% of the
+// fastest: 32^2, k = 3: 4 x 5 tiles, H = 6, 0.75 us (8 x 8, H = 4: 0.81); 64^2: 0.76 (0.81);
+// 192^2: 24 x 11 points, H = 3, 1.28 (1.33); 128^2 and 256^2 unchanged (0.86, 1.57).
+double plan_cost_small(int k, int TX, int TY, int H, int G, int rt)
+{
+    const double floor_ns = 140.0 + 50.0 * k, slope = 0.19 + 0.17 * k, exch = 1100.0 + 270.0 * k;
+    const int ext = G == 1 ? TX * TY : (TX + 2 * H) * (TY + 2 * H);
+    // two points per thread cost more each; four spill
+    const double per_pt = slope * (ext <= rt ? 1.0 : (ext <= 2 * rt ? 1.75 : 2.9));
+    if (G == 1) return floor_ns + per_pt * ext;
+    double pts = 0.0;
+    for (int s = 1; s <= H; ++s) pts += (double)(TX + 2 * (H - s) + 1) * (TY + 2 * (H - s) + 1);
+    return floor_ns + per_pt * pts / H + exch / H;
+}
+
 }  // namespace
 
 // Tile plan.  Tiles of at most 64 x 64 points, at most `max_blocks` of them; the
@@ -104,37 +122,44 @@ bool resident_plan(int n, int k, int max_blocks, int force_H, ResidentPlan *out)
     };
     const int RT = res::res_threads(k), max_points = 4 * RT;
     const bool heavy = RT < RES_THREADS, k34 = k >= 3 && k <= 4;
-    double best = -1.0;
-    for (int Gx = 1; Gx <= n && Gx <= max_blocks; ++Gx) {
-        const int TX = (n + Gx - 1) / Gx, TXmin = n / Gx;
-        if (TX > TMAX) continue;
-        for (int Gy = 1; Gy <= n && Gx * Gy <= max_blocks; ++Gy) {
-            const int TY = (n + Gy - 1) / Gy, TYmin = n / Gy;
-            if (TY > TMAX) continue;
-            const int G = Gx * Gy;
-            if (G == 1) {
-                if (TX * TY > max_points || !smem_ok(TX, TY, 1)) continue;
-                const double cost = plan_cost(TX, TY, 0, 1, RT, heavy, k34);
-                if (best < 0 || cost < best) {
-                    best = cost;
-                    *out = ResidentPlan{Gx, Gy, TX, TY, 0, 0, 0, cost};
+    const auto search = [&](auto cost_of) {
+        double best = -1.0;
+        for (int Gx = 1; Gx <= n && Gx <= max_blocks; ++Gx) {
+            const int TX = (n + Gx - 1) / Gx, TXmin = n / Gx;
+            if (TX > TMAX) continue;
+            for (int Gy = 1; Gy <= n && Gx * Gy <= max_blocks; ++Gy) {
+                const int TY = (n + Gy - 1) / Gy, TYmin = n / Gy;
+                if (TY > TMAX) continue;
+                const int G = Gx * Gy;
+                if (G == 1) {
+                    if (TX * TY > max_points || !smem_ok(TX, TY, 1)) continue;
+                    const double cost = cost_of(TX, TY, 0, 1);
+                    if (best < 0 || cost < best) {
+                        best = cost;
+                        *out = ResidentPlan{Gx, Gy, TX, TY, 0, 0, 0, cost};
+                    }
+                    continue;
                 }
-                continue;
-            }
-            for (int H = 1; H <= HMAX; ++H) {
-                if (force_H > 0 && H != force_H) continue;
-                if (H > TXmin || H > TYmin) break;
-                const int EW = TX + 2 * H, EH = TY + 2 * H;
-                if (EW * EH > max_points || !smem_ok(EW, EH, G)) break;
-                const double cost = plan_cost(TX, TY, H, G, RT, heavy, k34);
-                if (best < 0 || cost < best) {
-                    best = cost;
-                    *out = ResidentPlan{Gx, Gy, TX, TY, H, 0, 0, cost};
+                for (int H = 1; H <= HMAX; ++H) {
+                    if (force_H > 0 && H != force_H) continue;
+                    if (H > TXmin || H > TYmin) break;
+                    const int EW = TX + 2 * H, EH = TY + 2 * H;
+                    if (EW * EH > max_points || !smem_ok(EW, EH, G)) break;
+                    const double cost = cost_of(TX, TY, H, G);
+                    if (best < 0 || cost < best) {
+                        best = cost;
+                        *out = ResidentPlan{Gx, Gy, TX, TY, H, 0, 0, cost};
+                    }
                 }
             }
         }
-    }
-    if (best < 0) return false;
+        return best >= 0;
+    };
+    // small problems first; where their estimate wants more than a point per thread or an
+    // exchange every step or two (from about 200^2), plan_cost, fitted there, chooses
+    if (k > 4 || !search([&](int TX, int TY, int H, int G) { return plan_cost_small(k, TX, TY, H, G, RT); }) ||
+        (out->TXm + 2 * out->H) * (out->TYm + 2 * out->H) > RT || (out->Gx * out->Gy > 1 && out->H < 3))
+        if (!search([&](int TX, int TY, int H, int G) { return plan_cost(TX, TY, H, G, RT, heavy, k34); })) return false;
     const int EW = out->TXm + 2 * out->H, EH = out->TYm + 2 * out->H;
     // P points per thread, the fewest that fit RT threads, spread evenly over
     // round_up(ext / P, 32) threads; two points on at most 384 threads take the
