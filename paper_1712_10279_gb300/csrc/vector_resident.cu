@@ -57,6 +57,9 @@ constexpr int SMEM_MAX = 227 * 1024;
 // four channels; 170 registers a thread).
 constexpr int kTwoPoint384Max = 768;
 
+// points of the step after which the ring is h cells wide
+double ring_points(int TX, int TY, int h) { return (double)(TX + 2 * h + 1) * (TY + 2 * h + 1); }
+
 // Estimated nanoseconds per iteration (see resident_plan).  Constants fitted to
 // GB300 measurements of this kernel at k = 3: 3.5 ns per point of the region a
 // step updates (arithmetic, shared-memory traffic and the two barriers of a
@@ -73,7 +76,8 @@ constexpr int kTwoPoint384Max = 768;
 // so their steps are charged 65% more.  One point per thread stays
 // the cheapest where it fits (128^2, k = 3: 0.92 us per iteration at one point
 // against 1.23 at two).
-double plan_cost(int TX, int TY, int H, int G, int rt = RES_THREADS, bool heavy = false, bool k34 = false)
+// points: the points H steps between exchanges compute (ring_points)
+double plan_cost(int TX, int TY, int H, int G, double points, int rt = RES_THREADS, bool heavy = false, bool k34 = false)
 {
     auto spill = [&](int ext) {
         if (k34 && ext > 2 * rt) return 1.65;
@@ -82,10 +86,8 @@ double plan_cost(int TX, int TY, int H, int G, int rt = RES_THREADS, bool heavy 
     };
     const double per_pt = 3.5;
     if (G == 1) return per_pt * TX * TY * spill(TX * TY);
-    double pts = 0.0;
-    for (int s = 1; s <= H; ++s) pts += (double)(TX + 2 * (H - s) + 1) * (TY + 2 * (H - s) + 1);
     const int ext = (TX + 2 * H) * (TY + 2 * H);
-    return per_pt * spill(ext) * pts / H + 3100.0 / H;
+    return per_pt * spill(ext) * points / H + 3100.0 / H;
 }
 
 // Estimated nanoseconds per iteration of a single problem with up to four channels (the
@@ -94,16 +96,14 @@ double plan_cost(int TX, int TY, int H, int G, int rt = RES_THREADS, bool heavy 
 // Against all plans measured at k = 1 and 3, n = 32 .. 256, it picks within 3% of the
 // fastest: 32^2, k = 3: 4 x 5 tiles, H = 6, 0.75 us (8 x 8, H = 4: 0.81); 64^2: 0.76 (0.81);
 // 192^2: 24 x 11 points, H = 3, 1.28 (1.33); 128^2 and 256^2 unchanged (0.86, 1.57).
-double plan_cost_small(int k, int TX, int TY, int H, int G, int rt)
+double plan_cost_small(int k, int TX, int TY, int H, int G, double points, int rt)
 {
     const double floor_ns = 140.0 + 50.0 * k, slope = 0.19 + 0.17 * k, exch = 1100.0 + 270.0 * k;
     const int ext = G == 1 ? TX * TY : (TX + 2 * H) * (TY + 2 * H);
     // two points per thread cost more each; four spill
     const double per_pt = slope * (ext <= rt ? 1.0 : (ext <= 2 * rt ? 1.75 : 2.9));
     if (G == 1) return floor_ns + per_pt * ext;
-    double pts = 0.0;
-    for (int s = 1; s <= H; ++s) pts += (double)(TX + 2 * (H - s) + 1) * (TY + 2 * (H - s) + 1);
-    return floor_ns + per_pt * pts / H + exch / H;
+    return floor_ns + per_pt * points / H + exch / H;
 }
 
 }  // namespace
@@ -133,20 +133,23 @@ bool resident_plan(int n, int k, int max_blocks, int force_H, ResidentPlan *out)
                 const int G = Gx * Gy;
                 if (G == 1) {
                     if (TX * TY > max_points || !smem_ok(TX, TY, 1)) continue;
-                    const double cost = cost_of(TX, TY, 0, 1);
+                    const double cost = cost_of(TX, TY, 0, 1, 0.0);
                     if (best < 0 || cost < best) {
                         best = cost;
                         *out = ResidentPlan{Gx, Gy, TX, TY, 0, 0, 0, cost};
                     }
                     continue;
                 }
+                double points = 0.0;
                 for (int H = 1; H <= HMAX; ++H) {
+                    points += ring_points(TX, TY, H - 1);
                     if (force_H > 0 && H != force_H) continue;
                     if (H > TXmin || H > TYmin) break;
                     const int EW = TX + 2 * H, EH = TY + 2 * H;
-                    if (EW * EH > max_points || !smem_ok(EW, EH, G)) break;
-                    const double cost = cost_of(TX, TY, H, G);
+                    if (EW * EH > max_points) break;
+                    const double cost = cost_of(TX, TY, H, G, points);
                     if (best < 0 || cost < best) {
+                        if (!smem_ok(EW, EH, G)) break;
                         best = cost;
                         *out = ResidentPlan{Gx, Gy, TX, TY, H, 0, 0, cost};
                     }
@@ -157,9 +160,10 @@ bool resident_plan(int n, int k, int max_blocks, int force_H, ResidentPlan *out)
     };
     // small problems first; where their estimate wants more than a point per thread or an
     // exchange every step or two (from about 200^2), plan_cost, fitted there, chooses
-    if (k > 4 || !search([&](int TX, int TY, int H, int G) { return plan_cost_small(k, TX, TY, H, G, RT); }) ||
+    if (k > 4 || !search([&](int TX, int TY, int H, int G, double q) { return plan_cost_small(k, TX, TY, H, G, q, RT); }) ||
         (out->TXm + 2 * out->H) * (out->TYm + 2 * out->H) > RT || (out->Gx * out->Gy > 1 && out->H < 3))
-        if (!search([&](int TX, int TY, int H, int G) { return plan_cost(TX, TY, H, G, RT, heavy, k34); })) return false;
+        if (!search([&](int TX, int TY, int H, int G, double q) { return plan_cost(TX, TY, H, G, q, RT, heavy, k34); }))
+            return false;
     const int EW = out->TXm + 2 * out->H, EH = out->TYm + 2 * out->H;
     // P points per thread, the fewest that fit RT threads, spread evenly over
     // round_up(ext / P, 32) threads; two points on at most 384 threads take the
@@ -197,19 +201,22 @@ bool resident_plan_wave(int n, int k, int count, int max_blocks, ResidentPlan *o
             const double rounds = (double)((count + side - 1) / side);
             if (G == 1) {
                 if (TX * TY > max_points || !smem_ok(TX, TY, 1)) continue;
-                const double cost = rounds * plan_cost(TX, TY, 0, 1, RT, heavy, k34);
+                const double cost = rounds * plan_cost(TX, TY, 0, 1, 0.0, RT, heavy, k34);
                 if (best < 0 || cost < best) {
                     best = cost;
                     *out = ResidentPlan{Gx, Gy, TX, TY, 0, 0, 0, cost};
                 }
                 continue;
             }
+            double points = 0.0;
             for (int H = 1; H <= HMAX; ++H) {
+                points += ring_points(TX, TY, H - 1);
                 if (H > TXmin || H > TYmin) break;
                 const int EW = TX + 2 * H, EH = TY + 2 * H;
-                if (EW * EH > max_points || !smem_ok(EW, EH, G)) break;
-                const double cost = rounds * plan_cost(TX, TY, H, G, RT, heavy, k34);
+                if (EW * EH > max_points) break;
+                const double cost = rounds * plan_cost(TX, TY, H, G, points, RT, heavy, k34);
                 if (best < 0 || cost < best) {
+                    if (!smem_ok(EW, EH, G)) break;
                     best = cost;
                     *out = ResidentPlan{Gx, Gy, TX, TY, H, 0, 0, cost};
                 }
