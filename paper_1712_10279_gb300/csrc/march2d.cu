@@ -197,11 +197,13 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
     }
     float4 *b = (float4 *)ctx->ws, *S[3] = {b + b4, b + b4 + state4, b + b4 + 2 * state4};
 
-    // the check: strips of 30 columns, chunks that give every SM work, at most kMetricBlocks blocks
+    // the check: strips of 30 columns, chunks that give every SM work, at most kMetricBlocks
+    // blocks (k_finalize adds a row per block: with 998 blocks at 1024^2 it took 14.7 us, with
+    // 604 9.2)
     CheckArgs ca;
     memset(&ca, 0, sizeof ca);
     ca.strips = (n + 29) / 30;
-    ca.rows = std::max(4, (int)(((long)ca.strips * n + kMetricBlocks * kWarps - 1) / (kMetricBlocks * kWarps)));
+    ca.rows = std::max(4, (int)(((long)ca.strips * n + (long)kMetricBlocks * kWarps - 1) / ((long)kMetricBlocks * kWarps)));
     ca.items = ca.strips * ((n + ca.rows - 1) / ca.rows);
     const int mblocks = std::min((ca.items + kWarps - 1) / kWarps, kMetricBlocks);
     rc = ensure_buffer(ctx, (void **)&ctx->partials, &ctx->partials_cap, sizeof(double) * (size_t)mblocks * NRED, "partials");
@@ -296,7 +298,7 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
 }
 
 // ------------------------------------------------------------------ batches
-__global__ void k_finalize_many(const march::BatchItem *__restrict__ items, int nblocks, int t, int slot);
+__global__ void k_finalize_many(const march::BatchItem *__restrict__ items, int t, int slot);
 
 void march_scratch_free(BatchMarchScratch *s)
 {
@@ -310,7 +312,9 @@ void march_scratch_free(BatchMarchScratch *s)
 
 namespace {
 
-constexpr int kCheckBlocks = 8;       // blocks of a problem's check
+// A check's chunk of rows for `strip_rows` rows of strips: 16 warps per SM, enough to hide
+// the loads of a row (8 x 256^2, three channels: 140 us with 8 blocks a problem, 30 so).
+int check_chunk(long strip_rows, int sms) { return (int)std::max(2l, (strip_rows + 16l * sms - 1) / (16l * sms)); }
 
 // The problems of one channel count: passes over all of them at once, with chunks of the
 // same number of rows in every problem.
@@ -319,6 +323,7 @@ struct Group {
     std::vector<int> probs;
     Kernels K;
     Pass pass[3];                     // blocks: of the whole group
+    int check_rows = 2, check_blocks = 0;
 };
 
 // plan_pass for a group: the chunk length of the least arithmetic time
@@ -424,7 +429,19 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
             off[q] = floats4;
             floats4 += tile * (3 * (size_t)g.K.groups + g.K.bgroups);
         }
-    const size_t sums = sizeof(double) * NRED * kCheckBlocks * (size_t)count;
+    size_t sum_rows = 0;
+    for (Group &g : groups) {
+        long strip_rows = 0;
+        for (int q : g.probs) strip_rows += (long)((probs[q].g.n + 29) / 30) * probs[q].g.n;
+        g.check_rows = check_chunk(strip_rows, ctx->sm_count);
+        g.check_blocks = 0;
+        for (int q : g.probs) {
+            const int n = probs[q].g.n, items = (n + 29) / 30 * ((n + g.check_rows - 1) / g.check_rows);
+            g.check_blocks += (items + kWarps - 1) / kWarps;
+        }
+        sum_rows += g.check_blocks;
+    }
+    const size_t sums = sizeof(double) * NRED * sum_rows;
     rc = ensure_buffer(ctx, &scr->data, &scr->data_cap, sizeof(float4) * floats4 + sums, "batch states");
     if (rc) {
         ctx->err.clear();
@@ -446,13 +463,14 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
     DevStatus *dstat = (DevStatus *)scr->stat, *hstat = (DevStatus *)scr->hstat;
     blocks->assign(count, 1);
     int at = 0;
-    std::vector<size_t> map_at(groups.size() * 3, 0);
+    size_t sum_at = 0;
+    std::vector<size_t> map_at(groups.size() * 4, 0);      // of its three passes and its check
     std::vector<int> first_item(groups.size()), top(groups.size(), 0);
     for (size_t gi = 0; gi < groups.size(); ++gi) {
         const Group &g = groups[gi];
         first_item[gi] = at;
-        int next[3] = {0, 0, 0};
-        std::vector<int> gm[3];
+        int next[4] = {0, 0, 0, 0};
+        std::vector<int> gm[4];
         for (size_t i = 0; i < g.probs.size(); ++i, ++at) {
             const int q = g.probs[i], n = probs[q].g.n;
             const size_t tile = (size_t)n * ((n + 31) / 32) * 32;
@@ -466,7 +484,6 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
             d.b = data + off[q];
             for (int c = 0; c < 3; ++c) d.S[c] = d.b + tile * (g.K.bgroups + (size_t)c * g.K.groups);
             d.st = dstat + at;
-            d.partials = dsums + (size_t)at * NRED * kCheckBlocks;
             for (int c = 0; c < 3; ++c) {
                 if (!g.pass[c].stages) continue;
                 const int W = 32 - 2 * kStages[c];
@@ -480,16 +497,22 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
                 if (c == g.main_pass) (*blocks)[q] = nb;
             }
             d.check_strips = (n + 29) / 30;
-            d.check_rows = std::max(2, (d.check_strips * n + kCheckBlocks * kWarps - 1) / (kCheckBlocks * kWarps));
+            d.check_rows = g.check_rows;
             d.check_items = d.check_strips * ((n + d.check_rows - 1) / d.check_rows);
+            d.check_blocks = (d.check_items + kWarps - 1) / kWarps;
+            d.check_first = next[3];
+            d.partials = dsums + (sum_at + next[3]) * NRED;
+            gm[3].insert(gm[3].end(), d.check_blocks, (int)i);
+            next[3] += d.check_blocks;
             slot_of[q] = at;
             top[gi] = std::max(top[gi], n);
         }
-        for (int c = 0; c < 3; ++c) {
-            map_at[gi * 3 + c] = maps.size();
+        for (int c = 0; c < 4; ++c) {
+            map_at[gi * 4 + c] = maps.size();
             maps.insert(maps.end(), gm[c].begin(), gm[c].end());
-            groups[gi].pass[c].blocks = next[c];
+            if (c < 3) groups[gi].pass[c].blocks = next[c];
         }
+        sum_at += next[3];
     }
     rc = ensure_buffer(ctx, &scr->maps, &scr->maps_cap, sizeof(int) * maps.size(), "batch tables");
     if (rc) return rc;
@@ -512,7 +535,7 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
         const Group &g = groups[gi];
         const int prev = last && kStages[q] > 1 ? 1 : 0;
         launch_pdl(g.K.many[q], dim3(g.pass[q].blocks), dim3(32 * kWarps), (size_t)g.pass[q].smem, st,
-                   ditems + first_item[gi], dmaps + map_at[gi * 3 + q], cur[gi], prev);
+                   ditems + first_item[gi], dmaps + map_at[gi * 4 + q], cur[gi], prev);
         ctx->launches += 1;
         before[gi] = prev ? 2 : cur[gi];
         cur[gi] ^= 1;
@@ -528,9 +551,9 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
     auto check = [&](size_t gi, int t) {
         const Group &g = groups[gi];
         const unsigned np = (unsigned)g.probs.size();
-        launch_pdl(g.K.check_many, dim3(kCheckBlocks, np), dim3(32 * kWarps), 0, st, ditems + first_item[gi], cur[gi],
-                   before[gi]);
-        launch_pdl(k_finalize_many, dim3(np), dim3(kFinThreads), 0, st, ditems + first_item[gi], kCheckBlocks, t, cur[gi]);
+        launch_pdl(g.K.check_many, dim3(g.check_blocks), dim3(32 * kWarps), 0, st, ditems + first_item[gi],
+                   dmaps + map_at[gi * 4 + 3], cur[gi], before[gi]);
+        launch_pdl(k_finalize_many, dim3(np), dim3(kFinThreads), 0, st, ditems + first_item[gi], t, cur[gi]);
         ctx->launches += 2;
     };
     if (p.max_iters == 0)

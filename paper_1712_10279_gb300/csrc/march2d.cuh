@@ -525,13 +525,12 @@ __global__ void __launch_bounds__(NTHR) k_march_check(const __grid_constant__ Ch
     check_block<K, UN, WN>(a, g, (int)blockIdx.x, (int)gridDim.x);
 }
 
-// many problems: blockIdx.y is the problem; cur, prv: which states
+// many problems: map[block] is the block's problem; cur, prv: which states
 template <int K>
-__global__ void __launch_bounds__(NTHR) k_check_many(const BatchItem *__restrict__ items, int cur, int prv)
+__global__ void __launch_bounds__(NTHR) k_check_many(const BatchItem *__restrict__ items, const int *__restrict__ map,
+                                                     int cur, int prv)
 {
-    const BatchItem &d = items[blockIdx.y];
-    cudaGridDependencySynchronize();
-    if (d.st->stop) return;
+    const BatchItem &d = items[map[blockIdx.x]];
     CheckArgs a;
     a.cur = d.S[cur];
     a.prv = d.S[prv];
@@ -541,7 +540,10 @@ __global__ void __launch_bounds__(NTHR) k_check_many(const BatchItem *__restrict
     a.strips = d.check_strips;
     a.items = d.check_items;
     const MarchOp g = d.g;
-    check_block<K, VOMT_U_L12, VOMT_W_L1>(a, g, (int)blockIdx.x, (int)gridDim.x);
+    const int block = (int)blockIdx.x - d.check_first, blocks = d.check_blocks;
+    cudaGridDependencySynchronize();
+    if (d.st->stop) return;
+    check_block<K, VOMT_U_L12, VOMT_W_L1>(a, g, block, blocks);
 }
 
 // ------------------------------------------------------------------ layouts

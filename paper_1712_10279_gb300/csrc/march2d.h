@@ -50,7 +50,7 @@ struct BatchItem {
     struct {
         int rows, strips, warps, first;      // of a pass of 1, 2, 4 iterations; its first block
     } pass[3];
-    int check_rows, check_strips, check_items;
+    int check_rows, check_strips, check_items, check_first, check_blocks;
 };
 
 constexpr int kStages[3] = {1, 2, 4};   // iterations per pass of Kernels::step
@@ -62,7 +62,7 @@ struct Kernels {
     void (*out)(const PlanarArgs, const MarchOp, const float4 *, const float4 *, const DevStatus *);
     // many problems at once (default norms, up to five channels, resident engine's order)
     void (*many[3])(const BatchItem *, const int *, int, int);
-    void (*check_many)(const BatchItem *, int, int);
+    void (*check_many)(const BatchItem *, const int *, int, int);
     void (*in_many)(const BatchItem *);
     void (*out_many)(const BatchItem *);
     int groups, bgroups;              // groups of four values of a point: state, b
