@@ -6,7 +6,10 @@
 // thread recomputes the two neighbouring shrinks from phi and u instead of
 // waiting for the threads that own them, so one launch does a whole iteration
 // and no grid-wide barrier is needed between the u/w and phi halves
-// (Section 7.4 puts a synchronisation there).
+// (Section 7.4 puts a synchronisation there).  Vector problems with four and more
+// iterations between checks take the marching form instead (march2d.cuh); these kernels
+// serve matrix fields, shorter intervals, edges not listed in the order of the pairs, the
+// allocation-free entry point and the unrolled gradient's forward pass.
 #include <math.h>
 
 #include "internal.h"
@@ -475,58 +478,33 @@ __device__ __forceinline__ void finalize(const double *__restrict__ partials, in
                                          DevStatus *st, double *hist, int hist_cap, int slot)
 {
     if (st->stop) return;
-    __shared__ double S[NRED], F[NRED];
+    __shared__ double S[NRED];
     // warp q sums slot q: lane j takes rows j, j + 32, ..., then a butterfly over
     // the lanes (a fixed order, so the same sum on every run)
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     if (q < NRED) {
         double a = 0.0;
-        // eight rows are on their way at once
-        for (int b0 = lane; b0 < nblocks; b0 += 256) {
-            double x[8];
-#pragma unroll
-            for (int r = 0; r < 8; ++r) x[r] = b0 + 32 * r < nblocks ? partials[(size_t)(b0 + 32 * r) * NRED + q] : 0.0;
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-                if (b0 + 32 * r < nblocks) a = (q == RED_MAX) ? fmax(a, x[r]) : a + x[r];
+        for (int bk = lane; bk < nblocks; bk += 32) {
+            const double x = partials[(size_t)bk * NRED + q];
+            a = (q == RED_MAX) ? fmax(a, x) : a + x;
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             const double o = __shfl_xor_sync(0xffffffffu, a, off);
             a = (q == RED_MAX) ? fmax(a, o) : a + o;
         }
-        // the quotients and roots here, one per warp: in one thread, one after the other, they
-        // took most of the 9 us that a check waited for this kernel (FP64 is slow on this GPU)
-        if (lane == 0) {
-            S[q] = a;
-            double f = 0.0;
-            if (q == RED_DIST && cfg.eps > 0.0) f = a / (4.0 * cfg.eps);
-            else if (q == RED_RR || (q == RED_BB && a > 0.0)) f = sqrt(a);
-            else if (q == RED_BB) f = 1.0;
-            else if (q == RED_DU) f = a / cfg.mu;
-            else if (q == RED_DW && cfg.has_w) f = a / cfg.nu;
-            else if (q == RED_DP) f = a / cfg.tau;
-            F[q] = f;
-        }
-    }
-    __syncthreads();
-    __shared__ double ratio[2];
-    if (threadIdx.x == 0) {
-        const double P = S[RED_P], D = S[RED_D] - F[RED_DIST];
-        ratio[0] = fabs(P - D) / fmax(fabs(P), 1e-300);
-    } else if (threadIdx.x == 32) {
-        ratio[1] = F[RED_RR] / F[RED_BB];
+        if (lane == 0) S[q] = a;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         if (t < 0) t = st->iter - t;       // in a replayed graph: the last check's iteration plus -t
-        double P = S[RED_P], D = S[RED_D] - F[RED_DIST];
+        double P = S[RED_P], D = S[RED_D] - (cfg.eps > 0.0 ? S[RED_DIST] / (4.0 * cfg.eps) : 0.0);
         double m[NMET];
         m[0] = P;
         m[1] = D;
-        m[2] = ratio[0];
-        m[3] = ratio[1];
-        m[4] = F[RED_DU] + F[RED_DW] + F[RED_DP] - 2.0 * S[RED_X];
+        m[2] = fabs(P - D) / fmax(fabs(P), 1e-300);
+        m[3] = sqrt(S[RED_RR]) / (S[RED_BB] > 0.0 ? sqrt(S[RED_BB]) : 1.0);
+        m[4] = S[RED_DU] / cfg.mu + (cfg.has_w ? S[RED_DW] / cfg.nu : 0.0) + S[RED_DP] / cfg.tau - 2.0 * S[RED_X];
         m[5] = S[RED_MAX];
         m[6] = (double)t;
         bool finite = true;
