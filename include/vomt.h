@@ -250,8 +250,9 @@ int vomt_backward(vomt_ctx *ctx, int batch, int n, int pitch, int k, int n_edges
 /* Unrolled gradient: J_T = P(u^T, w^T), the primal objective after T
  * iterations of Section 7.2 from the zero iterate (tau, mu, nu, norms from p;
  * p->u_norm must be VOMT_U_L12), and its exact gradient by reverse mode through
- * the T iterations.  The forward pass keeps the iterate every `ckpt`
- * iterations; the reverse pass recomputes each segment from its checkpoint.
+ * the T iterations.  The forward pass keeps every iterate where that takes at
+ * most 1 GiB, else one every `ckpt` iterations, and the reverse pass recomputes
+ * each segment from its checkpoint.
  * rho0, rho1: device [k][n][n].  Outputs: d_rho0, d_rho1 device [k][n][n]
  * (either may be NULL), *d_alpha and *J host (either may be NULL); every
  * derivative is multiplied by `scale`.  Returns after the work finished.
@@ -305,7 +306,11 @@ int vomt_batch_layout(int count, vomt_instance *inst, size_t *total_floats);
  *     parameters.  Needs k <= 5 and
  *     p->max_iters < 2^20 - 2 (else VOMT_ERR_TOO_LARGE).
  * VOMT_ENGINE_AUTO or VOMT_ENGINE_BATCHED: the path vomt_batch_tune found
- * faster on ctx, else the one a cost model estimates faster.
+ * faster on ctx, else the one a cost model estimates faster.  Where that is the
+ * grouped path, the norms are the defaults, eps = 0, every check is at least four
+ * iterations from the last and edges are listed in the order of their pairs, the
+ * marching form of the streaming engine takes the batch if it is estimated faster
+ * still (results[q].variant = 0, .blocks those of a pass, .halo 0; the same iterates).
  * results: host array of `count` (may be NULL); results[q].blocks is the
  * number of tiles instance q ran on and .halo its ring width.  Returns
  * VOMT_OK, VOMT_NOT_CONVERGED if some instance hit the cap, or the first error
@@ -420,8 +425,8 @@ int momt_solve_complex(vomt_ctx *ctx, int n, int k, const float *Lam0, const flo
  * (sum of the three directions' nuclear norms); w_norm as momt_solve.  Default
  * mu = 1/(48 tau (n-1)^2); user steps must satisfy tau mu 12 (n-1)^2 + tau nu
  * lambda_max(-Delta_L) < 1.  p->engine is ignored; p->halo > 0 sets the z planes
- * each block marches through.  k = 2 runs the TMA form of the step where the
- * grid allows (result->variant), k = 3 the per-thread form.
+ * each block marches through.  Both k run the TMA form of the step where the
+ * grid allows (n >= 40).
  * Errors: as momt_solve. */
 int momt_solve3d(vomt_ctx *ctx, int n, int k, const float *Lam0, const float *Lam1, int N, const double *L,
                  double alpha, const vomt_params *p, float *U, float *W, float *Phi, vomt_result *result,

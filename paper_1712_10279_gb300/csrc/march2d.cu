@@ -407,7 +407,7 @@ double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &prob
 
 // The problems of a channel count advance together, a pass over all of them per launch; a
 // problem that has stopped costs its blocks a look at its status.  Eight pairs at 256^2
-// with three channels take about 5 us per iteration together, where one after another on
+// with three channels take 5.6 us per iteration together, where one after another on
 // every SM (the grouped resident form) they take 8 x 1.6.
 int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
                 cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)

@@ -13,15 +13,15 @@
 // The neighbours that a strip and a chunk lack cost redundant work: each stage loses one
 // column on either side and one row at either end, so a warp writes 32 - 2 S columns and
 // reads S more rows on either side of its chunk.  In return one pass over memory serves S
-// iterations: 2048^2 with three channels takes 25 us per iteration at S = 4 (a pass moves
-// 0.47 GB in 100 us, 70% of the measured copy rate, the rest is issue: 0.7 instructions
-// per cycle and scheduler), where one iteration per pass with TMA tiles takes 79 us and
-// is bound by HBM alone; 1024^2 with one channel 3.4 us (was 9.2), 512^2 with eight
-// channels 21 us (118 us: the recomputed shrinks of the one-iteration kernel spill).
+// iterations: 2048^2 with three channels takes 27 us per iteration at S = 4 (a pass moves
+// 0.47 GB in 107 us, 65% of the measured copy rate, the rest is issue), where one
+// iteration per pass with TMA tiles takes 79 us and is bound by HBM alone; 1024^2 with one
+// channel 3.6 us (was 9.2), 512^2 with eight channels 22 us (118 us: the recomputed shrinks
+// of the one-iteration kernel spill).
 //
 // Every value is rounded as the one-iteration kernels (or, RES, the resident kernels) round
-// it, operation by operation (edges listed in the order of the pairs), so that the iterates are theirs bit for bit: after hundreds
-// of iterations w, which is zero except where a difference of phi passes its threshold,
+// it, operation by operation (edges listed in the order of the pairs), so that the
+// iterates are theirs bit for bit: after hundreds of iterations w, which is zero except where a difference of phi passes its threshold,
 // differs by 1e-5 and more of its norm between two roundings of phi.  The sums over
 // channels of the graph gradient reduce to the two channels of a pair (the other terms are
 // exact zeros), which keeps its matrix out of the registers.
@@ -375,6 +375,8 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march_many(const Bat
 // predecessor prv.  The same march: both states' rows once, neighbours along x by
 // shuffles, the row below carried; strips write no columns, so a strip covers 30.  Sums
 // per thread and warp in pairs of FP32 numbers (CheckAcc), per block and grid in FP64.
+// About 15 us at 1024^2 with one channel, bound by the latency of a row's loads; loading
+// a row ahead costs more in resident warps than it hides (19 us).
 template <int K, int UN, int WN>
 __device__ __forceinline__ void check_block(const CheckArgs &a, const MarchOp &g, const int block, const int blocks)
 {
