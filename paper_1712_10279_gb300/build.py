@@ -35,7 +35,8 @@ def _sources():
 
 
 def _deps():
-    return _sources() + sorted(glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "vomt.h")]
+    headers = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
+    return _sources() + sorted(headers) + [os.path.join(INCLUDE, "vomt.h")]
 
 
 def up_to_date() -> bool:
