@@ -212,6 +212,25 @@ int vomt_solve3d(vomt_ctx *ctx, int n, const float *rho0, const float *rho1,
  * number of rows available, or a negative error. */
 int vomt_history(vomt_ctx *ctx, double *out, int cap);
 
+/* The form of the kernels that the last solve or unrolled gradient on ctx ran
+ * (of those that got as far as their first step; VOMT_FORM_NONE before that and
+ * for a null ctx).  result->engine and result->variant keep their
+ * meanings; this tells apart the forms that share a value there. */
+#define VOMT_FORM_NONE           0
+#define VOMT_FORM_RESIDENT       1   /* one persistent launch, state on chip */
+#define VOMT_FORM_STEP           2   /* 2-D, one iteration per launch, per-thread loads */
+#define VOMT_FORM_STEP_TMA       3   /* 2-D, one iteration per launch, TMA tiles */
+#define VOMT_FORM_MARCH          4   /* 2-D, several iterations per pass over the grid */
+#define VOMT_FORM_STEP3          5   /* 3-D, per-thread loads */
+#define VOMT_FORM_STEP3_TMA      6   /* 3-D, TMA tiles */
+#define VOMT_FORM_STEP3_PADDED   7   /* 3-D, TMA tiles on rows padded to 16 bytes */
+#define VOMT_FORM_BATCH_QUEUE    8   /* batch, one block per problem */
+#define VOMT_FORM_BATCH_GROUPED  9   /* batch, resident waves */
+#define VOMT_FORM_BATCH_MARCH   10   /* batch, marching form */
+#define VOMT_FORM_UNROLLED_KEPT 11   /* unrolled gradient, every iterate kept */
+#define VOMT_FORM_UNROLLED_CKPT 12   /* unrolled gradient, checkpoints and recomputed segments */
+int vomt_last_form(const vomt_ctx *ctx);
+
 /* Bounded waits of the resident engine (no counterpart in the paper; a test
  * and tuning hook).  In the resident engine one thread block waits on another
  * (halo words, check rows); every such wait gives up after a time limit, then

@@ -366,6 +366,12 @@ def set_wait_policy(budget_ms: float = 0.0, drop_exchange: int = 0, device: int 
     _native.check(_native.load().vomt_set_wait_policy(ctx, float(budget_ms), int(drop_exchange)), ctx)
 
 
+def last_form(device: int = 0) -> str:
+    """The form of the kernels that the last solve or unrolled gradient on `device` ran: one
+    of _native.FORMS (vomt_last_form)."""
+    return _native.FORMS[_native.load().vomt_last_form(_native.context(device))]
+
+
 def history(device: int = 0):
     """Rows (primal, dual, rel_gap, rel_res, fp_resid, dual_infeas, iter, converged) of every
     convergence check of the last solve on `device`."""

@@ -22,6 +22,9 @@ STATUS_NAMES = {
     -9: "CUDA", -10: "TOO_LARGE",
 }
 ENGINES = {"auto": 0, "stream": 1, "resident": 2, "batched": 3}
+# VOMT_FORM_*, in their order
+FORMS = ("none", "resident", "step", "step tma", "march", "step3", "step3 tma", "step3 padded", "batch queue",
+         "batch grouped", "batch march", "unrolled kept", "unrolled checkpoints")
 ENGINE_NAMES = {v: k for k, v in ENGINES.items()}
 
 
@@ -78,6 +81,7 @@ SIGNATURES = {
     "momt_solve3d": (c_int, [c_void_p, c_int, c_int, c_void_p, c_void_p, c_int, c_void_p, c_double,
                              ctypes.POINTER(Params), c_void_p, c_void_p, c_void_p, ctypes.POINTER(Result), c_void_p]),
     "vomt_history": (c_int, [c_void_p, P_double, c_int]),
+    "vomt_last_form": (c_int, [c_void_p]),
     "vomt_set_wait_policy": (c_int, [c_void_p, c_double, c_int]),
     "vomt_backward": (c_int, [c_void_p, c_int, c_int, c_int, c_int, c_int, c_int, c_void_p, c_void_p, c_void_p,
                               c_void_p, c_void_p, c_void_p, c_void_p]),

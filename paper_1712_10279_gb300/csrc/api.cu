@@ -217,6 +217,7 @@ int run_engine(vomt_ctx *ctx, const OpDev &op, const StepDev &s, const SolveCfg 
             rc = resident_solve(ctx, op, s, cfg, p, plan, rho0, rho1, u, w, phi, st);
             if (rc == VOMT_OK) {
                 *engine = VOMT_ENGINE_RESIDENT;
+                ctx->last_form = VOMT_FORM_RESIDENT;
                 return VOMT_OK;
             }
             if (!(rc == VOMT_ERR_TOO_LARGE && p.engine == VOMT_ENGINE_AUTO)) return rc;
@@ -450,6 +451,8 @@ extern "C" int vomt_set_wait_policy(vomt_ctx *ctx, double budget_ms, int drop_ex
     ctx->drop_exchange = drop_exchange;
     return VOMT_OK;
 }
+
+int vomt_last_form(const vomt_ctx *ctx) { return ctx ? ctx->last_form : VOMT_FORM_NONE; }
 
 int vomt_history(vomt_ctx *ctx, double *out, int cap)
 {

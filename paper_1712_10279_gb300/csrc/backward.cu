@@ -518,6 +518,7 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
             ws += hp[2 * q + 1];
         }
         for (int q = 0; q < rb; ++q) ga += hp[2 * (size_t)nb + q];
+        ctx->last_form = keep ? VOMT_FORM_UNROLLED_KEPT : VOMT_FORM_UNROLLED_CKPT;
         if (J) *J = jv;
         if (d_alpha) *d_alpha = scale * (ws + ga);
         if (!isfinite(jv)) return fail(ctx, VOMT_ERR_NONFINITE, "unrolled objective is not finite");

@@ -1024,6 +1024,7 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
                 rc = grouped_solve(ctx, b, count, hinst, arena, p, waves, st, &as_graph);
                 if (rc) return rc;
             }
+            ctx->last_form = marched ? VOMT_FORM_BATCH_MARCH : VOMT_FORM_BATCH_GROUPED;
             std::vector<int> tiles(count, 1), halo(count, 0);
             for (const Wave &w : waves)
                 for (int q : w.insts) {
@@ -1115,6 +1116,7 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
         ++ctx->launches;
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch solve");
+        ctx->last_form = VOMT_FORM_BATCH_QUEUE;
         int status = VOMT_OK;
         for (int q = 0; q < count; ++q) {
             const InstStatus &h = b->hstatus[q];

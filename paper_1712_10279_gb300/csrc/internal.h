@@ -174,6 +174,7 @@ struct vomt_ctx {
     size_t pstage_bytes = 0;
     int launches = 0;                        // kernels launched by the current call
     int last_blocks = 0, last_halo = 0, last_variant = 0;      // launch shape of the current call
+    int last_form = 0;                       // VOMT_FORM_* of the last solve or gradient
     // matrix-OMT compact staging (device)
     float *mstage = nullptr;
     size_t mstage_bytes = 0;

@@ -216,6 +216,7 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
     cudaError_t e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "status reset");
     *taken = true;
+    ctx->last_form = VOMT_FORM_MARCH;
     ctx->hist_raw = false;           // k_finalize writes finished rows
     ctx->last_blocks = pass[main_pass].blocks;
 

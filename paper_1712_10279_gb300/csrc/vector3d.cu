@@ -505,6 +505,7 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     Tma3Plan *tp = tma ? tma3_plan_create(n, np, k, l, p.u_norm, p.w_norm, so[0].phi, so[1].phi, b) : nullptr;
     if (!tp && np != n) return fail(ctx, VOMT_ERR_CUDA, "tensor maps of the padded volumes");
     ctx->last_variant = tp && np == n ? 1 : 0;
+    ctx->last_form = !tp ? VOMT_FORM_STEP3 : (np == n ? VOMT_FORM_STEP3_TMA : VOMT_FORM_STEP3_PADDED);
     // z chunk: the longest of 32, 16, 8, 4 planes that still gives 1.5 blocks per SM
     // (TMA form; longer chunks amortise the pipeline fill, but fewer blocks than SMs
     // leave HBM idle; 32 measured best at 128^3 and 256^3) or four blocks per SM

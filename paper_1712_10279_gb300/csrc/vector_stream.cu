@@ -629,6 +629,7 @@ int stream_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg
         ctx->last_blocks = ((n + 63) / 64) * ((n + 15) / 16);    // the step's 64 x 16 tiles
         ctx->last_variant = 1;
     }
+    ctx->last_form = tp ? VOMT_FORM_STEP_TMA : VOMT_FORM_STEP;
     auto check = [&](int t, int cur) {
         launch_pdl(L.metrics, dim3(mblocks), blk, 0, st, si[cur], si[cur ^ 1], (const float *)b, g, s, ctx->partials,
                    (const DevStatus *)ctx->dstatus);
