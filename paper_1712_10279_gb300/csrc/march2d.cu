@@ -135,6 +135,52 @@ Pass plan_pass(int n, int k, int groups, int S, int blocks_per_sm, int sms)
     return best;
 }
 
+// How the host learns that a solve with a tolerance has stopped: each next() queues a copy of
+// the status blocks and returns the copy before it once that has arrived (nullptr: none yet,
+// or no tolerance), so the GPU always has the work queued since then to go on with.
+struct StopPoll {
+    const bool on;
+    const cudaStream_t st;
+    const DevStatus *const dev;
+    DevStatus *const host;               // pinned, 2 * count blocks
+    const int count;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    int calls = 0;
+    cudaError_t error = cudaSuccess;
+    StopPoll(bool on_, cudaStream_t s, const DevStatus *d, DevStatus *h, int n) : on(on_), st(s), dev(d), host(h), count(n)
+    {
+        for (int q = 0; q < 2 && on; ++q)
+            if (error == cudaSuccess) error = cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming);
+    }
+    ~StopPoll()
+    {
+        for (cudaEvent_t e : ev)
+            if (e) cudaEventDestroy(e);
+    }
+    const DevStatus *next()
+    {
+        if (!on || error != cudaSuccess) return nullptr;
+        const int slot = calls++ & 1;
+        error = cudaMemcpyAsync(host + (size_t)slot * count, dev, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
+        if (error == cudaSuccess) error = cudaEventRecord(ev[slot], st);
+        if (error != cudaSuccess || calls < 2) return nullptr;
+        error = cudaEventSynchronize(ev[slot ^ 1]);
+        return error == cudaSuccess ? host + (size_t)(slot ^ 1) * count : nullptr;
+    }
+};
+
+// Estimated microseconds from one check to the next, `interval` iterations and the check.
+double interval_us(const Pass (&pass)[3], int main_pass, int interval)
+{
+    const double us = pass[main_pass].stages ? pass[main_pass].us / pass[main_pass].stages : 0.0;
+    return us * interval + 8.0;
+}
+
+// Checks from one poll to the next: about 150 us of work.  A poll costs the GPU a few
+// microseconds between two kernels, and after the deciding check the work up to the second
+// next poll still runs, as empty passes of about 2 us each.
+int poll_every(double check_us) { return (int)std::min(std::max(150.0 / check_us, 1.0), 1024.0); }
+
 }  // namespace
 
 // The solve of stream_solve for vector problems.  *taken = false (and VOMT_OK) where this
@@ -260,40 +306,26 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
         ctx->launches += 2;
     };
     if (p.max_iters == 0) check(0);
-    const bool tol_mode = cfg.tol_gap > 0.0;
-    cudaEvent_t ev[2] = {nullptr, nullptr};
-    if (tol_mode)
-        for (int q = 0; q < 2; ++q) cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming);
-    const int chunk = p.check_every * ((2048 + p.check_every - 1) / p.check_every);
-    int t = 0, nchunk = 0;
+    StopPoll poll(cfg.tol_gap > 0.0, st, ctx->dstatus, ctx->hstatus, 1);
+    const int every = poll_every(interval_us(pass, main_pass, interval));
+    int since = 0;
     bool stopped = false;
-    while (t < p.max_iters && !stopped) {
-        const int end = p.max_iters - t > chunk ? t + chunk : p.max_iters;
-        while (t < end) {
-            const int m = std::min(p.check_every, p.max_iters - t);
-            run(m);
-            t += m;
-            check(t);
-        }
-        if (tol_mode) {
-            const int slot = nchunk & 1;
-            cudaMemcpyAsync(&ctx->hstatus[slot], ctx->dstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st);
-            cudaEventRecord(ev[slot], st);
-            if (nchunk >= 1) {
-                // the previous chunk's flag: the GPU keeps running the chunk just queued
-                cudaEventSynchronize(ev[slot ^ 1]);
-                if (ctx->hstatus[slot ^ 1].stop) stopped = true;
-            }
-            ++nchunk;
-        }
+    for (int t = 0; t < p.max_iters && !stopped;) {
+        const int m = std::min(p.check_every, p.max_iters - t);
+        run(m);
+        t += m;
+        check(t);
+        if (++since < every) continue;
+        since = 0;
+        const DevStatus *h = poll.next();
+        stopped = poll.error != cudaSuccess || (h && h->stop);
     }
     K.out<<<lgrid, 128, 0, st>>>(planar, op, S[0], S[1], ctx->dstatus);
     ctx->launches += 1;
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = poll.error;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&ctx->hstatus[0], ctx->dstatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    for (int q = 0; q < 2; ++q)
-        if (ev[q]) cudaEventDestroy(ev[q]);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "solve");
     return VOMT_OK;
 }
