@@ -4,6 +4,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 
 #include "internal.h"
@@ -187,6 +188,39 @@ void fill_result(vomt_ctx *ctx, const SolveCfg &cfg, int engine, vomt_result *r,
     }
 }
 
+// Least iterations between checks from which the marching form of the streaming engine is
+// faster than the resident plan (0: never).  Plans with four points per thread (two from five
+// channels on) spill, and rings of one cell (two from three channels on) exchange too often,
+// so an iteration is faster in the marching form there (us, k = 1, 352^2: 1.50 against 1.95;
+// k = 3, 352^2: 2.25 against 3.85, 512^2: 3.3 against 8.3; k = 8, 256^2: 7.4 against 9.6) and
+// slower short of it (k = 3, 288^2: 1.94 against 1.76).  A check costs it 13 to 29 us, the
+// resident engine 8 to 17 (62 at k = 8, 256^2), so the less an iteration gains, the more of
+// them a check has to serve.  The lines are where both took the same time in solves of 200
+// iterations, at 13 intervals from 1 to 100 and 6 to 10 sizes per channel count (marching over
+// resident at intervals of 4, 20, 100: k = 1, 380^2 1.16, 1.01, 0.93, 470^2 1.28, 1.08, 0.97;
+// k = 3, 336^2 1.43, 1.09, 0.98, 352^2 1.05, 0.75, 0.67; k = 5, 240^2 1.43, 1.13, 1.05, 256^2
+// 1.14, 1.04, 0.98, 300^2 0.62, 0.57, 0.54; k = 6, 200^2 1.15, 0.95, 0.89; k = 7, 230^2 1.12,
+// 1.06, 1.03, 256^2 0.69, 0.90, 0.93).
+static int march_from(int k, const ResidentPlan &plan)
+{
+    const int H = plan.Gx * plan.Gy > 1 ? plan.H : 1 << 30;
+    if (k <= 2) {
+        if (H == 1) return 8;
+        if (plan.P <= 2) return 0;
+        return k == 1 && plan.threads > 384 ? 50 : 20;
+    }
+    if (k <= 4) {
+        if (plan.P > 2) return 4;
+        if (H == 1) return k == 3 ? 8 : 4;
+        return H == 2 ? (k == 3 ? 100 : 16) : 0;
+    }
+    if (plan.P == 1) return 0;
+    if (plan.P > 2 || k == 8) return 1;
+    if (H <= 2) return k == 5 ? 12 : (k == 6 ? 4 : 1);
+    if (H == 3) return k == 5 ? 20 : (k == 6 ? 8 : 1);
+    return k == 6 ? 50 : 0;
+}
+
 // Resident engine when the plan fits (AUTO / RESIDENT), else the streaming engine.
 int run_engine(vomt_ctx *ctx, const OpDev &op, const StepDev &s, const SolveCfg &cfg, const vomt_params &p,
                const float *rho0, const float *rho1, float *u, float *w, float *phi, cudaStream_t st, int *engine)
@@ -199,17 +233,12 @@ int run_engine(vomt_ctx *ctx, const OpDev &op, const StepDev &s, const SolveCfg 
     if (p.engine != VOMT_ENGINE_STREAM) {
         ResidentPlan plan;
         if (resident_plan(s.n, op.k, ctx->sm_count, p.halo, &plan)) {
-            // Tiles of four points per thread (two from five channels on) spill, and rings of one
-            // cell (two from three channels on) exchange too often; the marching form of the
-            // streaming engine is faster there (us per iteration, k = 1, 352^2: 1.50 against
-            // 1.95; k = 3, 320^2: 2.18 against 2.33, 352^2: 2.25 against 3.85, 512^2: 3.3 against
-            // 8.3; k = 4, 320^2: 3.0 against 3.7; k = 5, 256^2: 3.56 against 3.65; k = 8, 256^2:
-            // 7.4 against 9.6) and slower short of it (k = 1, 320^2: 1.48 against 1.30; k = 3,
-            // 288^2: 1.94 against 1.76; k = 8, 128^2: 5.3 against 3.4).  A ring width asked for
-            // asks for the resident engine.  For the default norms the marching kernels exist in
-            // the resident kernels' order of operations, so results stay what they were.
+            // A ring width asked for asks for the resident engine.  For the default norms the
+            // marching kernels exist in the resident kernels' order of operations, so results stay
+            // what they were.
+            const int from = march_from(op.k, plan);
             if (p.engine == VOMT_ENGINE_AUTO && p.halo == 0 && p.u_norm == VOMT_U_L12 && p.w_norm == VOMT_W_L1 && !s.reg &&
-                (plan.P > (op.k <= 4 ? 2 : 1) || (plan.Gx * plan.Gy > 1 && plan.H <= (op.k <= 2 ? 1 : 2)))) {
+                from > 0 && std::min(p.check_every, p.max_iters) >= from) {
                 bool taken = false;
                 rc = march_solve(ctx, op, s, cfg, p, true, rho0, rho1, u, w, phi, st, &taken);
                 if (rc || taken) return rc;

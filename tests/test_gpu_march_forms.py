@@ -112,7 +112,7 @@ def test_auto_marches_with_the_resident_results(k):
     """Past the sizes that the resident engine is good at, AUTO's marching form (in the resident
     engine's order of operations) returns that engine's iterates bit for bit, with costs and
     missing pairs too."""
-    n = {1: 400, 2: 352, 3: 340, 4: 322, 5: 260, 6: 230, 7: 210, 8: 200}[k]
+    n = {1: 400, 2: 352, 3: 340, 4: 322, 5: 260, 6: 256, 7: 256, 8: 200}[k]
     edges, cost = _graph(np.random.default_rng(k + 40), k)
     r0, r1 = _fields(n, k, n)
     kw = dict(max_iters=47, check_every=20, tau=0.7, cost=cost)
