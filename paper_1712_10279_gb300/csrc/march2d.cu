@@ -135,51 +135,62 @@ Pass plan_pass(int n, int k, int groups, int S, int blocks_per_sm, int sms)
     return best;
 }
 
-// How the host learns that a solve with a tolerance has stopped: each next() queues a copy of
-// the status blocks and returns the copy before it once that has arrived (nullptr: none yet,
-// or no tolerance), so the GPU always has the work queued since then to go on with.
+// How the host learns that a solve with a tolerance has stopped.  After a check it queues a
+// copy of the status blocks, goes on queueing work, and reads the copy once another kLead
+// microseconds of work (by the passes' estimates) are queued behind it, so that the GPU has
+// work while the host waits; after the deciding check no more than that runs, as empty
+// passes of under 2 us.  A copy takes the GPU a few microseconds between two kernels: one
+// after the first check, then at growing distances, kGap at most.
 struct StopPoll {
+    static constexpr double kLead = 80.0, kGap = 150.0;
     const bool on;
     const cudaStream_t st;
     const DevStatus *const dev;
-    DevStatus *const host;               // pinned, 2 * count blocks
+    DevStatus *const host;               // pinned, `count` blocks
     const int count;
-    cudaEvent_t ev[2] = {nullptr, nullptr};
-    int calls = 0;
+    cudaEvent_t ev = nullptr;
+    bool pending = false;
+    double clock = 0.0, collect_at = 0.0, due = 0.0, gap = 10.0;
     cudaError_t error = cudaSuccess;
     StopPoll(bool on_, cudaStream_t s, const DevStatus *d, DevStatus *h, int n) : on(on_), st(s), dev(d), host(h), count(n)
     {
-        for (int q = 0; q < 2 && on; ++q)
-            if (error == cudaSuccess) error = cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming);
+        if (on) error = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     }
     ~StopPoll()
     {
-        for (cudaEvent_t e : ev)
-            if (e) cudaEventDestroy(e);
+        if (ev) cudaEventDestroy(ev);
     }
-    const DevStatus *next()
+    void queued(double us) { clock += us; }
+    void checked()                       // a check has been queued
     {
-        if (!on || error != cudaSuccess) return nullptr;
-        const int slot = calls++ & 1;
-        error = cudaMemcpyAsync(host + (size_t)slot * count, dev, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
-        if (error == cudaSuccess) error = cudaEventRecord(ev[slot], st);
-        if (error != cudaSuccess || calls < 2) return nullptr;
-        error = cudaEventSynchronize(ev[slot ^ 1]);
-        return error == cudaSuccess ? host + (size_t)(slot ^ 1) * count : nullptr;
+        clock += kCheckUs;
+        if (!on || pending || clock < due || error != cudaSuccess) return;
+        error = cudaMemcpyAsync(host, dev, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
+        if (error == cudaSuccess) error = cudaEventRecord(ev, st);
+        pending = error == cudaSuccess;
+        collect_at = clock + kLead;
+        due = clock + gap;
+        gap = std::min(2.0 * gap, kGap);
     }
+    const DevStatus *arrived()           // the status of the last copy, once it is time to read it
+    {
+        if (!pending || clock < collect_at) return nullptr;
+        pending = false;
+        error = cudaEventSynchronize(ev);
+        return error == cudaSuccess ? host : nullptr;
+    }
+    static constexpr double kCheckUs = 12.0;
 };
 
-// Estimated microseconds from one check to the next, `interval` iterations and the check.
-double interval_us(const Pass (&pass)[3], int main_pass, int interval)
+// The pass to launch next, m iterations before a check: fewer-stage passes first.
+int next_pass(const Pass (&pass)[3], int main_pass, int m)
 {
-    const double us = pass[main_pass].stages ? pass[main_pass].us / pass[main_pass].stages : 0.0;
-    return us * interval + 8.0;
+    const int odd = m % kStages[main_pass];
+    if (odd == 0) return main_pass;
+    int r = main_pass - 1;
+    while (r > 0 && (!pass[r].stages || odd < kStages[r])) --r;
+    return r;
 }
-
-// Checks from one poll to the next: about 150 us of work.  A poll costs the GPU a few
-// microseconds between two kernels, and after the deciding check the work up to the second
-// next poll still runs, as empty passes of about 2 us each.
-int poll_every(double check_us) { return (int)std::min(std::max(150.0 / check_us, 1.0), 1024.0); }
 
 }  // namespace
 
@@ -289,13 +300,6 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
         before = a.prev ? a.prev : a.in;
         cur ^= 1;
     };
-    // m iterations, fewer-stage passes first
-    auto run = [&](int m) {
-        int q = main_pass, odd = m % kStages[q];
-        for (int r = q - 1; r >= 0; --r)
-            for (; pass[r].stages && odd >= kStages[r]; odd -= kStages[r], m -= kStages[r]) one(r, m == kStages[r]);
-        for (; m > 0; m -= kStages[q]) one(q, m == kStages[q]);
-    };
     auto check = [&](int t) {
         CheckArgs c = ca;
         c.cur = S[cur];
@@ -307,18 +311,24 @@ int march_solve(vomt_ctx *ctx, const OpDev &g, const StepDev &s, const SolveCfg 
     };
     if (p.max_iters == 0) check(0);
     StopPoll poll(cfg.tol_gap > 0.0, st, ctx->dstatus, ctx->hstatus, 1);
-    const int every = poll_every(interval_us(pass, main_pass, interval));
-    int since = 0;
-    bool stopped = false;
-    for (int t = 0; t < p.max_iters && !stopped;) {
-        const int m = std::min(p.check_every, p.max_iters - t);
-        run(m);
-        t += m;
+    auto stopped = [&]() {
+        const DevStatus *h = poll.arrived();
+        return poll.error != cudaSuccess || (h && h->stop);
+    };
+    bool stop = false;
+    for (int t = 0; t < p.max_iters && !stop;) {
+        for (int m = std::min(p.check_every, p.max_iters - t); m > 0 && !stop;) {
+            const int q = next_pass(pass, main_pass, m);
+            one(q, m == kStages[q]);
+            m -= kStages[q];
+            t += kStages[q];
+            poll.queued(pass[q].us);
+            stop = stopped();
+        }
+        if (stop) break;
         check(t);
-        if (++since < every) continue;
-        since = 0;
-        const DevStatus *h = poll.next();
-        stopped = poll.error != cudaSuccess || (h && h->stop);
+        poll.checked();
+        stop = stopped();
     }
     K.out<<<lgrid, 128, 0, st>>>(planar, op, S[0], S[1], ctx->dstatus);
     ctx->launches += 1;
@@ -349,15 +359,26 @@ namespace {
 // the loads of a row (8 x 256^2, three channels: 140 us with 8 blocks a problem, 30 so).
 int check_chunk(long strip_rows, int sms) { return (int)std::max(2l, (strip_rows + 16l * sms - 1) / (16l * sms)); }
 
-// The problems of one channel count: passes over all of them at once, with chunks of the
-// same number of rows in every problem.
+// The problems of one channel count: passes over those still running at once, with chunks of
+// the same number of rows in every problem.
 struct Group {
     int k = 0, main_pass = 0;
-    std::vector<int> probs;
+    std::vector<int> probs, live;     // all its problems; those the passes below are planned for
     Kernels K;
+    int per_sm[3] = {0, 0, 0};
     Pass pass[3];                     // blocks: of the whole group
     int check_rows = 2, check_blocks = 0;
+    int first_live = 0;               // its first item of the pass tables
+    size_t map_at[4] = {0, 0, 0, 0};  // block maps of its three passes and its check
+    int cur = 0, before = 0;          // states that hold the iterates and their predecessors
 };
+
+double points(const std::vector<BatchProblem> &probs, const std::vector<int> &which)
+{
+    double pts = 0.0;
+    for (int q : which) pts += (double)probs[q].g.n * probs[q].g.n;
+    return pts;
+}
 
 // plan_pass for a group: the chunk length of the least arithmetic time
 Pass plan_group(const std::vector<BatchProblem> &probs, const Group &gr, int S, int blocks_per_sm, int sms)
@@ -366,15 +387,11 @@ Pass plan_group(const std::vector<BatchProblem> &probs, const Group &gr, int S, 
     const double issue = 20.0 + 40.0 * k + 4.0 * k * (k - 1), lat = 180.0, ghz = 1.95;
     const long cap = (long)blocks_per_sm * sms;
     int top = 0;
-    double pts = 0.0;
-    for (int q : gr.probs) {
-        top = std::max(top, probs[q].g.n);
-        pts += (double)probs[q].g.n * probs[q].g.n;
-    }
+    for (int q : gr.live) top = std::max(top, probs[q].g.n);
     Pass best;
     for (int rows = 1; rows <= top; rows += rows < 32 ? 1 : rows / 16) {
         long blocks = 0, warps = 0;
-        for (int q : gr.probs) {
+        for (int q : gr.live) {
             const int n = probs[q].g.n;
             const long w = (long)((n + W - 1) / W) * ((n + rows - 1) / rows);
             warps += w;
@@ -387,9 +404,28 @@ Pass plan_group(const std::vector<BatchProblem> &probs, const Group &gr, int S, 
         const double us = cycles * S * (rows + 2 * S) / (ghz * 1e3);
         if (best.stages == 0 || us < best.us) best = Pass{S, rows, 0, (int)warps, (int)blocks, us};
     }
-    const double mb = 16e-6 * pts * (2 * gr.K.groups + (k + 3) / 4);
+    const double mb = 16e-6 * points(probs, gr.live) * (2 * gr.K.groups + (k + 3) / 4);
     best.us = 3.5 + std::max(best.us, mb / (mb > 110.0 ? 6.3 : 12.0));
     return best;
+}
+
+// The passes and the check of a group's live problems.
+void plan_live(const std::vector<BatchProblem> &probs, Group &g, int interval, int sms)
+{
+    g.main_pass = 0;
+    for (int q = 0; q < 3; ++q) {
+        if (g.per_sm[q] < 1) continue;
+        Pass &ps = g.pass[q];
+        ps = plan_group(probs, g, kStages[q], g.per_sm[q], sms);
+        const int share = (ps.blocks + sms - 1) / sms;      // see march_solve
+        ps.smem = std::max(g.K.smem, kSmemSM / (share + 1));
+        if (kStages[q] <= interval && (g.pass[g.main_pass].stages == 0 ||
+                                       ps.us / kStages[q] < g.pass[g.main_pass].us / kStages[g.main_pass]))
+            g.main_pass = q;
+    }
+    long strip_rows = 0;
+    for (int q : g.live) strip_rows += (long)((probs[q].g.n + 29) / 30) * probs[q].g.n;
+    g.check_rows = check_chunk(strip_rows, sms);
 }
 
 int plan_groups(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p, std::vector<Group> *out)
@@ -402,121 +438,43 @@ int plan_groups(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vom
         for (int q = 0; q < (int)probs.size(); ++q)
             if (probs[q].k == k) g.probs.push_back(q);
         if (g.probs.empty()) continue;
+        g.live = g.probs;
         g.K = pick(k, VOMT_U_L12, VOMT_W_L1, false, true);
         for (int q = 0; q < 3; ++q) {
             if (!g.K.many[q]) continue;
-            int per_sm = 0;
             cudaError_t e = cudaFuncSetAttribute((const void *)g.K.many[q], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  kSmemBlock);
             if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)g.K.many[q], 32 * kWarps,
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.per_sm[q], (const void *)g.K.many[q], 32 * kWarps,
                                                                   g.K.smem);
             if (e != cudaSuccess) return set_cuda_error(ctx, e, "marching kernel");
-            if (per_sm < 1) continue;
-            Pass &ps = g.pass[q];
-            ps = plan_group(probs, g, kStages[q], per_sm, ctx->sm_count);
-            const int share = (ps.blocks + ctx->sm_count - 1) / ctx->sm_count;      // see march_solve
-            ps.smem = std::max(g.K.smem, kSmemSM / (share + 1));
-            if (kStages[q] <= interval && (g.pass[g.main_pass].stages == 0 ||
-                                           ps.us / kStages[q] < g.pass[g.main_pass].us / kStages[g.main_pass]))
-                g.main_pass = q;
         }
-        if (g.pass[0].stages == 0) return VOMT_ERR_TOO_LARGE;
+        if (g.per_sm[0] < 1) return VOMT_ERR_TOO_LARGE;
+        plan_live(probs, g, interval, ctx->sm_count);
         out->push_back(g);
     }
     return VOMT_OK;
 }
 
-}  // namespace
-
-double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p)
-{
-    std::vector<Group> groups;
-    if (plan_groups(ctx, probs, p, &groups)) return 1e30;
-    double us = 0.0;
-    for (const Group &g : groups) us += g.pass[g.main_pass].us / kStages[g.main_pass];
-    return us;
-}
-
-// The problems of a channel count advance together, a pass over all of them per launch; a
-// problem that has stopped costs its blocks a look at its status.  Eight pairs at 256^2
-// with three channels take 5.6 us per iteration together, where one after another on
-// every SM (the grouped resident form) they take 8 x 1.6.
-int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
-                cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)
-{
-    *taken = false;
-    const int count = (int)probs.size();
-    if (count > 65535) return VOMT_OK;                // a launch's third dimension
-    std::vector<Group> groups;
-    int rc = plan_groups(ctx, probs, p, &groups);
-    if (rc) return rc == VOMT_ERR_TOO_LARGE ? VOMT_OK : rc;
-    // scratch: per problem b, two states, the state before a check; check sums; tables
-    std::vector<BatchItem> items(count);
-    std::vector<int> maps, slot_of(count);            // items are stored group by group
-    size_t floats4 = 0;
-    std::vector<size_t> off(count);
-    for (const Group &g : groups)
-        for (int q : g.probs) {
-            const size_t tile = (size_t)probs[q].g.n * ((probs[q].g.n + 31) / 32) * 32;
-            off[q] = floats4;
-            floats4 += tile * (3 * (size_t)g.K.groups + g.K.bgroups);
-        }
+// Pass tables of the live problems, group by group: an item each and, per pass and check,
+// the problem of every block.  Fills the groups' places in them.
+struct Tables {
+    std::vector<BatchItem> items;
+    std::vector<int> maps;
     size_t sum_rows = 0;
+};
+Tables build_tables(const std::vector<BatchProblem> &probs, std::vector<Group> &groups,
+                    const std::vector<BatchItem> &base, const std::vector<int> &slot_of, double *sums,
+                    std::vector<int> *blocks)
+{
+    Tables t;
     for (Group &g : groups) {
-        long strip_rows = 0;
-        for (int q : g.probs) strip_rows += (long)((probs[q].g.n + 29) / 30) * probs[q].g.n;
-        g.check_rows = check_chunk(strip_rows, ctx->sm_count);
-        g.check_blocks = 0;
-        for (int q : g.probs) {
-            const int n = probs[q].g.n, items = (n + 29) / 30 * ((n + g.check_rows - 1) / g.check_rows);
-            g.check_blocks += (items + kWarps - 1) / kWarps;
-        }
-        sum_rows += g.check_blocks;
-    }
-    const size_t sums = sizeof(double) * NRED * sum_rows;
-    rc = ensure_buffer(ctx, &scr->data, &scr->data_cap, sizeof(float4) * floats4 + sums, "batch states");
-    if (rc) {
-        ctx->err.clear();
-        return VOMT_OK;
-    }
-    rc = ensure_buffer(ctx, &scr->items, &scr->items_cap, sizeof(BatchItem) * count, "batch tables");
-    if (!rc) rc = ensure_buffer(ctx, &scr->stat, &scr->stat_cap, sizeof(DevStatus) * count, "batch status");
-    if (rc) return rc;
-    if (scr->hstat_cap < 2 * sizeof(DevStatus) * count) {
-        if (scr->hstat) cudaFreeHost(scr->hstat);
-        scr->hstat = nullptr;
-        scr->hstat_cap = 0;
-        cudaError_t e = cudaMallocHost(&scr->hstat, 2 * sizeof(DevStatus) * count);
-        if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch status");
-        scr->hstat_cap = 2 * sizeof(DevStatus) * count;
-    }
-    float4 *data = (float4 *)scr->data;
-    double *dsums = (double *)(data + floats4);
-    DevStatus *dstat = (DevStatus *)scr->stat, *hstat = (DevStatus *)scr->hstat;
-    blocks->assign(count, 1);
-    int at = 0;
-    size_t sum_at = 0;
-    std::vector<size_t> map_at(groups.size() * 4, 0);      // of its three passes and its check
-    std::vector<int> first_item(groups.size()), top(groups.size(), 0);
-    for (size_t gi = 0; gi < groups.size(); ++gi) {
-        const Group &g = groups[gi];
-        first_item[gi] = at;
         int next[4] = {0, 0, 0, 0};
         std::vector<int> gm[4];
-        for (size_t i = 0; i < g.probs.size(); ++i, ++at) {
-            const int q = g.probs[i], n = probs[q].g.n;
-            const size_t tile = (size_t)n * ((n + 31) / 32) * 32;
-            BatchItem &d = items[at];
-            memset(&d, 0, sizeof d);
-            d.g = probs[q].g;
-            d.g.g1 = 1.0f;
-            d.g.g2 = d.g.mu * d.g.ih;
-            d.cfg = probs[q].cfg;
-            d.planar = probs[q].planar;
-            d.b = data + off[q];
-            for (int c = 0; c < 3; ++c) d.S[c] = d.b + tile * (g.K.bgroups + (size_t)c * g.K.groups);
-            d.st = dstat + at;
+        g.first_live = (int)t.items.size();
+        for (size_t i = 0; i < g.live.size(); ++i) {
+            const int q = g.live[i], n = probs[q].g.n;
+            BatchItem d = base[slot_of[q]];
             for (int c = 0; c < 3; ++c) {
                 if (!g.pass[c].stages) continue;
                 const int W = 32 - 2 * kStages[c];
@@ -534,28 +492,127 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
             d.check_items = d.check_strips * ((n + d.check_rows - 1) / d.check_rows);
             d.check_blocks = (d.check_items + kWarps - 1) / kWarps;
             d.check_first = next[3];
-            d.partials = dsums + (sum_at + next[3]) * NRED;
+            d.partials = sums + (t.sum_rows + next[3]) * NRED;
             gm[3].insert(gm[3].end(), d.check_blocks, (int)i);
             next[3] += d.check_blocks;
-            slot_of[q] = at;
-            top[gi] = std::max(top[gi], n);
+            t.items.push_back(d);
         }
         for (int c = 0; c < 4; ++c) {
-            map_at[gi * 4 + c] = maps.size();
-            maps.insert(maps.end(), gm[c].begin(), gm[c].end());
-            if (c < 3) groups[gi].pass[c].blocks = next[c];
+            g.map_at[c] = t.maps.size();
+            t.maps.insert(t.maps.end(), gm[c].begin(), gm[c].end());
+            if (c < 3) g.pass[c].blocks = next[c];
         }
-        sum_at += next[3];
+        g.check_blocks = next[3];
+        t.sum_rows += next[3];
     }
-    rc = ensure_buffer(ctx, &scr->maps, &scr->maps_cap, sizeof(int) * maps.size(), "batch tables");
+    return t;
+}
+
+}  // namespace
+
+double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p)
+{
+    std::vector<Group> groups;
+    if (plan_groups(ctx, probs, p, &groups)) return 1e30;
+    double us = 0.0;
+    for (const Group &g : groups) us += g.pass[g.main_pass].us / kStages[g.main_pass];
+    return us;
+}
+
+// The problems of a channel count advance together, a pass over all of them per launch.
+// Eight pairs at 256^2 with three channels take 5.6 us per iteration together, where one
+// after another on every SM (the grouped resident form) they take 8 x 1.6.  A problem that
+// has stopped still costs its blocks the copies of a chunk's first rows, and the chunks of
+// the others stay as long as they were planned with it, so when a quarter of a group's points
+// has stopped, its passes are planned again for the problems left.
+int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
+                cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)
+{
+    *taken = false;
+    const int count = (int)probs.size(), sms = ctx->sm_count;
+    if (count > 65535) return VOMT_OK;                // a launch's third dimension
+    std::vector<Group> groups;
+    int rc = plan_groups(ctx, probs, p, &groups);
+    if (rc) return rc == VOMT_ERR_TOO_LARGE ? VOMT_OK : rc;
+    // scratch: per problem b, two states, the state before a check; check sums (rows for any
+    // subset of the problems: check_chunk gives 16 warps per SM, a partly filled chunk per
+    // strip and a partly filled block per problem); tables
+    size_t floats4 = 0, sum_rows = 0;
+    std::vector<size_t> off(count);
+    for (const Group &g : groups) {
+        size_t strips = 0;
+        for (int q : g.probs) {
+            const size_t n = probs[q].g.n, tile = n * ((n + 31) / 32) * 32;
+            off[q] = floats4;
+            floats4 += tile * (3 * (size_t)g.K.groups + g.K.bgroups);
+            strips += (n + 29) / 30;
+        }
+        sum_rows += (16 * (size_t)sms + strips) / kWarps + g.probs.size() + 1;
+    }
+    const size_t sums = sizeof(double) * NRED * sum_rows;
+    rc = ensure_buffer(ctx, &scr->data, &scr->data_cap, sizeof(float4) * floats4 + sums, "batch states");
+    if (rc) {
+        ctx->err.clear();
+        return VOMT_OK;
+    }
+    rc = ensure_buffer(ctx, &scr->items, &scr->items_cap, 2 * sizeof(BatchItem) * count, "batch tables");
+    if (!rc) rc = ensure_buffer(ctx, &scr->stat, &scr->stat_cap, sizeof(DevStatus) * count, "batch status");
     if (rc) return rc;
-    cudaError_t e = cudaMemcpyAsync(scr->items, items.data(), sizeof(BatchItem) * count, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(scr->maps, maps.data(), sizeof(int) * maps.size(), cudaMemcpyHostToDevice, st);
+    if (scr->hstat_cap < 2 * sizeof(DevStatus) * count) {
+        if (scr->hstat) cudaFreeHost(scr->hstat);
+        scr->hstat = nullptr;
+        scr->hstat_cap = 0;
+        cudaError_t e = cudaMallocHost(&scr->hstat, 2 * sizeof(DevStatus) * count);
+        if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch status");
+        scr->hstat_cap = 2 * sizeof(DevStatus) * count;
+    }
+    float4 *data = (float4 *)scr->data;
+    double *dsums = (double *)(data + floats4);
+    DevStatus *dstat = (DevStatus *)scr->stat, *hstat = (DevStatus *)scr->hstat;
+    // what does not depend on the passes, all problems group by group
+    std::vector<BatchItem> base(count);
+    std::vector<int> slot_of(count), first_item(groups.size()), top(groups.size(), 0);
+    int at = 0;
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+        const Group &g = groups[gi];
+        first_item[gi] = at;
+        for (int q : g.probs) {
+            const int n = probs[q].g.n;
+            const size_t tile = (size_t)n * ((n + 31) / 32) * 32;
+            BatchItem &d = base[at];
+            memset(&d, 0, sizeof d);
+            d.g = probs[q].g;
+            d.g.g1 = 1.0f;
+            d.g.g2 = d.g.mu * d.g.ih;
+            d.cfg = probs[q].cfg;
+            d.planar = probs[q].planar;
+            d.b = data + off[q];
+            for (int c = 0; c < 3; ++c) d.S[c] = d.b + tile * (g.K.bgroups + (size_t)c * g.K.groups);
+            d.st = dstat + at;
+            slot_of[q] = at++;
+            top[gi] = std::max(top[gi], n);
+        }
+    }
+    blocks->assign(count, 1);
+    std::vector<Tables> plans;           // kept until the copies from them are done
+    plans.push_back(build_tables(probs, groups, base, slot_of, dsums, blocks));
+    // (room for the maps of a later plan: blocks of up to a wave more per pass and check)
+    rc = ensure_buffer(ctx, &scr->maps, &scr->maps_cap,
+                       sizeof(int) * (plans[0].maps.size() + 4 * 8 * (size_t)sms * groups.size()), "batch tables");
+    if (rc) return rc;
+    BatchItem *const ditems = (BatchItem *)scr->items, *const dlive = ditems + count;
+    int *const dmaps = (int *)scr->maps;
+    auto upload = [&]() {
+        const Tables &t = plans.back();
+        cudaError_t r = cudaMemcpyAsync(dlive, t.items.data(), sizeof(BatchItem) * t.items.size(), cudaMemcpyHostToDevice, st);
+        return r != cudaSuccess ? r : cudaMemcpyAsync(dmaps, t.maps.data(), sizeof(int) * t.maps.size(),
+                                                      cudaMemcpyHostToDevice, st);
+    };
+    cudaError_t e = cudaMemcpyAsync(ditems, base.data(), sizeof(BatchItem) * count, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = upload();
     if (e == cudaSuccess) e = cudaMemsetAsync(dstat, 0, sizeof(DevStatus) * count, st);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch tables");
     *taken = true;
-    const BatchItem *ditems = (const BatchItem *)scr->items;
-    const int *dmaps = (const int *)scr->maps;
     auto layout_grid = [&](size_t gi) {
         return dim3((top[gi] + 127) / 128, std::min(top[gi], 256), (unsigned)groups[gi].probs.size());
     };
@@ -563,73 +620,87 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
         groups[gi].K.in_many<<<layout_grid(gi), 128, 0, st>>>(ditems + first_item[gi]);
         ctx->launches += 1;
     }
-    std::vector<int> cur(groups.size(), 0), before(groups.size(), 0);
-    auto one = [&](size_t gi, int q, bool last) {
-        const Group &g = groups[gi];
+    auto one = [&](Group &g, int q, bool last) {
         const int prev = last && kStages[q] > 1 ? 1 : 0;
         launch_pdl(g.K.many[q], dim3(g.pass[q].blocks), dim3(32 * kWarps), (size_t)g.pass[q].smem, st,
-                   ditems + first_item[gi], dmaps + map_at[gi * 4 + q], cur[gi], prev);
+                   (const BatchItem *)dlive + g.first_live, (const int *)dmaps + g.map_at[q], g.cur, prev);
         ctx->launches += 1;
-        before[gi] = prev ? 2 : cur[gi];
-        cur[gi] ^= 1;
+        g.before = prev ? 2 : g.cur;
+        g.cur ^= 1;
     };
-    auto advance = [&](size_t gi, int m) {        // m iterations, fewer-stage passes first
-        const Group &g = groups[gi];
-        const int q = g.main_pass;
-        int odd = m % kStages[q];
-        for (int r = q - 1; r >= 0; --r)
-            for (; g.pass[r].stages && odd >= kStages[r]; odd -= kStages[r], m -= kStages[r]) one(gi, r, m == kStages[r]);
-        for (; m > 0; m -= kStages[q]) one(gi, q, m == kStages[q]);
-    };
-    auto check = [&](size_t gi, int t) {
-        const Group &g = groups[gi];
-        const unsigned np = (unsigned)g.probs.size();
-        launch_pdl(g.K.check_many, dim3(g.check_blocks), dim3(32 * kWarps), 0, st, ditems + first_item[gi],
-                   dmaps + map_at[gi * 4 + 3], cur[gi], before[gi]);
-        launch_pdl(k_finalize_many, dim3(np), dim3(kFinThreads), 0, st, ditems + first_item[gi], t, cur[gi]);
+    auto check = [&](Group &g, int t) {
+        launch_pdl(g.K.check_many, dim3(g.check_blocks), dim3(32 * kWarps), 0, st, (const BatchItem *)dlive + g.first_live,
+                   (const int *)dmaps + g.map_at[3], g.cur, g.before);
+        launch_pdl(k_finalize_many, dim3((unsigned)g.live.size()), dim3(kFinThreads), 0, st,
+                   (const BatchItem *)dlive + g.first_live, t, g.cur);
         ctx->launches += 2;
     };
     if (p.max_iters == 0)
-        for (size_t gi = 0; gi < groups.size(); ++gi) check(gi, 0);
-    const bool tol_mode = p.tol_gap > 0.0;
-    cudaEvent_t ev[2] = {nullptr, nullptr};
-    if (tol_mode)
-        for (int q = 0; q < 2; ++q) cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming);
-    const int chunk = p.check_every * ((2048 + p.check_every - 1) / p.check_every);
-    int t = 0, nchunk = 0;
-    bool stopped = false;
-    while (t < p.max_iters && !stopped) {
-        const int end = p.max_iters - t > chunk ? t + chunk : p.max_iters;
-        while (t < end) {
-            const int m = std::min(p.check_every, p.max_iters - t);
-            t += m;
-            for (size_t gi = 0; gi < groups.size(); ++gi) {
-                advance(gi, m);
-                check(gi, t);
-            }
+        for (Group &g : groups) check(g, 0);
+    StopPoll poll(p.tol_gap > 0.0, st, dstat, hstat, count);
+    const int interval = std::max(1, std::min(p.check_every, p.max_iters));
+    // plan the passes again for the problems that run on, where enough have stopped
+    auto thin_out = [&](const DevStatus *h) -> cudaError_t {
+        std::vector<std::vector<int>> live(groups.size());
+        bool again = false;
+        for (size_t gi = 0; gi < groups.size(); ++gi) {
+            for (int q : groups[gi].live)
+                if (!h[slot_of[q]].stop) live[gi].push_back(q);
+            again = again || points(probs, live[gi]) < 0.75 * points(probs, groups[gi].live);
         }
-        if (tol_mode) {
-            const int slot = nchunk & 1;
-            cudaMemcpyAsync(hstat + (size_t)slot * count, dstat, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
-            cudaEventRecord(ev[slot], st);
-            if (nchunk >= 1) {
-                // the previous chunk's flags: the GPU keeps running the chunk just queued
-                cudaEventSynchronize(ev[slot ^ 1]);
-                stopped = true;
-                for (int q = 0; q < count; ++q) stopped = stopped && hstat[(size_t)(slot ^ 1) * count + q].stop;
-            }
-            ++nchunk;
+        if (!again) return cudaSuccess;
+        std::vector<Group> next = groups;
+        std::vector<int> nblocks = *blocks;
+        for (size_t gi = 0; gi < groups.size(); ++gi) {
+            next[gi].live = live[gi];
+            if (!live[gi].empty()) plan_live(probs, next[gi], interval, sms);
         }
+        Tables t = build_tables(probs, next, base, slot_of, dsums, &nblocks);
+        if (t.sum_rows > sum_rows || sizeof(int) * t.maps.size() > scr->maps_cap) return cudaSuccess;
+        groups.swap(next);
+        blocks->swap(nblocks);
+        plans.push_back(std::move(t));
+        return upload();
+    };
+    // whether the solve is over: all problems have stopped, or an error (in e or the poll's)
+    auto stopped = [&]() {
+        const DevStatus *h = poll.arrived();
+        if (poll.error != cudaSuccess) return true;
+        if (!h) return false;
+        bool all = true;
+        for (int q = 0; q < count; ++q) all = all && h[q].stop;
+        if (!all) e = thin_out(h);
+        return all || e != cudaSuccess;
+    };
+    bool stop = false;
+    for (int t = 0; t < p.max_iters && !stop;) {
+        const int m = std::min(p.check_every, p.max_iters - t);
+        t += m;
+        for (size_t gi = 0; gi < groups.size() && !stop; ++gi) {
+            for (int left = m; left > 0 && !stop && !groups[gi].live.empty();) {
+                Group &g = groups[gi];                // (planned anew at any poll)
+                const int q = next_pass(g.pass, g.main_pass, left);
+                one(g, q, left == kStages[q]);
+                left -= kStages[q];
+                poll.queued(g.pass[q].us);
+                stop = stopped();
+            }
+            if (stop || groups[gi].live.empty()) continue;
+            check(groups[gi], t);
+            if (gi + 1 < groups.size()) poll.queued(StopPoll::kCheckUs);
+        }
+        if (stop) break;
+        poll.checked();
+        stop = stopped();
     }
     for (size_t gi = 0; gi < groups.size(); ++gi) {
         groups[gi].K.out_many<<<layout_grid(gi), 128, 0, st>>>(ditems + first_item[gi]);
         ctx->launches += 1;
     }
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = poll.error;
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(hstat, dstat, sizeof(DevStatus) * count, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    for (int q = 0; q < 2; ++q)
-        if (ev[q]) cudaEventDestroy(ev[q]);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch solve");
     status->resize(count);
     for (int q = 0; q < count; ++q) (*status)[q] = hstat[slot_of[q]];
