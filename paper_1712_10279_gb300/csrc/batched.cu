@@ -1011,9 +1011,14 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
         if (grouped && p.engine != VOMT_ENGINE_RESIDENT && p.u_norm == VOMT_U_L12 && p.w_norm == VOMT_W_L1 && p.eps == 0.0 &&
             !ctx->drop_exchange && std::min(p.check_every, p.max_iters) >= 4) {
             const int iters = std::max(p.max_iters, 1);
+            std::vector<int> sides, ks;
+            for (const InstDev &I : hinst) {
+                sides.push_back(I.n);
+                ks.push_back(I.k);
+            }
             std::vector<BatchProblem> probs;
-            if (march_problems(hinst, arena, p, &probs) &&
-                march_batch_estimate(ctx, probs, p) < 0.5e-3 * grouped_estimate(waves, iters) / iters) {
+            if (march_batch_estimate(ctx, &b->march, sides, ks, p) < 0.5e-3 * grouped_estimate(waves, iters) / iters &&
+                march_problems(hinst, arena, p, &probs)) {
                 rc = march_batch(ctx, &b->march, probs, p, st, &mstat, &mblocks, &marched);
                 if (rc) return rc;
             }

@@ -364,6 +364,8 @@ int check_chunk(long strip_rows, int sms) { return (int)std::max(2l, (strip_rows
 struct Group {
     int k = 0, main_pass = 0;
     std::vector<int> probs, live;     // all its problems; those the passes below are planned for
+    std::vector<std::pair<int, int>> sides;       // of the live ones: side, how many
+    double points = 0.0;              // of the live ones
     Kernels K;
     int per_sm[3] = {0, 0, 0};
     Pass pass[3];                     // blocks: of the whole group
@@ -373,29 +375,21 @@ struct Group {
     int cur = 0, before = 0;          // states that hold the iterates and their predecessors
 };
 
-double points(const std::vector<BatchProblem> &probs, const std::vector<int> &which)
-{
-    double pts = 0.0;
-    for (int q : which) pts += (double)probs[q].g.n * probs[q].g.n;
-    return pts;
-}
-
 // plan_pass for a group: the chunk length of the least arithmetic time
-Pass plan_group(const std::vector<BatchProblem> &probs, const Group &gr, int S, int blocks_per_sm, int sms)
+Pass plan_group(const Group &gr, int S, int blocks_per_sm, int sms)
 {
     const int k = gr.k, W = 32 - 2 * S;
     const double issue = 20.0 + 40.0 * k + 4.0 * k * (k - 1), lat = 180.0, ghz = 1.95;
     const long cap = (long)blocks_per_sm * sms;
-    int top = 0;
-    for (int q : gr.live) top = std::max(top, probs[q].g.n);
+    const int top = gr.sides.back().first;
     Pass best;
     for (int rows = 1; rows <= top; rows += rows < 32 ? 1 : rows / 16) {
         long blocks = 0, warps = 0;
-        for (int q : gr.live) {
-            const int n = probs[q].g.n;
+        for (const auto &side : gr.sides) {
+            const int n = side.first;
             const long w = (long)((n + W - 1) / W) * ((n + rows - 1) / rows);
-            warps += w;
-            blocks += (w + kWarps - 1) / kWarps;
+            warps += w * side.second;
+            blocks += (w + kWarps - 1) / kWarps * side.second;
         }
         if (blocks > (1l << 30)) continue;
         const long full = blocks / cap, rest = blocks % cap;
@@ -404,53 +398,71 @@ Pass plan_group(const std::vector<BatchProblem> &probs, const Group &gr, int S, 
         const double us = cycles * S * (rows + 2 * S) / (ghz * 1e3);
         if (best.stages == 0 || us < best.us) best = Pass{S, rows, 0, (int)warps, (int)blocks, us};
     }
-    const double mb = 16e-6 * points(probs, gr.live) * (2 * gr.K.groups + (k + 3) / 4);
+    const double mb = 16e-6 * gr.points * (2 * gr.K.groups + (k + 3) / 4);
     best.us = 3.5 + std::max(best.us, mb / (mb > 110.0 ? 6.3 : 12.0));
     return best;
 }
 
-// The passes and the check of a group's live problems.
-void plan_live(const std::vector<BatchProblem> &probs, Group &g, int interval, int sms)
+// The passes and the check of a group's live problems; n: the problems' sides.
+void plan_live(const std::vector<int> &n, Group &g, int interval, int sms)
 {
+    std::vector<int> s;
+    for (int q : g.live) s.push_back(n[q]);
+    std::sort(s.begin(), s.end());
+    g.sides.clear();
+    g.points = 0.0;
+    long strip_rows = 0;
+    for (int side : s) {
+        if (g.sides.empty() || g.sides.back().first != side) g.sides.push_back({side, 0});
+        g.sides.back().second += 1;
+        g.points += (double)side * side;
+        strip_rows += (long)((side + 29) / 30) * side;
+    }
+    g.check_rows = check_chunk(strip_rows, sms);
     g.main_pass = 0;
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < 3 && !s.empty(); ++q) {
         if (g.per_sm[q] < 1) continue;
         Pass &ps = g.pass[q];
-        ps = plan_group(probs, g, kStages[q], g.per_sm[q], sms);
+        ps = plan_group(g, kStages[q], g.per_sm[q], sms);
         const int share = (ps.blocks + sms - 1) / sms;      // see march_solve
         ps.smem = std::max(g.K.smem, kSmemSM / (share + 1));
         if (kStages[q] <= interval && (g.pass[g.main_pass].stages == 0 ||
                                        ps.us / kStages[q] < g.pass[g.main_pass].us / kStages[g.main_pass]))
             g.main_pass = q;
     }
-    long strip_rows = 0;
-    for (int q : g.live) strip_rows += (long)((probs[q].g.n + 29) / 30) * probs[q].g.n;
-    g.check_rows = check_chunk(strip_rows, sms);
 }
 
-int plan_groups(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p, std::vector<Group> *out)
+// A problem's side and channel count are all that its passes are planned from.
+int plan_groups(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<int> &n, const std::vector<int> &ks,
+                const vomt_params &p, std::vector<Group> *out)
 {
     out->clear();
     const int interval = std::max(1, std::min(p.check_every, p.max_iters));
     for (int k = 1; k <= 5; ++k) {
         Group g;
         g.k = k;
-        for (int q = 0; q < (int)probs.size(); ++q)
-            if (probs[q].k == k) g.probs.push_back(q);
+        for (int q = 0; q < (int)n.size(); ++q)
+            if (ks[q] == k) g.probs.push_back(q);
         if (g.probs.empty()) continue;
         g.live = g.probs;
         g.K = pick(k, VOMT_U_L12, VOMT_W_L1, false, true);
         for (int q = 0; q < 3; ++q) {
             if (!g.K.many[q]) continue;
-            cudaError_t e = cudaFuncSetAttribute((const void *)g.K.many[q], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 kSmemBlock);
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g.per_sm[q], (const void *)g.K.many[q], 32 * kWarps,
-                                                                  g.K.smem);
-            if (e != cudaSuccess) return set_cuda_error(ctx, e, "marching kernel");
+            int &per_sm = scr->per_sm[k - 1][q];
+            if (per_sm < 0) {
+                int got = 0;
+                cudaError_t e = cudaFuncSetAttribute((const void *)g.K.many[q],
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBlock);
+                if (e == cudaSuccess)
+                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, (const void *)g.K.many[q], 32 * kWarps,
+                                                                      g.K.smem);
+                if (e != cudaSuccess) return set_cuda_error(ctx, e, "marching kernel");
+                per_sm = got;
+            }
+            g.per_sm[q] = per_sm;
         }
         if (g.per_sm[0] < 1) return VOMT_ERR_TOO_LARGE;
-        plan_live(probs, g, interval, ctx->sm_count);
+        plan_live(n, g, interval, ctx->sm_count);
         out->push_back(g);
     }
     return VOMT_OK;
@@ -510,10 +522,11 @@ Tables build_tables(const std::vector<BatchProblem> &probs, std::vector<Group> &
 
 }  // namespace
 
-double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p)
+double march_batch_estimate(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<int> &n,
+                            const std::vector<int> &k, const vomt_params &p)
 {
     std::vector<Group> groups;
-    if (plan_groups(ctx, probs, p, &groups)) return 1e30;
+    if (plan_groups(ctx, scr, n, k, p, &groups)) return 1e30;
     double us = 0.0;
     for (const Group &g : groups) us += g.pass[g.main_pass].us / kStages[g.main_pass];
     return us;
@@ -531,8 +544,13 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
     *taken = false;
     const int count = (int)probs.size(), sms = ctx->sm_count;
     if (count > 65535) return VOMT_OK;                // a launch's third dimension
+    std::vector<int> side(count), ks(count);
+    for (int q = 0; q < count; ++q) {
+        side[q] = probs[q].g.n;
+        ks[q] = probs[q].k;
+    }
     std::vector<Group> groups;
-    int rc = plan_groups(ctx, probs, p, &groups);
+    int rc = plan_groups(ctx, scr, side, ks, p, &groups);
     if (rc) return rc == VOMT_ERR_TOO_LARGE ? VOMT_OK : rc;
     // scratch: per problem b, two states, the state before a check; check sums (rows for any
     // subset of the problems: check_chunk gives 16 warps per SM, a partly filled chunk per
@@ -644,16 +662,20 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
         std::vector<std::vector<int>> live(groups.size());
         bool again = false;
         for (size_t gi = 0; gi < groups.size(); ++gi) {
+            double left = 0.0;
             for (int q : groups[gi].live)
-                if (!h[slot_of[q]].stop) live[gi].push_back(q);
-            again = again || points(probs, live[gi]) < 0.75 * points(probs, groups[gi].live);
+                if (!h[slot_of[q]].stop) {
+                    live[gi].push_back(q);
+                    left += (double)side[q] * side[q];
+                }
+            again = again || left < 0.75 * groups[gi].points;
         }
         if (!again) return cudaSuccess;
         std::vector<Group> next = groups;
         std::vector<int> nblocks = *blocks;
         for (size_t gi = 0; gi < groups.size(); ++gi) {
             next[gi].live = live[gi];
-            if (!live[gi].empty()) plan_live(probs, next[gi], interval, sms);
+            plan_live(side, next[gi], interval, sms);
         }
         Tables t = build_tables(probs, next, base, slot_of, dsums, &nblocks);
         if (t.sum_rows > sum_rows || sizeof(int) * t.maps.size() > scr->maps_cap) return cudaSuccess;

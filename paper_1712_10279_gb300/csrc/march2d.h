@@ -92,13 +92,16 @@ struct BatchProblem {
     SolveCfg cfg;
     march::PlanarArgs planar;
 };
-struct BatchMarchScratch {            // device and pinned memory of march_batch, kept by the caller
+struct BatchMarchScratch {            // what march_batch keeps on its context
     void *items = nullptr, *maps = nullptr, *data = nullptr, *stat = nullptr, *hstat = nullptr;
     size_t items_cap = 0, maps_cap = 0, data_cap = 0, stat_cap = 0, hstat_cap = 0;
+    // blocks per SM of each pass kernel (-1: its launch attributes are still to be set)
+    int per_sm[5][3] = {{-1, -1, -1}, {-1, -1, -1}, {-1, -1, -1}, {-1, -1, -1}, {-1, -1, -1}};
 };
 void march_scratch_free(BatchMarchScratch *s);
-// microseconds an iteration of the batch takes by estimate
-double march_batch_estimate(vomt_ctx *ctx, const std::vector<BatchProblem> &probs, const vomt_params &p);
+// microseconds an iteration of problems with these sides and channel counts takes by estimate
+double march_batch_estimate(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<int> &n,
+                            const std::vector<int> &k, const vomt_params &p);
 // *taken = false where the memory is not to be had; status[q]: the host copy of each problem's
 // final status block, blocks[q]: the blocks of its main pass
 int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
