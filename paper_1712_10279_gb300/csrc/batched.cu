@@ -960,7 +960,7 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
             if (wide)
                 k_batch_validate<WideSum><<<count * kValChunks, 256, 0, st>>>(b->dinst, arena, b->dval);
             else
-                k_batch_validate<PairSum><<<count * kValChunks, 256, 0, st>>>(b->dinst, arena, b->dval);
+                k_batch_validate<TripleSum><<<count * kValChunks, 256, 0, st>>>(b->dinst, arena, b->dval);
             ++ctx->launches;
             e = cudaMemcpyAsync(hv.data(), b->dval, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -44,9 +44,9 @@ PairTable make_pairs(int k)
     return t;
 }
 
-// What a block of 256 threads has seen of matrix densities: sum tr Lam0, sum tr Lam1 (FP32
-// pairs per thread and warp, FP64 where those overflow), min diagonal entry, max asymmetry, max |X_ab|, count of
-// non-finite entries.
+// What a block of 256 threads has seen of matrix densities: sum tr Lam0, sum tr Lam1 (three
+// FP32 numbers per thread and warp, FP64 where those overflow), min diagonal entry, max
+// asymmetry, max |X_ab|, count of non-finite entries.
 template <typename Sum>
 struct MatrixCheck {
     Sum t[2];
@@ -409,7 +409,7 @@ static int momt_any(int dim, vomt_ctx *ctx, int n, int k, const float *Lam0, con
             if (wide)
                 k_mat_validate<dev::WideSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
             else
-                k_mat_validate<dev::PairSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
+                k_mat_validate<dev::TripleSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
             ++ctx->launches;
             e = cudaMemcpyAsync(hv.data(), ctx->partials, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -548,7 +548,7 @@ extern "C" int momt_solve_complex(vomt_ctx *ctx, int n, int k, const float *Lam0
             if (wide)
                 k_herm_validate<dev::WideSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
             else
-                k_herm_validate<dev::PairSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
+                k_herm_validate<dev::TripleSum><<<vb, 256, 0, st>>>(nn, k, Lam0, Lam1, ctx->partials);
             ++ctx->launches;
             e = cudaMemcpyAsync(hv.data(), ctx->partials, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -563,7 +563,7 @@ int validate_densities(vomt_ctx *ctx, int planes, int n, const float *rho0, cons
         if (wide)
             k_validate<dev::WideSum><<<blocks, 256, 0, st>>>(count, rho0, rho1, ctx->partials);
         else
-            k_validate<dev::PairSum><<<blocks, 256, 0, st>>>(count, rho0, rho1, ctx->partials);
+            k_validate<dev::TripleSum><<<blocks, 256, 0, st>>>(count, rho0, rho1, ctx->partials);
         ctx->launches += 1;
         cudaError_t e = cudaMemcpyAsync(h.data(), ctx->partials, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -886,7 +886,7 @@ int noalloc_solve(int n, const float *rho0, const float *rho1, const vomt_graph 
         if (wide)
             k_validate<dev::WideSum><<<vblocks, 256, 0, st>>>(count, rho0, rho1, vpart);
         else
-            k_validate<dev::PairSum><<<vblocks, 256, 0, st>>>(count, rho0, rho1, vpart);
+            k_validate<dev::TripleSum><<<vblocks, 256, 0, st>>>(count, rho0, rho1, vpart);
         ++launches;
         e = cudaMemcpyAsync(hv, vpart, sizeof(double) * 5 * (size_t)vblocks, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
