@@ -37,26 +37,23 @@ namespace {
 constexpr int AX = 32, AY = 8, AT = AX * AY;
 constexpr size_t kKeepBytes = (size_t)1 << 30;      // most memory for keeping every iterate of an unrolled solve
 
-// A cluster of kEnvCluster blocks per problem; a warp takes whole rows.  The sums are FP32
-// pairs per thread and warp and FP64 beyond, and meet through distributed shared memory, so
-// the call needs no scratch and calls on several streams do not disturb each other.
-// Bound by the latency of two passes over a problem (256^2, three channels: eight problems
-// took 727 us with one block each, FP64 sums per value and a division per index).
+// Most blocks of a problem's cluster; a warp takes whole rows.  The sums meet through
+// distributed shared memory, so the call needs no scratch and calls on several streams do not
+// disturb each other.
 constexpr int kEnvCluster = 8;
 
-__global__ void __launch_bounds__(1024) k_envelope(int n, int pitch, int k, int l, int wn, const float *__restrict__ phi,
-                                                   const float *__restrict__ w, const float *__restrict__ gscale,
-                                                   float *__restrict__ d_rho0, float *__restrict__ d_rho1,
-                                                   float *__restrict__ d_alpha)
+// This block's sums of phi and of ||w|| (L1; Sum: TripleSum, or WideSum where that overflows),
+// then the cluster's: totals[0], totals[1], the same in every thread.  The squares of the
+// joint norm and their root are FP64.
+template <typename Sum>
+__device__ __forceinline__ void envelope_totals(cooperative_groups::cluster_group &cluster, int n, int pitch, int k, int l,
+                                                int wn, const float *P, const float *Wb, int first, int step,
+                                                double (&totals)[2])
 {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int problem = blockIdx.x / kEnvCluster, rank = blockIdx.x % kEnvCluster;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int first = rank * 32 + wid, step = kEnvCluster * 32;       // this warp's rows
-    const size_t pw = (size_t)n * pitch, pcnt = (size_t)k * pw;
-    const float *P = phi + problem * pcnt, *Wb = w + problem * (size_t)l * pw;
-    dev::PairSum s, sw;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const size_t pw = (size_t)n * pitch;
+    Sum s, sw;
+    double joint = 0.0;
     for (int r = first; r < k * n; r += step) {
         const float *row = P + (size_t)r * pitch;
 #pragma unroll 4
@@ -71,47 +68,92 @@ __global__ void __launch_bounds__(1024) k_envelope(int n, int pitch, int k, int 
                     for (int i = lane; i < n; i += 32) sw.add(fabsf(row[e * pw + i]));
             } else {
                 for (int i = lane; i < n; i += 32) {
-                    float a = 0.0f;
-                    for (int e = 0; e < l; ++e) a += row[e * pw + i] * row[e * pw + i];
-                    sw.add(sqrtf(a));
+                    double a = 0.0;
+                    for (int e = 0; e < l; ++e) {
+                        const double x = row[e * pw + i];
+                        a += x * x;
+                    }
+                    joint += sqrt(a);
                 }
             }
         }
     }
-    __shared__ double sh[32][2], sum[2];
+    // warps, blocks, cluster: kept in Sum's form all the way
+    __shared__ uint32_t sh[32][2][3], block[2][3];
+    __shared__ double joints[32], block_joint, out[2];
     s.warp();
     sw.warp();
+    if (wn != VOMT_W_L1)
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) joint += __shfl_down_sync(0xffffffffu, joint, off);
     if (lane == 0) {
-        sh[wid][0] = s.value();
-        sh[wid][1] = sw.value();
+        s.save(sh[wid][0]);
+        sw.save(sh[wid][1]);
+        joints[wid] = joint;
     }
     __syncthreads();
-    if (threadIdx.x < 2) {
+    if (wid < 2) {                        // warp 0: phi, warp 1: w
+        Sum t;
+        if (lane < warps) t.merge(sh[lane][wid]);
+        t.warp();
+        if (lane == 0) t.save(block[wid]);
+    } else if (threadIdx.x == 64) {
         double t = 0.0;
-        for (int q = 0; q < 32; ++q) t += sh[q][threadIdx.x];
-        sum[threadIdx.x] = t;
+        for (int q = 0; q < warps; ++q) t += joints[q];
+        block_joint = t;
     }
     cluster.sync();
-    double total = 0.0, wtotal = 0.0;
-    for (int q = 0; q < kEnvCluster; ++q) {
-        const double *o = cluster.map_shared_rank(sum, q);
-        total += o[0];
-        if (threadIdx.x == 0) wtotal += o[1];
+    if (threadIdx.x < 2) {
+        Sum t;
+        double j = 0.0;
+        for (int q = 0; q < (int)cluster.num_blocks(); ++q) {
+            t.merge(cluster.map_shared_rank(&block[threadIdx.x][0], q));
+            if (threadIdx.x == 1) j += *cluster.map_shared_rank(&block_joint, q);
+        }
+        out[threadIdx.x] = t.value() + j;
     }
-    cluster.sync();                       // no block leaves while another reads its sums
-    const double mean = total / ((double)k * n * n);
-    const float mh = (float)mean, ml = (float)(mean - (double)mh);
+    __syncthreads();
+    totals[0] = out[0];
+    totals[1] = out[1];
+    cluster.sync();                       // no block leaves, or sums again, while another reads its sums
+}
+
+// A cluster of one to kEnvCluster blocks per problem (vomt_backward).  Bound by the latency of
+// two passes over a problem.
+__global__ void __launch_bounds__(1024) k_envelope(int n, int pitch, int k, int l, int wn, const float *__restrict__ phi,
+                                                   const float *__restrict__ w, const float *__restrict__ gscale,
+                                                   float *__restrict__ d_rho0, float *__restrict__ d_rho1,
+                                                   float *__restrict__ d_alpha)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int blocks = (int)cluster.num_blocks(), problem = blockIdx.x / blocks, rank = blockIdx.x % blocks;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int first = rank * warps + wid, step = blocks * warps;      // this warp's rows
+    const size_t pw = (size_t)n * pitch, pcnt = (size_t)k * pw;
+    const float *P = phi + problem * pcnt, *Wb = w + problem * (size_t)l * pw;
+    double totals[2];
+    envelope_totals<dev::TripleSum>(cluster, n, pitch, k, l, wn, P, Wb, first, step, totals);
+    if (!isfinite(totals[0]) || !isfinite(totals[1]))
+        envelope_totals<dev::WideSum>(cluster, n, pitch, k, l, wn, P, Wb, first, step, totals);
+    // phi - mean, the mean in three FP32 numbers and the rounding errors carried to one final
+    // addition: the FP64 difference rounded to FP32, at FP32's rate
+    const double mean = totals[0] / ((double)k * n * n);
+    const float mh = (float)mean, mm = (float)(mean - (double)mh), ml = (float)(mean - (double)mh - (double)mm);
     const float g = gscale ? gscale[problem] : 1.0f;
     for (int r = first; r < k * n; r += step) {
         const size_t o = (size_t)r * pitch;
 #pragma unroll 4
         for (int i = lane; i < n; i += 32) {
-            const float v = g * ((P[o + i] - mh) - ml);
+            float e, f, h;
+            const float d = dev::two_sum(P[o + i], -mh, e), t = dev::two_sum(e, -mm, f);
+            const float c = dev::two_sum(d, t, h);
+            const float v = g * (c + (h + (f - ml)));
             if (d_rho1) d_rho1[problem * pcnt + o + i] = v;
             if (d_rho0) d_rho0[problem * pcnt + o + i] = -v;
         }
     }
-    if (threadIdx.x == 0 && rank == 0 && d_alpha) d_alpha[problem] = (float)(g * wtotal);
+    if (threadIdx.x == 0 && rank == 0 && d_alpha) d_alpha[problem] = (float)(g * totals[1]);
 }
 
 // The reverse step's sums, each rounded in a fixed way: the shrink's derivative jumps where

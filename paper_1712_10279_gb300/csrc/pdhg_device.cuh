@@ -211,19 +211,31 @@ struct TripleSum {
         mid = two_sum(mid, e, f);
         lo += f;
     }
+    __device__ __forceinline__ void merge(float oh, float om, float ol)
+    {
+        float f;
+        add(oh);
+        mid = two_sum(mid, om, f);
+        lo += ol + f;
+    }
     __device__ __forceinline__ void warp()          // lane 0 ends with the warp's sum
     {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float oh = __shfl_down_sync(0xffffffffu, hi, off), om = __shfl_down_sync(0xffffffffu, mid, off);
-            const float ol = __shfl_down_sync(0xffffffffu, lo, off);
-            float f;
-            add(oh);
-            mid = two_sum(mid, om, f);
-            lo += ol + f;
-        }
+        for (int off = 16; off > 0; off >>= 1)
+            merge(__shfl_down_sync(0xffffffffu, hi, off), __shfl_down_sync(0xffffffffu, mid, off),
+                  __shfl_down_sync(0xffffffffu, lo, off));
     }
     __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
+    __device__ __forceinline__ void save(uint32_t *w) const
+    {
+        w[0] = __float_as_uint(hi);
+        w[1] = __float_as_uint(mid);
+        w[2] = __float_as_uint(lo);
+    }
+    __device__ __forceinline__ void merge(const uint32_t *w)
+    {
+        merge(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]));
+    }
 };
 
 // The same in FP64, for sums beyond FP32's range.
@@ -236,6 +248,13 @@ struct WideSum {
         for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     }
     __device__ __forceinline__ double value() const { return v; }
+    __device__ __forceinline__ void save(uint32_t *w) const
+    {
+        w[0] = (uint32_t)__double2loint(v);
+        w[1] = (uint32_t)__double2hiint(v);
+        w[2] = 0;
+    }
+    __device__ __forceinline__ void merge(const uint32_t *w) { v += __hiloint2double((int)w[1], (int)w[0]); }
 };
 
 // Input checks of densities: what a block of 256 threads has seen, stored as five FP64
