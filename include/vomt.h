@@ -197,7 +197,8 @@ int vomt_solve_host(vomt_ctx *ctx, int n, const float *rho0, const float *rho1,
  * {L1, L2}; p->eps must be 0; p->engine is ignored; p->halo > 0 sets the
  * number of z planes each thread block marches through (0: the library's
  * choice, about four blocks per SM).  result->variant tells whether the TMA
- * form of the step ran on unpadded rows (n a multiple of 4, n >= 40, k <= 6).  Default mu
+ * form of the step ran on unpadded rows (n a multiple of 4, n >= 40, k <= 6);
+ * vomt_last_form() also tells the padded ones.  Default mu
  * is 1/(48 tau (n-1)^2) (1/(24 tau (n-1)^2) without edges), since
  * ||grad||^2 <= 12 (n-1)^2 in 3-D; user mu, nu must satisfy
  * tau mu 12 (n-1)^2 + tau nu lambda_max(-Delta_G) < 1.  The history is that of
@@ -230,6 +231,13 @@ int vomt_history(vomt_ctx *ctx, double *out, int cap);
 #define VOMT_FORM_UNROLLED_KEPT 11   /* unrolled gradient, every iterate kept */
 #define VOMT_FORM_UNROLLED_CKPT 12   /* unrolled gradient, checkpoints and recomputed segments */
 int vomt_last_form(const vomt_ctx *ctx);
+
+/* Most device memory that a call on ctx takes for a faster form beyond what the
+ * plain form of the same call needs (1 GiB by default; 0: plain forms only):
+ * rows of 3-D volumes padded to 16 bytes.  The results are the same either way.
+ * Applies to later calls on ctx.  Returns VOMT_OK, or VOMT_ERR_BAD_ARG for a null
+ * ctx. */
+int vomt_set_memory_limit(vomt_ctx *ctx, size_t bytes);
 
 /* Bounded waits of the resident engine (no counterpart in the paper; a test
  * and tuning hook).  In the resident engine one thread block waits on another

@@ -366,6 +366,13 @@ def set_wait_policy(budget_ms: float = 0.0, drop_exchange: int = 0, device: int 
     _native.check(_native.load().vomt_set_wait_policy(ctx, float(budget_ms), int(drop_exchange)), ctx)
 
 
+def set_memory_limit(nbytes: int = 1 << 30, device: int = 0):
+    """Most device memory the library takes for a faster form beyond what the plain form of the
+    same call needs (0: plain forms only; vomt_set_memory_limit)."""
+    ctx = _native.context(device)
+    _native.check(_native.load().vomt_set_memory_limit(ctx, int(nbytes)), ctx)
+
+
 def last_form(device: int = 0) -> str:
     """The form of the kernels that the last solve or unrolled gradient on `device` ran: one
     of _native.FORMS (vomt_last_form)."""

@@ -81,6 +81,7 @@ SIGNATURES = {
     "momt_solve3d": (c_int, [c_void_p, c_int, c_int, c_void_p, c_void_p, c_int, c_void_p, c_double,
                              ctypes.POINTER(Params), c_void_p, c_void_p, c_void_p, ctypes.POINTER(Result), c_void_p]),
     "vomt_history": (c_int, [c_void_p, P_double, c_int]),
+    "vomt_set_memory_limit": (c_int, [c_void_p, ctypes.c_size_t]),
     "vomt_last_form": (c_int, [c_void_p]),
     "vomt_set_wait_policy": (c_int, [c_void_p, c_double, c_int]),
     "vomt_backward": (c_int, [c_void_p, c_int, c_int, c_int, c_int, c_int, c_int, c_void_p, c_void_p, c_void_p,

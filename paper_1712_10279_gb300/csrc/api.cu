@@ -481,6 +481,13 @@ extern "C" int vomt_set_wait_policy(vomt_ctx *ctx, double budget_ms, int drop_ex
     return VOMT_OK;
 }
 
+int vomt_set_memory_limit(vomt_ctx *ctx, size_t bytes)
+{
+    if (!ctx) return VOMT_ERR_BAD_ARG;
+    ctx->spare_bytes = bytes;
+    return VOMT_OK;
+}
+
 int vomt_last_form(const vomt_ctx *ctx) { return ctx ? ctx->last_form : VOMT_FORM_NONE; }
 
 int vomt_history(vomt_ctx *ctx, double *out, int cap)

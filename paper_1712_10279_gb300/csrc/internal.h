@@ -175,6 +175,8 @@ struct vomt_ctx {
     int launches = 0;                        // kernels launched by the current call
     int last_blocks = 0, last_halo = 0, last_variant = 0;      // launch shape of the current call
     int last_form = 0;                       // VOMT_FORM_* of the last solve or gradient
+    // most memory taken for a faster form beyond what the plain one needs (vomt_set_memory_limit)
+    size_t spare_bytes = (size_t)1 << 30;
     // matrix-OMT compact staging (device)
     float *mstage = nullptr;
     size_t mstage_bytes = 0;

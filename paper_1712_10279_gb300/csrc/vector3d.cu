@@ -17,6 +17,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <memory>
+
 #include "internal.h"
 #include "pdhg_device.cuh"
 #include "vector3d.cuh"
@@ -464,6 +466,10 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     // 120 us an iteration with per-thread loads)
     bool tma = tma3_supported(n, k, l, p.u_norm, p.w_norm);
     int np = tma ? (n + 3) / 4 * 4 : n;
+    if ((size_t)(9 * k + 2 * l) * n * n * (np - n) * sizeof(float) > ctx->spare_bytes) {
+        tma = false;
+        np = n;
+    }
     // workspace: b, then two states {phi, u_x, u_y, u_z, w}
     auto workspace = [&]() {
         return ensure_buffer(ctx, (void **)&ctx->ws, &ctx->ws_floats,
@@ -477,15 +483,26 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
         if (!rc) ctx->err.clear();
     }
     if (rc) return rc;
-    const size_t points = (size_t)n * n * n, m = (size_t)n * n * np, per_state = (size_t)(4 * k + l) * m;
+    const size_t points = (size_t)n * n * n;
     float *b = ctx->ws;
     S3Out so[2];
     S3In si[2];
-    for (int q = 0; q < 2; ++q) {
-        float *base = ctx->ws + (size_t)k * m + q * per_state;
-        so[q] = S3Out{base, base + (size_t)k * m, base + (size_t)2 * k * m, base + (size_t)3 * k * m,
-                      base + (size_t)4 * k * m};
-        si[q] = S3In{so[q].phi, so[q].ux, so[q].uy, so[q].uz, so[q].w};
+    auto layout = [&]() {
+        const size_t m = (size_t)n * n * np, per_state = (size_t)(4 * k + l) * m;
+        for (int q = 0; q < 2; ++q) {
+            float *base = ctx->ws + (size_t)k * m + q * per_state;
+            so[q] = S3Out{base, base + (size_t)k * m, base + (size_t)2 * k * m, base + (size_t)3 * k * m,
+                          base + (size_t)4 * k * m};
+            si[q] = S3In{so[q].phi, so[q].ux, so[q].uy, so[q].uz, so[q].w};
+        }
+    };
+    layout();
+    std::unique_ptr<Tma3Plan, void (*)(Tma3Plan *)> plan(nullptr, tma3_plan_destroy);
+    if (tma) plan.reset(tma3_plan_create(n, np, k, l, p.u_norm, p.w_norm, so[0].phi, so[1].phi, b));
+    const Tma3Plan *tp = plan.get();
+    if (!tp && np != n) {             // no tensor maps: the per-thread form, which takes plain rows
+        np = n;
+        layout();
     }
     const int nblocks = (int)((points + T3 - 1) / T3);
     const int mblocks = nblocks < kMetricBlocks ? nblocks : kMetricBlocks;     // blocks of a check
@@ -502,8 +519,6 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     L3 L = pick3(k, p.u_norm, p.w_norm);
     e = cudaFuncSetAttribute((const void *)L.step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "3-D step shared memory");
-    Tma3Plan *tp = tma ? tma3_plan_create(n, np, k, l, p.u_norm, p.w_norm, so[0].phi, so[1].phi, b) : nullptr;
-    if (!tp && np != n) return fail(ctx, VOMT_ERR_CUDA, "tensor maps of the padded volumes");
     ctx->last_variant = tp && np == n ? 1 : 0;
     ctx->last_form = !tp ? VOMT_FORM_STEP3 : (np == n ? VOMT_FORM_STEP3_TMA : VOMT_FORM_STEP3_PADDED);
     // z chunk: the longest of 32, 16, 8, 4 planes that still gives 1.5 blocks per SM
@@ -565,7 +580,6 @@ int solve3d_core(vomt_ctx *ctx, int n, const OpDev &g, const StepDev &s, const S
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     for (int q = 0; q < 2; ++q)
         if (ev[q]) cudaEventDestroy(ev[q]);
-    tma3_plan_destroy(tp);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "3-D solve");
     return VOMT_OK;
 }
