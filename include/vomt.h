@@ -234,9 +234,10 @@ int vomt_last_form(const vomt_ctx *ctx);
 
 /* Most device memory that a call on ctx takes for a faster form beyond what the
  * plain form of the same call needs (1 GiB by default; 0: plain forms only):
- * rows of 3-D volumes padded to 16 bytes.  The results are the same either way.
- * Applies to later calls on ctx.  Returns VOMT_OK, or VOMT_ERR_BAD_ARG for a null
- * ctx. */
+ * rows of 3-D volumes padded to 16 bytes, the iterates of an unrolled gradient.
+ * The results are the same either way.  The context keeps such memory for later
+ * calls; gradient scratch larger than the new limit is freed.  Applies to later
+ * calls on ctx.  Returns VOMT_OK, or VOMT_ERR_BAD_ARG for a null ctx. */
 int vomt_set_memory_limit(vomt_ctx *ctx, size_t bytes);
 
 /* Bounded waits of the resident engine (no counterpart in the paper; a test
@@ -277,9 +278,10 @@ int vomt_backward(vomt_ctx *ctx, int batch, int n, int pitch, int k, int n_edges
 /* Unrolled gradient: J_T = P(u^T, w^T), the primal objective after T
  * iterations of Section 7.2 from the zero iterate (tau, mu, nu, norms from p;
  * p->u_norm must be VOMT_U_L12), and its exact gradient by reverse mode through
- * the T iterations.  The forward pass keeps every iterate where that takes at
- * most 1 GiB, else one every `ckpt` iterations, and the reverse pass recomputes
- * each segment from its checkpoint.
+ * the T iterations.  The forward pass keeps every iterate where that takes no
+ * more than the context's memory limit (vomt_set_memory_limit), else one every
+ * `ckpt` iterations, and the reverse pass recomputes each segment from its
+ * checkpoint; both give the same gradients.
  * rho0, rho1: device [k][n][n].  Outputs: d_rho0, d_rho1 device [k][n][n]
  * (either may be NULL), *d_alpha and *J host (either may be NULL); every
  * derivative is multiplied by `scale`.  Returns after the work finished.

@@ -5,8 +5,9 @@ solved on the GPU; its backward is the envelope gradient computed by the CUDA
 kernel behind ``vomt_backward`` (dV/drho1 = phi*, dV/drho0 = -phi*, centred;
 dV/dalpha = sum ||w*||).  ``unrolled_cost`` is J_T, the primal objective after T
 iterations from zero, whose backward runs the reverse-mode kernels behind
-``vomt_unrolled_grad`` (checkpoints every ``ckpt`` iterations).  The Python
-here only marshals tensors; every step runs in the library.
+``vomt_unrolled_grad`` (every iterate kept within the library's memory limit, see
+``set_memory_limit``, else checkpoints every ``ckpt`` iterations).  The Python here only
+marshals tensors; every step runs in the library.
 """
 from __future__ import annotations
 
@@ -125,8 +126,9 @@ class _UnrolledCost(torch.autograd.Function):
 
 
 def unrolled_cost(rho0, rho1, edges, alpha=1.0, T=200, ckpt=20, **kw):
-    """J_T = P(u^T, w^T) after T iterations from zero; backward by reverse mode with
-    checkpoints every `ckpt` iterations (vomt_unrolled_grad)."""
+    """J_T = P(u^T, w^T) after T iterations from zero; backward by reverse mode
+    (vomt_unrolled_grad), with checkpoints every `ckpt` iterations where the iterates take more
+    than the library's memory limit (set_memory_limit)."""
     return _UnrolledCost.apply(rho0, rho1, alpha, list(edges), int(T), int(ckpt), dict(kw))
 
 

@@ -12,8 +12,8 @@
 // Unrolled gradient.  J_T = P(u^T, w^T), the primal objective after T
 // iterations of Section 7.2 from the zero iterate, is differentiated by reverse
 // mode through the T iterations.  The forward pass keeps every iterate where that
-// takes at most 1 GiB, else one every `ckpt` iterations, from which the reverse pass
-// recomputes a segment at a time; the reverse pass applies the transposed Jacobian of
+// takes no more than the context's memory limit, else one every `ckpt` iterations, from
+// which the reverse pass recomputes a segment at a time; the reverse pass applies the transposed Jacobian of
 // one iteration per step (k_adj_step; at 256^2, three channels, 4.3 us a step, 15 us
 // marching two rows per warp, and 2.9 us a forward step): the chain rule through phi' = phi + tau(div_x ubar + div_G wbar +
 // rho1 - rho0), through u' = shrink(u + mu grad phi; mu) and through
@@ -35,7 +35,6 @@ namespace vomt {
 namespace {
 
 constexpr int AX = 32, AY = 8, AT = AX * AY;
-constexpr size_t kKeepBytes = (size_t)1 << 30;      // most memory for keeping every iterate of an unrolled solve
 
 // Most blocks of a problem's cluster; a warp takes whole rows.  The sums meet through
 // distributed shared memory, so the call needs no scratch and calls on several streams do not
@@ -487,13 +486,14 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         march::MarchOp mop;
         if (!march_op(op, s, &mop)) return fail(ctx, VOMT_ERR_BAD_ARG, "unrolled gradient: not a channel graph");
         const size_t nn = (size_t)n * n, SZ = (size_t)(3 * K + l) * nn;
-        // Every iterate is kept where that takes at most kKeepBytes: nothing is computed twice
-        // then (256^2, three channels, 200 iterations: 0.6 GB and 190 launches fewer).  Beyond, or
-        // where the memory is not to be had, checkpoints every `ckpt` iterations.
-        bool keep = ((size_t)T + 1) * SZ * sizeof(float) <= kKeepBytes;
-        const int nck = T / ckpt + 1;
+        // Every iterate is kept where that takes no more than the context's memory limit:
+        // nothing is computed twice then (256^2, three channels, 200 iterations: 0.6 GB and 190
+        // launches fewer).  Beyond, or where the memory is not to be had, checkpoints every `ckpt`
+        // iterations.
+        bool keep = ((size_t)T + 1) * SZ * sizeof(float) <= ctx->spare_bytes;
+        const int nck = T / ckpt + 1, slots = std::min(ckpt, T) + 1;      // checkpoints, recompute slots
         auto floats = [&]() {
-            return (size_t)2 * K * nn + 2 * SZ + (keep ? (size_t)T + 1 : (size_t)nck + ckpt + 1) * SZ;
+            return (size_t)2 * K * nn + 2 * SZ + (keep ? (size_t)T + 1 : (size_t)nck + slots) * SZ;
         };
         rc = ensure_buffer(ctx, (void **)&ctx->gbuf, &ctx->gbuf_bytes, floats() * sizeof(float), "gradient scratch");
         if (rc && keep) {
@@ -511,7 +511,7 @@ extern "C" int vomt_unrolled_grad(vomt_ctx *ctx, int n, const float *rho0, const
         float *b = ctx->gbuf, *grho = b + (size_t)K * nn;
         float *adj = grho + (size_t)K * nn;                 // 2 adjoint states
         float *ck = adj + 2 * SZ;                           // the iterates kept (all, or nck checkpoints)
-        float *seg = ck + (size_t)nck * SZ;                 // ckpt + 1 recompute slots
+        float *seg = ck + (size_t)nck * SZ;                 // `slots` recompute slots
         double *part = ctx->gpart, *apart = part + 2 * (size_t)nb;
         const int pb = (int)(((size_t)K * nn + 255) / 256 < 2048 ? ((size_t)K * nn + 255) / 256 : 2048);
         e = cudaMemsetAsync(ctx->dstatus, 0, sizeof(DevStatus), st);
