@@ -374,7 +374,9 @@ __global__ void __launch_bounds__(NTHR, min_blocks(K, S)) k_march_many(const Bat
 // The terms of a convergence check (the sums RED_*) of the iterate cur and its
 // predecessor prv.  The same march: both states' rows once, neighbours along x by
 // shuffles, the row below carried; strips write no columns, so a strip covers 30.  Sums
-// per thread and warp in pairs of FP32 numbers (CheckAcc), per block and grid in FP64.
+// per thread and warp in pairs of FP32 numbers (CheckAcc), per block and grid in FP64; the
+// constraint residual, which cancels several digits, as a pair too (residual_pair), where the
+// one-iteration kernels form it in FP64.
 // About 15 us at 1024^2 with one channel, bound by the latency of a row's loads; loading
 // a row ahead costs more in resident warps than it hides (19 us).
 template <int K, int UN, int WN>
@@ -485,17 +487,16 @@ __device__ __forceinline__ void check_block(const CheckArgs &a, const MarchOp &g
                 const float o = fmaxf(dn_w - alpha, 0.0f);
                 if (g.l > 0) dist += o * o;
             }
-            float rr = 0.0f;
 #pragma unroll
             for (int c = 0; c < K; ++c) {
-                const float rc = dev::residual_c(ih, uxs[c], uxl[c], unn[c], un_[c], gwb[c]);
-                rr += rc * rc;
+                float lo;
+                const float rc = dev::residual_pair(ih, uxs[c], uxl[c], unn[c], un_[c], gwb[c], lo);
+                if (own) acc.add_square(RED_RR, rc, lo);
                 fx += dph[c] * ddiv[c];
                 un_[c] = unn[c];
                 dn[c] = dnn[c];
             }
             if (own) {
-                acc.add(RED_RR, rr);
                 acc.add(RED_P, nu_pt + alpha * nw_pt);
                 if (g.reg) {
                     acc.add(RED_P, g.eps * q2);

@@ -170,6 +170,25 @@ __device__ __forceinline__ float residual_c(float ih, float ux, float xl, float 
     return r + (e4 + (pe + ih * ((e1 + e2) + e3)));
 }
 
+// The same with nothing dropped but the rounding of the smallest terms: the residual as a
+// normalised pair hi + lo, correct to about 2^-48 of hi.
+__device__ __forceinline__ float residual_pair(float ih, float ux, float xl, float uy, float yd, float gb, float &lo)
+{
+    float e1, e2, e3, e4, f1, f2, g1, g2, h;
+    const float d1 = two_sum(ux, -xl, e1);
+    const float d2 = two_sum(uy, -yd, e2);
+    const float s = two_sum(d1, d2, e3);
+    const float p = ih * s;
+    const float pe = fmaf(ih, s, -p);
+    const float r = two_sum(p, gb, e4);
+    const float t = two_sum(two_sum(e1, e2, f1), e3, f2);
+    const float q = ih * t;
+    const float c = two_sum(two_sum(pe, q, g1), e4, g2);
+    const float hi = two_sum(r, c, h);
+    lo = h + ((g1 + g2) + (fmaf(ih, t, -q) + ih * (f1 + f2)));
+    return hi;
+}
+
 // A running sum kept as a pair of FP32 numbers by TwoSum (about twice FP32 precision).  FP64
 // additions run at a sixty-fourth of the FP32 rate on this GPU, so a pass that adds every
 // value it reads in FP64 is bound by them.
@@ -331,6 +350,13 @@ struct CheckAcc {
         const float h = __double2float_rn(x);
         add(q, h);
         lo[q] += __double2float_rn(x - (double)h);
+    }
+    // (x + y)^2, y below the rounding of x
+    __device__ __forceinline__ void add_square(int q, float x, float y)
+    {
+        const float s = x * x;
+        add(q, s);
+        lo[q] += fmaf(x, x, -s) + 2.0f * x * y;
     }
     __device__ __forceinline__ void max(int q, float x) { hi[q] = fmaxf(hi[q], x); }
 };
