@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(AT) k_adj_step(const __grid_constant__ march::
     constexpr int LK = ALK<K>::v;
     const int n = g.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int i = blockIdx.x * 30 - 1 + lane, j = blockIdx.y * AY + wid;
-    dev::PairSum sum;                     // this thread's share of -dJ/dalpha / nu
+    dev::TripleSum sum;                   // this thread's share of -dJ/dalpha / nu
     if (j < n) {                          // whole warps
         const bool in = i >= 0 && i < n, own = in && lane >= 1 && lane < 31;
         const bool hR = i < n - 1, hL = i > 0, hU = j < n - 1, hD = j > 0;
@@ -364,10 +364,10 @@ __global__ void __launch_bounds__(AT) k_adj_step(const __grid_constant__ march::
             }
         }
     }
-    // the block's sum: FP32 pairs over a warp, FP64 over the warps; the terms cancel, so each
-    // enters unrounded and nu multiplies the sum
+    // the block's sum: three FP32 numbers over a warp that has terms, FP64 over the warps; the
+    // terms cancel, so each enters unrounded and nu multiplies the sum
     __shared__ double sh[AY];
-    sum.warp();
+    if (__any_sync(0xffffffffu, sum.hi != 0.0f || sum.mid != 0.0f || sum.lo != 0.0f)) sum.warp();
     if (lane == 0) sh[wid] = sum.value();
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -189,38 +189,14 @@ __device__ __forceinline__ float residual_pair(float ih, float ux, float xl, flo
     return hi;
 }
 
-// A running sum kept as a pair of FP32 numbers by TwoSum (about twice FP32 precision).  FP64
-// additions run at a sixty-fourth of the FP32 rate on this GPU, so a pass that adds every
-// value it reads in FP64 is bound by them.
-struct PairSum {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x)
-    {
-        float e;
-        hi = two_sum(hi, x, e);
-        lo += e;
-    }
-    __device__ __forceinline__ void merge(float oh, float ol)
-    {
-        float e;
-        hi = two_sum(hi, oh, e);
-        lo += ol + e;
-    }
-    __device__ __forceinline__ void warp()          // lane 0 ends with the warp's sum
-    {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1)
-            merge(__shfl_down_sync(0xffffffffu, hi, off), __shfl_down_sync(0xffffffffu, lo, off));
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // A running sum kept as three FP32 numbers by TwoSum, what the first addition rounds off
 // going to the second number and what that rounds off to the third: no less accurate than an
-// FP64 sum at FP32's rate.  Over 96 x 2048 values summed per thread and warp and then in FP64,
-// the error against exact sums, over the sum of the magnitudes, is (root mean square) 6.6e-17
-// for densities (FP64 8.2e-17, pairs 3.1e-16), 2.2e-19 for potentials (2.2e-19, 5.5e-19) and 0
-// for terms that cancel to 1e-6 (0, 1.9e-18).  A sum beyond FP32's range becomes NaN.
+// FP64 sum at FP32's rate (FP64 additions run at a sixty-fourth of it on this GPU, so a pass
+// that adds every value it reads in FP64 is bound by them).  Over 96 x 2048 values summed per
+// thread and warp and then in FP64, the error against exact sums, over the sum of the
+// magnitudes, is (root mean square) 6.6e-17 for densities (FP64 8.2e-17, pairs 3.1e-16), 2.2e-19
+// for potentials (2.2e-19, 5.5e-19) and 0 for terms that cancel to 1e-6 (0, 1.9e-18).  A sum
+// beyond FP32's range becomes NaN.
 struct TripleSum {
     float hi = 0.0f, mid = 0.0f, lo = 0.0f;
     __device__ __forceinline__ void add(float x)
