@@ -234,10 +234,11 @@ int vomt_last_form(const vomt_ctx *ctx);
 
 /* Most device memory that a call on ctx takes for a faster form beyond what the
  * plain form of the same call needs (1 GiB by default; 0: plain forms only):
- * rows of 3-D volumes padded to 16 bytes, the iterates of an unrolled gradient.
- * The results are the same either way.  The context keeps such memory for later
- * calls; gradient scratch larger than the new limit is freed.  Applies to later
- * calls on ctx.  Returns VOMT_OK, or VOMT_ERR_BAD_ARG for a null ctx. */
+ * rows of 3-D volumes padded to 16 bytes, the iterates of an unrolled gradient,
+ * the states of a batch in the marching form (64, 160 and 368 bytes per point at
+ * one, three and five channels; a batch beyond the limit runs in parts).  The
+ * results are the same either way.  The context keeps such memory for later calls;
+ * what is larger than the new limit is freed.  Applies to later calls on ctx.  Returns VOMT_OK, or VOMT_ERR_BAD_ARG for a null ctx. */
 int vomt_set_memory_limit(vomt_ctx *ctx, size_t bytes);
 
 /* Bounded waits of the resident engine (no counterpart in the paper; a test

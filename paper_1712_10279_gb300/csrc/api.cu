@@ -485,9 +485,11 @@ int vomt_set_memory_limit(vomt_ctx *ctx, size_t bytes)
 {
     if (!ctx) return VOMT_ERR_BAD_ARG;
     ctx->spare_bytes = bytes;
+    cudaError_t e = cudaSetDevice(ctx->device);
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "cudaSetDevice");
+    batch_state_trim(ctx->batch, bytes);
     if (ctx->gbuf_bytes > bytes) {
-        cudaError_t e = cudaSetDevice(ctx->device);
-        if (e == cudaSuccess) e = cudaFree(ctx->gbuf);
+        e = cudaFree(ctx->gbuf);
         ctx->gbuf = nullptr;
         ctx->gbuf_bytes = 0;
         if (e != cudaSuccess) return set_cuda_error(ctx, e, "gradient scratch");

@@ -458,6 +458,14 @@ void batch_state_free(BatchState *b)
     delete b;
 }
 
+void batch_state_trim(BatchState *b, size_t bytes)
+{
+    if (!b || b->march.data_cap <= bytes) return;
+    cudaFree(b->march.data);
+    b->march.data = nullptr;
+    b->march.data_cap = 0;
+}
+
 static int batch_reserve(vomt_ctx *ctx, BatchState *b, int count)
 {
     if (b->cap >= count) return VOMT_OK;

@@ -147,6 +147,7 @@ int hermitian_to_op(int k, int N, const double *L, OpDev *op, double *lmax, doub
 namespace vomt {
 struct BatchState;
 void batch_state_free(BatchState *b);
+void batch_state_trim(BatchState *b, size_t bytes);      // gives back optional memory beyond `bytes`
 }  // namespace vomt
 
 // The opaque context.

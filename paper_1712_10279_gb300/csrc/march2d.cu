@@ -522,13 +522,48 @@ Tables build_tables(const std::vector<BatchProblem> &probs, std::vector<Group> &
 
 }  // namespace
 
+namespace {
+
+// Bytes of a problem's three states and b.
+size_t state_bytes(int n, int k)
+{
+    const size_t l = (size_t)k * (k - 1) / 2, tile = (size_t)n * ((n + 31) / 32) * 32;
+    return sizeof(float4) * tile * (3 * ((3 * k + l + 3) / 4) + (k + 3) / 4);
+}
+
+// Runs of problems that are advanced together: as many as fit the context's memory limit.
+// The first problem of each, and the end; empty where one problem alone does not fit.
+std::vector<int> batch_parts(const vomt_ctx *ctx, const std::vector<int> &n, const std::vector<int> &k)
+{
+    std::vector<int> first;
+    size_t bytes = 0;
+    for (int q = 0; q < (int)n.size(); ++q) {
+        const size_t need = state_bytes(n[q], k[q]);
+        if (need > ctx->spare_bytes) return {};
+        if (q == 0 || bytes + need > ctx->spare_bytes) {
+            first.push_back(q);
+            bytes = 0;
+        }
+        bytes += need;
+    }
+    first.push_back((int)n.size());
+    return first;
+}
+
+}  // namespace
+
 double march_batch_estimate(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<int> &n,
                             const std::vector<int> &k, const vomt_params &p)
 {
-    std::vector<Group> groups;
-    if (plan_groups(ctx, scr, n, k, p, &groups)) return 1e30;
-    double us = 0.0;
-    for (const Group &g : groups) us += g.pass[g.main_pass].us / kStages[g.main_pass];
+    const std::vector<int> first = batch_parts(ctx, n, k);
+    double us = first.empty() ? 1e30 : 0.0;
+    for (size_t i = 0; i + 1 < first.size(); ++i) {
+        std::vector<Group> groups;
+        if (plan_groups(ctx, scr, {n.begin() + first[i], n.begin() + first[i + 1]},
+                        {k.begin() + first[i], k.begin() + first[i + 1]}, p, &groups))
+            return 1e30;
+        for (const Group &g : groups) us += g.pass[g.main_pass].us / kStages[g.main_pass];
+    }
     return us;
 }
 
@@ -538,8 +573,8 @@ double march_batch_estimate(vomt_ctx *ctx, BatchMarchScratch *scr, const std::ve
 // has stopped still costs its blocks the copies of a chunk's first rows, and the chunks of
 // the others stay as long as they were planned with it, so when a quarter of a group's points
 // has stopped, its passes are planned again for the problems left.
-int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
-                cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)
+static int march_part(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
+                      cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)
 {
     *taken = false;
     const int count = (int)probs.size(), sms = ctx->sm_count;
@@ -726,6 +761,47 @@ int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchPr
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch solve");
     status->resize(count);
     for (int q = 0; q < count; ++q) (*status)[q] = hstat[slot_of[q]];
+    return VOMT_OK;
+}
+
+// The parts of a batch one after the other, in the same scratch.
+int march_batch(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<BatchProblem> &probs, const vomt_params &p,
+                cudaStream_t st, std::vector<DevStatus> *status, std::vector<int> *blocks, bool *taken)
+{
+    *taken = false;
+    std::vector<int> n, k;
+    for (const BatchProblem &b : probs) {
+        n.push_back(b.g.n);
+        k.push_back(b.k);
+    }
+    const std::vector<int> first = batch_parts(ctx, n, k);
+    if (first.empty()) return VOMT_OK;
+    // the largest part's scratch before the first part runs: a part that has run cannot be
+    // left to another path (check sums: march_part's bound, of up to five groups)
+    size_t most = 0;
+    for (size_t i = 0; i + 1 < first.size(); ++i) {
+        size_t bytes = 0, rows = 5 * (4 * (size_t)ctx->sm_count + 2);
+        for (int q = first[i]; q < first[i + 1]; ++q) {
+            bytes += state_bytes(n[q], k[q]);
+            rows += (size_t)(n[q] + 29) / 30 + 1;
+        }
+        most = std::max(most, bytes + sizeof(double) * NRED * rows);
+    }
+    if (ensure_buffer(ctx, &scr->data, &scr->data_cap, most, "batch states")) {
+        ctx->err.clear();
+        return VOMT_OK;
+    }
+    status->clear();
+    blocks->clear();
+    for (size_t i = 0; i + 1 < first.size(); ++i) {
+        std::vector<DevStatus> s;
+        std::vector<int> b;
+        const int rc = march_part(ctx, scr, {probs.begin() + first[i], probs.begin() + first[i + 1]}, p, st, &s, &b, taken);
+        if (rc) return rc;
+        if (!*taken) return i == 0 ? VOMT_OK : fail(ctx, VOMT_ERR_CUDA, "batch states");
+        status->insert(status->end(), s.begin(), s.end());
+        blocks->insert(blocks->end(), b.begin(), b.end());
+    }
     return VOMT_OK;
 }
 
