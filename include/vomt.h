@@ -353,7 +353,9 @@ int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance *inst, floa
  * tolerance) on the one-block-per-instance path with 128, 256 and 512 threads
  * per block, and on the grouped path where it applies; keeps the fastest
  * thread count and the faster path for later vomt_solve_batched calls on ctx
- * with VOMT_ENGINE_AUTO / VOMT_ENGINE_BATCHED.  Returns the best thread count
+ * with VOMT_ENGINE_AUTO / VOMT_ENGINE_BATCHED.  The marching form is timed too
+ * (sample_iters >= 4), and used or not used accordingly for batches of the same
+ * sides, channel and edge counts; other batches go by estimate.  Returns the best thread count
  * in *best_threads and the times (milliseconds) in ms[0..3] (128, 256, 512
  * threads, then the grouped path or -1); either pointer may be NULL.
  * Overwrites the arena's u, w, phi. */

@@ -482,8 +482,8 @@ class Batch:
 
     def tune(self, sample_iters=50, **kw):
         """Time the one-block-per-problem path with 128 / 256 / 512 threads per block and
-        the grouped path on `sample_iters` iterations; keep the fastest on this device's
-        context.  Returns (best thread count, {128: ms, 256: ms, 512: ms, "grouped": ms
+        the grouped path (and the marching form, for batches shaped like this one) on
+        `sample_iters` iterations; keep the fastest on this device's context.  Returns (best thread count, {128: ms, 256: ms, 512: ms, "grouped": ms
         or -1 where that path does not apply})."""
         p = _params(kw.get("tau"), None, None, kw.get("u_norm", U_L12), kw.get("w_norm", W_L1), sample_iters,
                     sample_iters, 0.0, 0.0, False, "batched")

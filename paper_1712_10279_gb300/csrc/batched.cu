@@ -419,6 +419,11 @@ struct BatchState {
     BatchArgs g_args;
     int tuned_threads = 0;
     int tuned_engine = 0;      // set by vomt_batch_tune: the faster path for AUTO solves (0: by estimate)
+    // whether the marching form was faster still, for batches of the tuned one's sides, channels
+    // and edges: 1 or 0 (-1: not timed); trying: the tuner is timing it
+    int tuned_march = -1;
+    bool trying_march = false;
+    std::vector<int> tuned_shapes;
     // grouped path: job tables, exchange scratch, control word, per-problem status
     void *gjobs = nullptr;
     size_t gjobs_bytes = 0;
@@ -665,6 +670,13 @@ static bool march_problems(const std::vector<InstDev> &h, float *arena, const vo
         out->push_back(b);
     }
     return true;
+}
+
+static std::vector<int> batch_shapes(const std::vector<InstDev> &h)
+{
+    std::vector<int> s;
+    for (const InstDev &I : h) s.insert(s.end(), {I.n, I.k, I.l});
+    return s;
 }
 
 static int grouped_solve(vomt_ctx *ctx, BatchState *b, int count, const std::vector<InstDev> &h, float *arena,
@@ -997,27 +1009,35 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
         // path: grouped resident waves, or one block per problem from a queue
         std::vector<Wave> waves;
         bool grouped = false;
+        const bool may_march = (p.engine == VOMT_ENGINE_AUTO || p.engine == VOMT_ENGINE_BATCHED) && p.u_norm == VOMT_U_L12 &&
+                               p.w_norm == VOMT_W_L1 && p.eps == 0.0 && !ctx->drop_exchange &&
+                               std::min(p.check_every, p.max_iters) >= 4;
+        int march = -1;            // 1, 0: by the tuner's timing of such a batch
+        if (may_march && b->trying_march) march = 1;
+        else if (may_march && b->tuned_march >= 0 && b->tuned_shapes == batch_shapes(hinst)) march = b->tuned_march;
         if (p.engine == VOMT_ENGINE_RESIDENT) {
             if (!grouped_plan(ctx, count, hinst, p, waves))
                 return fail(ctx, VOMT_ERR_TOO_LARGE,
                             "grouped batch path needs k <= 5, a resident tile plan and max_iters < 2^20 - 2");
             grouped = true;
         } else if (p.engine == VOMT_ENGINE_AUTO || p.engine == VOMT_ENGINE_BATCHED) {
-            if (b->tuned_engine == VOMT_ENGINE_RESIDENT)
+            if (b->tuned_engine == VOMT_ENGINE_RESIDENT || march > 0)
                 grouped = grouped_plan(ctx, count, hinst, p, waves);
             else if (b->tuned_engine == 0)
                 grouped = grouped_plan(ctx, count, hinst, p, waves) &&
                           grouped_estimate(waves, std::max(p.max_iters, 1)) <
                               queue_estimate(hinst, std::max(p.max_iters, 1), ctx->sm_count);
         }
-        // The marching form takes a grouped batch (same results, bit for bit) where it is
-        // estimated faster.  The estimate of a wave is about twice what it takes (256^2, three
-        // channels: 3.06 us per iteration against 1.57).
+        // The marching form takes a grouped batch (same results, bit for bit) where the tuner
+        // timed it faster or, for batches it has not seen, where it is estimated faster.  The
+        // estimate of a wave is about twice what it takes (256^2, three channels: 3.06 us per
+        // iteration against 1.57); of 22 batches of 2 to 300 problems the choice was the faster
+        // one at every interval between checks, by 2% (2 x 256^2, a check every 4 iterations) to
+        // 3.2 times (32 of 64^2 and 128^2 with five channels).
         std::vector<DevStatus> mstat;
         std::vector<int> mblocks;
         bool marched = false;
-        if (grouped && p.engine != VOMT_ENGINE_RESIDENT && p.u_norm == VOMT_U_L12 && p.w_norm == VOMT_W_L1 && p.eps == 0.0 &&
-            !ctx->drop_exchange && std::min(p.check_every, p.max_iters) >= 4) {
+        if (grouped && may_march && march != 0) {
             const int iters = std::max(p.max_iters, 1);
             std::vector<int> sides, ks;
             for (const InstDev &I : hinst) {
@@ -1025,7 +1045,8 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
                 ks.push_back(I.k);
             }
             std::vector<BatchProblem> probs;
-            if (march_batch_estimate(ctx, &b->march, sides, ks, p) < 0.5e-3 * grouped_estimate(waves, iters) / iters &&
+            if ((march > 0 ||
+                 march_batch_estimate(ctx, &b->march, sides, ks, p) < 0.5e-3 * grouped_estimate(waves, iters) / iters) &&
                 march_problems(hinst, arena, p, &probs)) {
                 rc = march_batch(ctx, &b->march, probs, p, st, &mstat, &mblocks, &marched);
                 if (rc) return rc;
@@ -1155,10 +1176,9 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
     }
 }
 
-extern "C" int vomt_batch_tune(vomt_ctx *ctx, int count, const vomt_instance *inst, float *arena,
-                               const vomt_params *pin, int sample_iters, int *best_threads, double *ms)
+static int batch_tune(vomt_ctx *ctx, int count, const vomt_instance *inst, float *arena, const vomt_params *pin,
+                      int sample_iters, int *best_threads, double *ms)
 {
-    if (!ctx || sample_iters < 1) return VOMT_ERR_BAD_ARG;
     vomt_params p;
     vomt_default_params(&p);
     if (pin) p = *pin;
@@ -1205,6 +1225,7 @@ extern "C" int vomt_batch_tune(vomt_ctx *ctx, int count, const vomt_instance *in
     if (best_threads) *best_threads = pick;
     // the grouped resident path, where it can take the problems
     b->tuned_engine = VOMT_ENGINE_STREAM;
+    b->tuned_march = -1;
     if (ms) ms[3] = -1.0;
     std::vector<InstDev> hinst;
     std::vector<int> order;
@@ -1219,9 +1240,32 @@ extern "C" int vomt_batch_tune(vomt_ctx *ctx, int count, const vomt_instance *in
         if (rc < 0) return rc;
         if (ms) ms[3] = t;
         if (t < best) b->tuned_engine = VOMT_ENGINE_RESIDENT;
+        best = std::min(best, t);
+        // the marching form, where it takes them
+        b->trying_march = true;
+        q.engine = VOMT_ENGINE_AUTO;
+        double tm = 0.0;
+        rc = timed(q, &tm);
+        b->trying_march = false;
+        if (rc < 0) return rc;
+        if (ctx->last_form == VOMT_FORM_BATCH_MARCH) {
+            b->tuned_march = tm < best ? 1 : 0;
+            b->tuned_shapes = batch_shapes(hinst);
+        }
     }
     ctx->err.clear();
     return VOMT_OK;
+}
+
+extern "C" int vomt_batch_tune(vomt_ctx *ctx, int count, const vomt_instance *inst, float *arena,
+                               const vomt_params *pin, int sample_iters, int *best_threads, double *ms)
+{
+    if (!ctx || sample_iters < 1) return VOMT_ERR_BAD_ARG;
+    try {
+        return batch_tune(ctx, count, inst, arena, pin, sample_iters, best_threads, ms);
+    } catch (...) {
+        return fail(ctx, VOMT_ERR_BAD_ARG, "internal exception");
+    }
 }
 
 extern "C" int vomt_batch_set_threads(vomt_ctx *ctx, int threads)
