@@ -382,18 +382,25 @@ __global__ void __launch_bounds__(512) k_batch(BatchArgs a)
 namespace vomt {
 namespace {
 
-// Blocks per instance of the density checks: an instance of 256^2 with five channels is
-// 2.6 MB, 0.6 ms for one block.
+// Blocks per instance of the density checks, one per 16384 values of the largest instance: one
+// of 256^2 with five channels is 2.6 MB, 0.6 ms for one block, while 16 blocks for each of 64
+// instances of 32^2 cost 20 us, most of it the host's look at their results.
 constexpr int kValChunks = 16;
+int val_chunks(const std::vector<InstDev> &h)
+{
+    size_t most = 0;
+    for (const InstDev &I : h) most = std::max(most, (size_t)I.k * I.n * I.n);
+    return (int)std::min<size_t>(std::max<size_t>((most + 16383) / 16384, 1), kValChunks);
+}
 
 // per instance and chunk (a block each): sum rho0, sum rho1, min rho0, min rho1, non-finite count
 template <typename Sum>
-__global__ void __launch_bounds__(256) k_batch_validate(const InstDev *inst, const float *arena, double *out)
+__global__ void __launch_bounds__(256) k_batch_validate(const InstDev *inst, const float *arena, int chunks, double *out)
 {
-    const InstDev &I = inst[blockIdx.x / kValChunks];
-    const size_t cnt = (size_t)I.k * I.n * I.n, chunk = blockIdx.x % kValChunks;
+    const InstDev &I = inst[blockIdx.x / chunks];
+    const size_t cnt = (size_t)I.k * I.n * I.n, chunk = blockIdx.x % chunks;
     const float *r0 = arena + I.o_rho0, *r1 = arena + I.o_rho1;
-    const size_t q0 = cnt * chunk / kValChunks, q1 = cnt * (chunk + 1) / kValChunks;
+    const size_t q0 = cnt * chunk / chunks, q1 = cnt * (chunk + 1) / chunks;
     DensityCheck<Sum> c;
 #pragma unroll 4
     for (size_t q = q0 + threadIdx.x; q < q1; q += 256) c.add(r0[q], r1[q]);
@@ -974,13 +981,14 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
         e = cudaMemcpyAsync(b->dinst, hinst.data(), sizeof(InstDev) * count, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(b->dorder, order.data(), sizeof(int) * count, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return set_cuda_error(ctx, e, "batch table upload");
-        // density checks, kValChunks blocks per instance
-        std::vector<double> hv((size_t)5 * kValChunks * count);
+        // density checks, several blocks per instance
+        const int chunks = val_chunks(hinst);
+        std::vector<double> hv((size_t)5 * chunks * count);
         for (int wide = 0; wide < 2; ++wide) {
             if (wide)
-                k_batch_validate<WideSum><<<count * kValChunks, 256, 0, st>>>(b->dinst, arena, b->dval);
+                k_batch_validate<WideSum><<<count * chunks, 256, 0, st>>>(b->dinst, arena, chunks, b->dval);
             else
-                k_batch_validate<TripleSum><<<count * kValChunks, 256, 0, st>>>(b->dinst, arena, b->dval);
+                k_batch_validate<TripleSum><<<count * chunks, 256, 0, st>>>(b->dinst, arena, chunks, b->dval);
             ++ctx->launches;
             e = cudaMemcpyAsync(hv.data(), b->dval, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -991,8 +999,8 @@ extern "C" int vomt_solve_batched(vomt_ctx *ctx, int count, const vomt_instance 
         }
         for (int q = 0; q < count; ++q) {
             double h[5] = {0.0, 0.0, INFINITY, INFINITY, 0.0};
-            for (int c = 0; c < kValChunks; ++c) {
-                const double *v = &hv[(size_t)5 * ((size_t)q * kValChunks + c)];
+            for (int c = 0; c < chunks; ++c) {
+                const double *v = &hv[(size_t)5 * ((size_t)q * chunks + c)];
                 h[0] += v[0];
                 h[1] += v[1];
                 h[2] = fmin(h[2], v[2]);
