@@ -434,16 +434,16 @@ extern "C" int vomt_backward(vomt_ctx *ctx, int batch, int n, int pitch, int k, 
     if (!phi || (n_edges > 0 && !w)) return fail(ctx, VOMT_ERR_BAD_ARG, "backward: null array");
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "cudaSetDevice");
-    // Blocks of 16384 values and more, no more of them than two per SM, and threads with eight
+    // Blocks of 16384 values and more, no more of them than two per SM, and threads with sixteen
     // values and more.  A block too many costs more than it saves: with eight blocks of 1024
-    // threads for every problem, 2048 of 16^2 took 1430 us (64 before, one block each) and 512
-    // of 32^2, three channels, 370 (60), while eight of 256^2 want all 64 blocks (677 us with one
-    // block each, FP64 sums per value and a division per index).
+    // threads for every problem, 2048 of 16^2 took 1430 us (now 23) and 512 of 32^2, three
+    // channels, 370 (now 32), while eight of 256^2 want all 64 blocks (23 us, 677 with one block
+    // each, FP64 sums per value and a division per index).
     const double values = (double)(k + n_edges) * n * n;
     unsigned blocks = 1, threads = 128;
     while (blocks < kEnvCluster && values >= 16384.0 * 2 * blocks && (double)batch * 2 * blocks <= 2.0 * ctx->sm_count)
         blocks *= 2;
-    while (threads < 1024 && values > 8.0 * blocks * threads) threads *= 2;
+    while (threads < 1024 && values > 16.0 * blocks * threads) threads *= 2;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
