@@ -421,7 +421,7 @@ def extra_differentiable(dev, count=64, cap=150000, tol=1e-3):
     _, ms_u = _gpu_ms(unrolled)
     return dict(workload="%d colour-image pairs 256x256 k=3 (seeds 2000..), alpha=1, per-pair tau from "
                          "vomt_batch_tune_tau, forward to rel gap and rel res <= %g (Section 8.1's rule), cap %d; "
-                         "unrolled T=200, checkpoints every 20" % (count, tol, cap),
+                         "unrolled T=200, every iterate kept (0.6 GB)" % (count, tol, cap),
                 tau_tune_ms=tau_tune_ms, forward_backward_batched_ms=ms_fb, plain_forward_loop_ms=ms_p,
                 fwd_bwd_over_plain_time=ms_fb / ms_p, unrolled_fwd_bwd_ms=ms_u,
                 plain_converged=sum(r["status"] == 0 for r in rp), plain_iters_mean=statistics.mean(r["iters"] for r in rp),
@@ -537,12 +537,17 @@ def extra_hbm_bound(dev, peak, n=2048, iters=1000):
         sol, ms = _gpu_ms(lambda: V.solve(d0, d1, edges, 1.0, max_iters=iters, check_every=CHECK_EVERY,
                                           engine="stream"))
         it = sol.result["iters"]
-        bpg = 4 * (7 * k + 2 * len(edges))
+        # a pass over the grid reads the state and b and writes the state, in groups of four
+        # floats per point, and serves four iterations
+        groups, bgroups, per_pass = (3 * k + k * (k - 1) // 2 + 3) // 4, (k + 3) // 4, 4
+        bpg = 16 * (2 * groups + bgroups) / per_pass
         gbs = bpg * nn_ * nn_ * it / (ms / 1e3) / 1e9
-        out[name] = dict(n=nn_, k=k, iters=it, us_per_iter=1e3 * ms / it, algorithmic_bytes_per_gp_it=bpg,
+        out[name] = dict(n=nn_, k=k, iters=it, us_per_iter=1e3 * ms / it, form=V.last_form(),
+                         iterations_per_pass=per_pass, bytes_per_gp_it=bpg,
+                         one_iteration_per_pass_bytes_per_gp_it=4 * (7 * k + 2 * len(edges)),
                          achieved_GBps=gbs, frac_of_measured_hbm=gbs / peak,
-                         note="checks every %d iterations included; 1000 iterations run as replays of "
-                              "a captured graph of 100" % CHECK_EVERY)
+                         note="marching form; checks every %d iterations and the layout conversions of "
+                              "the call included" % CHECK_EVERY)
     return out
 
 

@@ -68,9 +68,18 @@ extern "C" {
 #define VOMT_W_NUC 2   /* matrix OMT: ||W||_{1,nuc} = sum_s ||W_s||_nuc (Section 6.2) */
 
 /* Engines.  AUTO picks RESIDENT when the whole state fits in the SMs'
- * registers and shared memory, else STREAM. */
+ * registers and shared memory, else STREAM; with the default norms and eps = 0 it
+ * picks STREAM also where that is faster than the resident engine (from about 337^2 at
+ * one and two channels, 313^2 at three and four, 241^2 and less at five to eight, and
+ * with enough iterations between checks), with the same iterates bit for bit.
+ * The streaming engine's marching form runs several iterations per pass over the
+ * grid.  It takes vector problems with four and more iterations between checks (any
+ * number from five channels on) whose edges are listed in the order of their pairs
+ * (0,1), (0,2), ..., (1,2), ... (either way round, pairs may be missing); with edges in
+ * any other order the sums over a channel's edges are taken as listed, by the kernels
+ * with one iteration per launch (up to 2.7 times the time). */
 #define VOMT_ENGINE_AUTO      0
-#define VOMT_ENGINE_STREAM    1   /* one fused stencil launch per iteration, state in HBM */
+#define VOMT_ENGINE_STREAM    1   /* stencil passes over the state in HBM */
 #define VOMT_ENGINE_RESIDENT  2   /* one persistent launch, state on chip for the whole solve */
 
 #define VOMT_MAX_CHANNELS 8        /* k <= 8, so l <= 28 */
@@ -339,8 +348,11 @@ int vomt_batch_layout(int count, vomt_instance *inst, size_t *total_floats);
  * faster on ctx, else the one a cost model estimates faster.  Where that is the
  * grouped path, the norms are the defaults, eps = 0, every check is at least four
  * iterations from the last and edges are listed in the order of their pairs, the
- * marching form of the streaming engine takes the batch if it is estimated faster
- * still (results[q].variant = 0, .blocks those of a pass, .halo 0; the same iterates).
+ * marching form of the streaming engine takes the batch if it is estimated (or was
+ * timed) faster still: all problems of a channel count advance together, in parts
+ * where their states exceed the memory limit, and passes are planned anew as
+ * problems stop (results[q].variant = 0, .blocks those of problem q's last pass, .halo 0;
+ * the same iterates).
  * results: host array of `count` (may be NULL); results[q].blocks is the
  * number of tiles instance q ran on and .halo its ring width.  Returns
  * VOMT_OK, VOMT_NOT_CONVERGED if some instance hit the cap, or the first error

@@ -14,7 +14,7 @@
 // mode through the T iterations.  The forward pass keeps every iterate where that
 // takes no more than the context's memory limit, else one every `ckpt` iterations, from
 // which the reverse pass recomputes a segment at a time; the reverse pass applies the transposed Jacobian of
-// one iteration per step (k_adj_step; at 256^2, three channels, 4.3 us a step, 15 us
+// one iteration per step (k_adj_step; at 256^2, three channels, 4.6 us a step, 15 us
 // marching two rows per warp, and 2.9 us a forward step): the chain rule through phi' = phi + tau(div_x ubar + div_G wbar +
 // rho1 - rho0), through u' = shrink(u + mu grad phi; mu) and through
 // w' = shrink_w(w + nu grad_G phi; alpha nu), with div_x^T = -grad_x

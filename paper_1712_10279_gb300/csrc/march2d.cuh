@@ -13,11 +13,12 @@
 // The neighbours that a strip and a chunk lack cost redundant work: each stage loses one
 // column on either side and one row at either end, so a warp writes 32 - 2 S columns and
 // reads S more rows on either side of its chunk.  In return one pass over memory serves S
-// iterations: 2048^2 with three channels takes 27 us per iteration at S = 4 (a pass moves
-// 0.47 GB in 107 us, 65% of the measured copy rate, the rest is issue), where one
-// iteration per pass with TMA tiles takes 79 us and is bound by HBM alone; 1024^2 with one
-// channel 3.6 us (was 9.2), 512^2 with eight channels 22 us (118 us: the recomputed shrinks
-// of the one-iteration kernel spill).
+// iterations: at 2048^2 with three channels a pass of S = 4 moves 0.47 GB in 107 us, 65% of
+// the measured copy rate, with three quarters of the issue slots busy (190 instructions per
+// point and iteration); with a check every 100 iterations and the layout conversions a
+// solve takes 29.4 us per iteration, where one iteration per pass with TMA tiles takes 79
+// us and is bound by HBM alone.  1024^2 with one channel 3.9 us (was 9.2), 512^2 with eight
+// channels 22 us (118 us: the recomputed shrinks of the one-iteration kernel spill).
 //
 // Every value is rounded as the one-iteration kernels (or, RES, the resident kernels) round
 // it, operation by operation (edges listed in the order of the pairs), so that the

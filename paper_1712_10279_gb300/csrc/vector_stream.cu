@@ -7,7 +7,7 @@
 // waiting for the threads that own them, so one launch does a whole iteration
 // and no grid-wide barrier is needed between the u/w and phi halves
 // (Section 7.4 puts a synchronisation there).  Vector problems with four and more
-// iterations between checks take the marching form instead (march2d.cuh); these kernels
+// iterations between checks (any number from five channels on) take the marching form instead (march2d.cuh); these kernels
 // serve matrix fields, shorter intervals, edges not listed in the order of the pairs, the
 // allocation-free entry point and the unrolled gradient's forward pass.
 #include <math.h>
