@@ -463,6 +463,7 @@ int plan_groups(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<int> &n
         }
         if (g.per_sm[0] < 1) return VOMT_ERR_TOO_LARGE;
         plan_live(n, g, interval, ctx->sm_count);
+        if (g.pass[0].stages == 0) return VOMT_ERR_TOO_LARGE;
         out->push_back(g);
     }
     return VOMT_OK;
@@ -524,6 +525,8 @@ Tables build_tables(const std::vector<BatchProblem> &probs, std::vector<Group> &
 
 namespace {
 
+constexpr int kMaxPart = 65535;      // problems of a part: a launch's third dimension
+
 // Bytes of a problem's three states and b.
 size_t state_bytes(int n, int k)
 {
@@ -531,8 +534,9 @@ size_t state_bytes(int n, int k)
     return sizeof(float4) * tile * (3 * ((3 * k + l + 3) / 4) + (k + 3) / 4);
 }
 
-// Runs of problems that are advanced together: as many as fit the context's memory limit.
-// The first problem of each, and the end; empty where one problem alone does not fit.
+// Runs of problems that are advanced together: as many as fit the context's memory limit and
+// a launch's third dimension.  The first problem of each, and the end; empty where one problem
+// alone does not fit.
 std::vector<int> batch_parts(const vomt_ctx *ctx, const std::vector<int> &n, const std::vector<int> &k)
 {
     std::vector<int> first;
@@ -540,7 +544,7 @@ std::vector<int> batch_parts(const vomt_ctx *ctx, const std::vector<int> &n, con
     for (int q = 0; q < (int)n.size(); ++q) {
         const size_t need = state_bytes(n[q], k[q]);
         if (need > ctx->spare_bytes) return {};
-        if (q == 0 || bytes + need > ctx->spare_bytes) {
+        if (q == 0 || bytes + need > ctx->spare_bytes || q - first.back() == kMaxPart) {
             first.push_back(q);
             bytes = 0;
         }
@@ -578,7 +582,6 @@ static int march_part(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<B
 {
     *taken = false;
     const int count = (int)probs.size(), sms = ctx->sm_count;
-    if (count > 65535) return VOMT_OK;                // a launch's third dimension
     std::vector<int> side(count), ks(count);
     for (int q = 0; q < count; ++q) {
         side[q] = probs[q].g.n;
