@@ -658,7 +658,19 @@ static int march_part(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<B
     if (rc) return rc;
     BatchItem *const ditems = (BatchItem *)scr->items, *const dlive = ditems + count;
     int *const dmaps = (int *)scr->maps;
+    // The kernels read the tables before they wait for the kernel before them, so the first one
+    // after a copy of new tables is launched as an ordinary kernel, after the copy.
+    bool fresh = true;
+    auto launch = [&](auto kern, unsigned grid, unsigned block, size_t smem, auto... args) {
+        if (fresh)
+            kern<<<grid, block, smem, st>>>(args...);
+        else
+            launch_pdl(kern, dim3(grid), dim3(block), smem, st, args...);
+        fresh = false;
+        ctx->launches += 1;
+    };
     auto upload = [&]() {
+        fresh = true;
         const Tables &t = plans.back();
         cudaError_t r = cudaMemcpyAsync(dlive, t.items.data(), sizeof(BatchItem) * t.items.size(), cudaMemcpyHostToDevice, st);
         return r != cudaSuccess ? r : cudaMemcpyAsync(dmaps, t.maps.data(), sizeof(int) * t.maps.size(),
@@ -678,18 +690,15 @@ static int march_part(vomt_ctx *ctx, BatchMarchScratch *scr, const std::vector<B
     }
     auto one = [&](Group &g, int q, bool last) {
         const int prev = last && kStages[q] > 1 ? 1 : 0;
-        launch_pdl(g.K.many[q], dim3(g.pass[q].blocks), dim3(32 * kWarps), (size_t)g.pass[q].smem, st,
-                   (const BatchItem *)dlive + g.first_live, (const int *)dmaps + g.map_at[q], g.cur, prev);
-        ctx->launches += 1;
+        launch(g.K.many[q], g.pass[q].blocks, 32 * kWarps, (size_t)g.pass[q].smem, (const BatchItem *)dlive + g.first_live,
+               (const int *)dmaps + g.map_at[q], g.cur, prev);
         g.before = prev ? 2 : g.cur;
         g.cur ^= 1;
     };
     auto check = [&](Group &g, int t) {
-        launch_pdl(g.K.check_many, dim3(g.check_blocks), dim3(32 * kWarps), 0, st, (const BatchItem *)dlive + g.first_live,
-                   (const int *)dmaps + g.map_at[3], g.cur, g.before);
-        launch_pdl(k_finalize_many, dim3((unsigned)g.live.size()), dim3(kFinThreads), 0, st,
-                   (const BatchItem *)dlive + g.first_live, t, g.cur);
-        ctx->launches += 2;
+        launch(g.K.check_many, g.check_blocks, 32 * kWarps, 0, (const BatchItem *)dlive + g.first_live,
+               (const int *)dmaps + g.map_at[3], g.cur, g.before);
+        launch(k_finalize_many, (unsigned)g.live.size(), kFinThreads, 0, (const BatchItem *)dlive + g.first_live, t, g.cur);
     };
     if (p.max_iters == 0)
         for (Group &g : groups) check(g, 0);
